@@ -17,6 +17,7 @@
 #include "emd_tc.cuh"
 #include "emd_fft.cuh"
 #include "emd_halo.cuh"
+#include "emd_taps.cuh"
 
 using emd::Shape;
 
@@ -36,7 +37,7 @@ void set_err(const char* fmt, ...) {
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 struct Layout {
-  size_t x0, x1, N, Den, u, y, kf, ka, fraw, part, sums, err, total;
+  size_t x0, x1, N, Den, u, y, kf, ka, fraw, part, sums, err, counters, work, total;
 };
 
 Layout make_layout(const Shape& s) {
@@ -60,6 +61,10 @@ Layout make_layout(const Shape& s) {
   L.part = take(parts * sizeof(double));
   L.sums = take(8 * sizeof(double));
   L.err = take(sizeof(int));
+  // the launch forms of the FP32 direct iteration (emd_taps.cuh)
+  const emd::DirectPlan dp = emd::direct_plan(s, false);
+  L.counters = take(dp.planes ? (size_t)emd::direct_counter_ints(s) * sizeof(int) : 0);
+  L.work = take((size_t)dp.planes * s.g.plane * sizeof(float));
   L.total = off;
   return L;
 }
@@ -71,6 +76,18 @@ bool is_device_ptr(const void* p) {
     return false;
   }
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
+// memory that a kernel on `device` may read as it is (another GPU's memory is
+// copied instead)
+bool readable_on(const void* p, int device) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeManaged ||
+         (at.type == cudaMemoryTypeDevice && at.device == device);
 }
 
 }  // namespace
@@ -92,6 +109,12 @@ struct emd_ctx {
   float *kf = nullptr, *ka = nullptr, *fraw = nullptr;
   double *part = nullptr, *sums = nullptr;
   int* err = nullptr;
+  // launch forms of the FP32 direct iteration: plans per noise model, work
+  // planes and counters in the arena, host copies of the kernels (taps form)
+  emd::DirectPlan plan[2];
+  int* counters = nullptr;
+  float* work = nullptr;
+  std::vector<float> hkf, hka;
   double logdet = 0.0, suy = 0.0, su = 0.0, nvalid = 0.0;
   // noise model: Gaussian (Eq. (1)) or Student-t with nu degrees of freedom
   int noise = EMD_NOISE_GAUSSIAN;
@@ -211,6 +234,33 @@ emd::FusedArgs fused_args(emd_ctx* c) {
   a.t1 = c->s.n;
   a.nu = c->noise == EMD_NOISE_STUDENT_T ? (float)c->nu : 0.f;
   return a;
+}
+
+emd::DirectLaunch direct_launch(emd_ctx* c) {
+  emd::DirectLaunch d;
+  d.a = fused_args(c);
+  if (c->noise == EMD_NOISE_STUDENT_T) d.a.Nw = c->Ns;
+  d.work = c->work;
+  d.counters = c->counters;
+  return d;
+}
+
+// k iterations with the launch form of the context's plan (not kFormHalo)
+int iterate_direct(emd_ctx* c, int k) {
+  const emd::DirectPlan& p = c->plan[c->noise == EMD_NOISE_STUDENT_T];
+  while (k > 0) {
+    const emd::DirectLaunch d = direct_launch(c);
+    int done = 1;
+    if (p.form == emd::kFormTaps) {
+      CK(emd::launch_taps_iter(c->s, p, d, c->hkf.data(), c->hka.data(), false, c->st));
+    } else {
+      done = std::min(k, emd::split_iters_per_launch(c->s));
+      CK(emd::launch_split_iters(c->s, p, d, c->x[c->cur], c->x[c->cur ^ 1], done, false, c->st));
+    }
+    c->cur ^= done & 1;
+    k -= done;
+  }
+  return EMD_OK;
 }
 
 // copy an (n x H x W) natural array into n padded planes
@@ -343,6 +393,9 @@ emd_ctx* emd_create(int H, int W, int n, int psf_k, int r) {
   c->part = reinterpret_cast<double*>(c->arena + c->L.part);
   c->sums = reinterpret_cast<double*>(c->arena + c->L.sums);
   c->err = reinterpret_cast<int*>(c->arena + c->L.err);
+  c->counters = reinterpret_cast<int*>(c->arena + c->L.counters);
+  c->work = reinterpret_cast<float*>(c->arena + c->L.work);
+  for (int m = 0; m < 2; ++m) c->plan[m] = emd::direct_plan(s, m == 1);
   g_err.clear();
   return c;
 }
@@ -663,8 +716,14 @@ int emd_set_frames(emd_ctx* c, const float* y, const float* v, const float* f,
   c->fft_ready = false;
   c->nt_ready = false;
   const size_t npix = (size_t)s.n * s.H * s.W;
-  if (int rc = put_planes(c, c->y, y, s.n)) return rc;
-  if (int rc = put_planes(c, c->u, v, s.n)) return rc;  // v, converted in place below
+  // this device's arrays are read by the set-up kernel as they are (33
+  // exposures of 1024^2: two copies per exposure and a pass less); others go
+  // to the planes first and are converted in place
+  const bool ydev = readable_on(y, c->device), vdev = readable_on(v, c->device);
+  if (!ydev)
+    if (int rc = put_planes(c, c->y, y, s.n)) return rc;
+  if (!vdev)
+    if (int rc = put_planes(c, c->u, v, s.n)) return rc;
   CK(cudaMemcpyAsync(c->fraw, f, (size_t)s.n * s.K * s.K * sizeof(float), cudaMemcpyDefault,
                      c->st));
   const uint8_t* dmask = nullptr;
@@ -679,11 +738,18 @@ int emd_set_frames(emd_ctx* c, const float* y, const float* v, const float* f,
     }
   }
   CK(cudaMemsetAsync(c->err, 0, sizeof(int), c->st));
-  emd::SetupArgs sa{dmask, c->u, c->y, c->part, c->err};
+  emd::SetupArgs sa{dmask, ydev ? y : nullptr, vdev ? v : nullptr, c->u, c->y, c->part, c->err};
   CK(emd::launch_setup(s, sa, c->st));
   if (tmp) CK(cudaFreeAsync(tmp, c->st));
   CK(emd::launch_reduce_final(c->part, emd::kRedBlocks, 4, c->sums, c->st));
   CK(emd::launch_build_kernels(s, c->fraw, c->kf, c->ka, c->st));
+  if (c->plan[0].form == emd::kFormTaps) {
+    const size_t nk = (size_t)s.n * s.R2 * s.Kc * s.KP;
+    c->hkf.resize(nk);
+    c->hka.resize(nk);
+    CK(cudaMemcpyAsync(c->hkf.data(), c->kf, nk * sizeof(float), cudaMemcpyDeviceToHost, c->st));
+    CK(cudaMemcpyAsync(c->hka.data(), c->ka, nk * sizeof(float), cudaMemcpyDeviceToHost, c->st));
+  }
   double h[4];
   int herr = 0;
   CK(cudaMemcpyAsync(h, c->sums, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
@@ -699,8 +765,16 @@ int emd_set_frames(emd_ctx* c, const float* y, const float* v, const float* f,
   c->su = h[2];
   c->nvalid = h[3];
   // numerator N = sum_t F_t^T (u_t y_t)
-  emd::FusedArgs a = fused_args(c);
-  CK(emd::launch_fused(s, a, 1, c->part, c->st));
+  // (the Gaussian numerator whatever the noise model; the same sums in the
+  // same order from every form)
+  emd::DirectLaunch d = direct_launch(c);
+  d.a.Nw = c->N;
+  if (c->plan[0].form == emd::kFormTaps)
+    CK(emd::launch_taps_iter(s, c->plan[0], d, c->hkf.data(), c->hka.data(), true, c->st));
+  else if (c->plan[0].form == emd::kFormSplit)
+    CK(emd::launch_split_iters(s, c->plan[0], d, c->x[0], c->x[1], 1, true, c->st));
+  else
+    CK(emd::launch_fused(s, d.a, 1, c->part, c->st));
   // default strictly positive start
   double x0 = 1.0;
   if (c->su > 0.0) {
@@ -830,6 +904,9 @@ int emd_iterate(emd_ctx* c, int k) {
     }
     return EMD_OK;
   }
+  // FP32 direct, no tile shape fixed: the launch form of this shape, if any
+  if (c->prec == EMD_PREC_FP32 && c->tile_forced < 0 && c->plan[0].form != emd::kFormHalo)
+    return iterate_direct(c, k);
   if (c->noise == EMD_NOISE_STUDENT_T) {
     // heavy-tailed EM: the numerator depends on x through the weights u' of
     // the current x. The halo-exchange kernel computes the forward model
@@ -1006,7 +1083,9 @@ int emd_get_tile_shape(emd_ctx* c, int* shape, int* decided) {
   DeviceGuard dg(c->device);
   tile_trials_poll(c);
   int cfg = c->tile_forced, dec = 1;
-  if (cfg < 0) {
+  if (cfg < 0 && c->plan[0].form != emd::kFormHalo) {
+    cfg = 0;  // nothing to decide: a launch form runs, its largest tiles of 64 rows
+  } else if (cfg < 0) {
     std::lock_guard<std::mutex> lk(g_tile_mu);
     auto it = g_tile_decided.find(tile_key(c, c->noise == EMD_NOISE_STUDENT_T));
     if (it != g_tile_decided.end()) {
@@ -1076,7 +1155,10 @@ int emd_loglik_chi2(emd_ctx* c, double* out, double* chi2) {
   // EMD_PREC_FP32_PAIR); FP64 partial sums added in a fixed order
   const int max_parts = (int)((c->L.sums - c->L.part) / sizeof(double));
   int nparts = 0;
-  if (c->prec != EMD_PREC_FP32_PAIR && max_parts >= c->s.gx * c->s.gy) {
+  if (c->prec != EMD_PREC_FP32_PAIR && c->plan[0].form == emd::kFormTaps) {
+    CK(emd::launch_taps_chi2(c->s, c->plan[0], a, c->hkf.data(), c->part, max_parts, &nparts,
+                             c->st));
+  } else if (c->prec != EMD_PREC_FP32_PAIR && max_parts >= c->s.gx * c->s.gy) {
     cudaError_t e = cudaSuccess;
     nparts = emd::launch_halo_chi2(c->s, a, c->part, max_parts, c->st, &e);
     CK(e);

@@ -3,71 +3,184 @@
 // register-blocked FP32 correlation, where a thread accumulates an RY x RX
 // block of outputs
 //     acc[p][c] += sum_{a < Kc, b < KP} k[a][b] src[oy + p + a][ox + c + b]
-// from a shared-memory plane, one 16-byte kernel quad and a (RX + 4)-float
-// window of the source row at a time.
+// from a shared-memory plane.
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace emd {
 
+// A staged plane whose rows carry a skew of 4 floats every RY rows, RY the
+// row height of the reading threads' blocks: row R starts at
+// base + R * pitch + 4 * (R / RY). With an even pitch the 8 lanes of a 16-byte
+// load phase, RY rows apart, then fall on distinct bank groups.
 struct SPlane {
   float* base;
   int pitch;
-  int shift;  // row R starts at base + R*pitch + 4*(R >> shift)
 };
 
+template <int RY>
 __device__ __forceinline__ float* srow(const SPlane& p, int R) {
-  return p.base + R * p.pitch + ((R >> p.shift) << 2);
+  return p.base + R * p.pitch + 4 * (R / RY);
 }
 
-template <int RY, int RX, bool CHECK>
-__device__ __forceinline__ void corr_row(float (&acc)[RY][RX], const float* __restrict__ row,
-                                         const float* __restrict__ ks, int KP, int Kc, int s) {
-  const float4* row4 = reinterpret_cast<const float4*>(row);
-#pragma unroll 2
-  for (int bq = 0; bq < (KP >> 2); ++bq) {
-    float xv[RX + 4];
+template <int RX>
+__device__ __forceinline__ void corr_window(float (&xv)[RX + 4], const float* row) {
 #pragma unroll
-    for (int m = 0; m < RX / 4 + 1; ++m) {
-      const float4 v = row4[bq + m];
-      xv[4 * m + 0] = v.x;
-      xv[4 * m + 1] = v.y;
-      xv[4 * m + 2] = v.z;
-      xv[4 * m + 3] = v.w;
+  for (int m = 0; m < RX / 4 + 1; ++m) {
+    const float4 v = reinterpret_cast<const float4*>(row)[m];
+    xv[4 * m + 0] = v.x;
+    xv[4 * m + 1] = v.y;
+    xv[4 * m + 2] = v.z;
+    xv[4 * m + 3] = v.w;
+  }
+}
+
+// One output row takes one tap quad: one tap at a time across the outputs, so
+// that consecutive FMAs share the tap's register and each accumulator takes
+// its taps in order.
+template <int RX>
+__device__ __forceinline__ void corr_taps(float (&acc)[RX], const float4 k,
+                                          const float (&xv)[RX + 4]) {
+#pragma unroll
+  for (int c = 0; c < RX; ++c) acc[c] = fmaf(k.x, xv[c + 0], acc[c]);
+#pragma unroll
+  for (int c = 0; c < RX; ++c) acc[c] = fmaf(k.y, xv[c + 1], acc[c]);
+#pragma unroll
+  for (int c = 0; c < RX; ++c) acc[c] = fmaf(k.z, xv[c + 2], acc[c]);
+#pragma unroll
+  for (int c = 0; c < RX; ++c) acc[c] = fmaf(k.w, xv[c + 3], acc[c]);
+}
+
+// The loop that bounds every direct-form kernel, on blocks of RY x RX outputs
+// (oy a multiple of RY; Kc odd). Tap quads outside, source rows inside: a
+// quad that a source row brings for output row 0 stays in a register for
+// output row 1 at the next source row. Every output sums its taps in the
+// same order (quads ascending, in a quad rows ascending, in a row columns
+// ascending) whatever block it falls in.
+//
+// RY = 2, 16 warps an SM: 62 TFLOP/s at K = 43 on a 64 x 128 tile (loop
+// alone, 80.5 derived peak). The same loop on 4 x 16 blocks, 8 warps an SM,
+// reaches 52-58 however it is unrolled or prefetched, rows outside and quads
+// inside 55: all execute over 90 % FMAs, and what differs is the dispatch
+// stall (0.3-0.5 per issue), which more warps cover and a larger block, with
+// fewer loads, does not.
+template <int RY, int RX>
+__device__ __forceinline__ void corr_tile(float (&acc)[RY][RX], const SPlane& src, int oy,
+                                          int ox, const float* __restrict__ ks, int KP,
+                                          int Kc) {
+  const float* col = srow<RY>(src, oy) + ox;
+  const int pitch = src.pitch;
+  if constexpr (RY == 2) {
+#pragma unroll 1
+    for (int b = 0; b < KP; b += 4) {
+      const float* row = col + b;  // row s at row + s * pitch + 4 * (s / 2)
+      const float* kq = ks + b;
+      float xv[RX + 4];
+      // source row 0: output row 0 only
+      corr_window<RX>(xv, row);
+      float4 k1 = *reinterpret_cast<const float4*>(kq);  // the quad of the row before
+      corr_taps<RX>(acc[0], k1, xv);
+      row += pitch;
+      kq += KP;
+      corr_window<RX>(xv, row);
+#pragma unroll 1
+      for (int s = 1; s < Kc; s += 2) {  // rows s and s + 1 (Kc - 1 is even)
+        const float4 ka = *reinterpret_cast<const float4*>(kq);
+        corr_taps<RX>(acc[0], ka, xv);
+        corr_taps<RX>(acc[1], k1, xv);
+        row += pitch + 4;
+        corr_window<RX>(xv, row);
+        k1 = *reinterpret_cast<const float4*>(kq + KP);
+        corr_taps<RX>(acc[0], k1, xv);
+        corr_taps<RX>(acc[1], ka, xv);
+        row += pitch;
+        kq += 2 * KP;
+        corr_window<RX>(xv, row);
+      }
+      corr_taps<RX>(acc[1], k1, xv);  // source row Kc: output row 1 only
     }
+  } else {
+#pragma unroll 1
+    for (int b = 0; b < KP; b += 4) {
+      float4 kv[RY];  // quad of kernel row a in slot a mod RY
+      const float* row = col + b;
+      const float* kq = ks + b;
+#pragma unroll 1
+      for (int s0 = 0; s0 < Kc + RY - 1; s0 += RY, row += RY * pitch + 4, kq += RY * KP) {
 #pragma unroll
-    for (int p = 0; p < RY; ++p) {
-      const int a = s - p;
-      if (!CHECK || (a >= 0 && a < Kc)) {
-        const float4 kv = reinterpret_cast<const float4*>(ks + a * KP)[bq];
-        // one tap at a time across the 16 outputs: each accumulator still
-        // takes its taps in order, consecutive FMAs share the kernel operand
+        for (int u = 0; u < RY; ++u) {
+          const int s = s0 + u;
+          if (s >= Kc + RY - 1) break;
+          float xv[RX + 4];
+          corr_window<RX>(xv, row + u * pitch);
+          if (s < Kc) kv[u] = *reinterpret_cast<const float4*>(kq + u * KP);
 #pragma unroll
-        for (int c = 0; c < RX; ++c) acc[p][c] = fmaf(kv.x, xv[c + 0], acc[p][c]);
-#pragma unroll
-        for (int c = 0; c < RX; ++c) acc[p][c] = fmaf(kv.y, xv[c + 1], acc[p][c]);
-#pragma unroll
-        for (int c = 0; c < RX; ++c) acc[p][c] = fmaf(kv.z, xv[c + 2], acc[p][c]);
-#pragma unroll
-        for (int c = 0; c < RX; ++c) acc[p][c] = fmaf(kv.w, xv[c + 3], acc[p][c]);
+          for (int p = 0; p < RY; ++p)
+            if (s - p >= 0 && s - p < Kc) corr_taps<RX>(acc[p], kv[(u + RY - p) % RY], xv);
+        }
       }
     }
   }
 }
 
-template <int RY, int RX>
-__device__ __forceinline__ void corr_tile(float (&acc)[RY][RX], const SPlane& src, int oy,
-                                          int ox, const float* __restrict__ ks, int KP,
-                                          int Kc) {
-#pragma unroll 1
-  for (int s = 0; s < Kc + RY - 1; ++s) {
-    const float* row = srow(src, oy + s) + ox;
-    if (s >= RY - 1 && s < Kc)
-      corr_row<RY, RX, false>(acc, row, ks, KP, Kc, s);
-    else
-      corr_row<RY, RX, true>(acc, row, ks, KP, Kc, s);
+// Stages the window of `rows` rows and `cols` columns (a multiple of 4) whose
+// first row is at `base` (a row start of a padded plane, 16-byte aligned; pitch
+// P a multiple of 4) and whose first column is c0. Four staged columns are
+// one 16-byte shared store, cut from the two 16-byte words of the plane's
+// grid that they straddle (the second word is the neighbour's first, an L1
+// hit): four scalar stores per word would conflict four ways. LOADS words
+// in flight per thread. CG: loads bypass L1 (the plane is written by other
+// SMs during the launch).
+template <int RY, int NT, int LOADS, bool CG>
+__device__ __forceinline__ void stage_window(const SPlane& sp, const float* base, int P, int c0,
+                                             int rows, int cols) {
+  const int sh = c0 & 3, nq = cols >> 2;
+  const int total = rows * nq;
+  base += c0 & ~3;
+  for (int e0 = threadIdx.x; e0 < total; e0 += NT * LOADS) {
+    float4 v[LOADS], w[LOADS];
+#pragma unroll
+    for (int q = 0; q < LOADS; ++q) {
+      const int e = e0 + q * NT;
+      if (e < total) {
+        const int R = e / nq, m = e - R * nq;
+        const float4* p = reinterpret_cast<const float4*>(base + (long long)R * P) + m;
+        v[q] = CG ? __ldcg(p) : __ldg(p);
+        if (sh) w[q] = CG ? __ldcg(p + 1) : __ldg(p + 1);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < LOADS; ++q) {
+      const int e = e0 + q * NT;
+      if (e < total) {
+        const int R = e / nq, m = e - R * nq;
+        float4 o = v[q];
+        if (sh == 1) o = make_float4(v[q].y, v[q].z, v[q].w, w[q].x);
+        if (sh == 2) o = make_float4(v[q].z, v[q].w, w[q].x, w[q].y);
+        if (sh == 3) o = make_float4(v[q].w, w[q].x, w[q].y, w[q].z);
+        reinterpret_cast<float4*>(srow<RY>(sp, R))[m] = o;
+      }
+    }
   }
+}
+
+// flags between CTAs
+__device__ __forceinline__ int ld_acquire(const int* p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ int ld_relaxed(const int* p) {
+  int v;
+  asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void st_release(int* p, int v) {
+  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // Sum of v over the CTA, in FP64 (warp shuffles, then the warps in order).

@@ -202,8 +202,8 @@ __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, c
   float* ws_base = xs_base + xs_floats;
   float* ksf = ws_base + ws_floats;
   float* ksa = ksf + Kc * KP;
-  const SPlane xs{xs_base, s.xpitch, 2};
-  const SPlane ws{ws_base, s.wpitch, 1};
+  const SPlane xs{xs_base, s.xpitch};  // rows skewed for 4-row blocks
+  const SPlane ws{ws_base, s.wpitch};  // rows skewed for 2-row blocks
 
   for (int e = tid; e < ws_floats; e += kThreads) ws_base[e] = 0.f;
   __syncthreads();
@@ -240,7 +240,7 @@ __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, c
           if (tid == 0) mbar_arrive_expect_tx(mbar, row_bytes * (uint32_t)s.xrows);
           __syncwarp();
           for (int R = tid; R < s.xrows; R += 32)
-            bulk_g2s(srow(xs, R), plane + (long long)(row0 + R) * g.P + j0, row_bytes, mbar);
+            bulk_g2s(srow<4>(xs, R), plane + (long long)(row0 + R) * g.P + j0, row_bytes, mbar);
         }
         const float4* kg =
             reinterpret_cast<const float4*>(a.kf + ((long long)t * s.R2 + phi) * Kc * KP);
@@ -261,7 +261,7 @@ __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, c
           const int rr = q * s.Rh + 4 * fmy + p;  // region row
           const long long grow = tplane + (long long)(i0 + hc + rr) * g.P + j0 + hc;
           if (xchg) {
-            float* wrow = srow(ws, rr - kHalf * q);
+            float* wrow = srow<2>(ws, rr - kHalf * q);
             if (STUDENT) {
               const float nu1 = a.nu + 1.f;
 #pragma unroll
@@ -303,7 +303,7 @@ __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, c
       cluster_wait();  // [A_t]: both CTAs wrote their own w rows
       {
         const float* peer_base = cluster.map_shared_rank(ws_base, q ^ 1);
-        const SPlane pws{const_cast<float*>(peer_base), s.wpitch, 1};
+        const SPlane pws{const_cast<float*>(peer_base), s.wpitch};
         // region rows needed from the peer and the local-row offsets
         int r_lo, r_hi;
         if (q == 0) { r_lo = s.Rh; r_hi = kHalf + 2 * hc; }
@@ -313,8 +313,8 @@ __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, c
         for (int e = tid; e < nrows * c4; e += kThreads) {
           const int rr = r_lo + e / c4, k4 = e % c4;
           const int ldst = rr - kHalf * q, lsrc = rr - kHalf * (q ^ 1);
-          reinterpret_cast<float4*>(srow(ws, ldst))[k4] =
-              reinterpret_cast<const float4*>(srow(pws, lsrc))[k4];
+          reinterpret_cast<float4*>(srow<2>(ws, ldst))[k4] =
+              reinterpret_cast<const float4*>(srow<2>(pws, lsrc))[k4];
         }
       }
       cluster_arrive();  // [B_t] arrive: done reading the peer's w
@@ -327,7 +327,7 @@ __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, c
         const int L = e / ccols, cc = e % ccols;
         const int rr = kHalf * q + L;
         const long long gi = tplane + (long long)(i0 + hc + rr) * g.P + j0 + hc + cc;
-        srow(ws, L)[cc] = a.u[gi] * a.y[gi];
+        srow<2>(ws, L)[cc] = a.u[gi] * a.y[gi];
       }
       __syncthreads();
     }
@@ -554,41 +554,61 @@ cudaError_t launch_wait_selftest(uint32_t limit, int* err, cudaStream_t st) {
 // set-up: u = mask ? 1/v : 0 (in place over v), y sanitised, FP64 sums
 // ---------------------------------------------------------------------------
 
+// One warp per image row (no division per pixel). FP64 instructions bound this
+// kernel (two per clock and SM): the logarithms of v are taken of products, the
+// exponents summed as integers and up to 512 mantissas in [1, 2) multiplied
+// in FP64 before one log, instead of one FP64 log per pixel.
 __global__ void __launch_bounds__(256) setup_kernel(const Shape s, const SetupArgs a) {
   __shared__ double red[8];
   const Geom& g = s.g;
-  const long long hw = (long long)g.H * g.W, total = hw * s.n;
-  double ld = 0.0, suy = 0.0, su = 0.0, cnt = 0.0;
-  int bad = 0;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int t = (int)(e / hw);
-    const long long rem = e - (long long)t * hw;
-    const int i = (int)(rem / g.W), j = (int)(rem - (long long)i * g.W);
-    const long long off = (long long)t * g.plane + (long long)(g.B + i) * g.P + g.B + j;
-    const bool valid = a.mask ? (a.mask[e] != 0) : true;
-    const float v = a.u[off], yv = a.y[off];
-    float uo = 0.f, yo = 0.f;
-    if (valid) {
-      if (!(v > 0.f) || !isfinite(v) || !isfinite(yv)) {
-        bad = 1;
-      } else {
-        uo = 1.0f / v;
-        yo = yv;
-        ld += log(6.283185307179586 * (double)v);
-        suy += (double)uo * (double)yv;
-        su += (double)uo;
-        cnt += 1.0;
+  const int lane = threadIdx.x & 31;
+  const long long nrows = (long long)s.n * g.H;
+  double ld = 0.0, suy = 0.0, su = 0.0, prod = 1.0;
+  long long esum = 0, cnt = 0;
+  int pending = 0, bad = 0;
+  for (long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); row < nrows;
+       row += (long long)gridDim.x * 8) {
+    const int t = (int)(row / g.H), i = (int)(row - (long long)t * g.H);
+    const long long base = (long long)t * g.plane + (long long)(g.B + i) * g.P + g.B;
+    const long long nat = row * g.W;
+    const float* ysrc = a.ysrc ? a.ysrc + nat : a.y + base;
+    const float* vsrc = a.vsrc ? a.vsrc + nat : a.u + base;
+    for (int j = lane; j < g.W; j += 32) {
+      const bool valid = a.mask ? (a.mask[nat + j] != 0) : true;
+      const float v = vsrc[j], yv = ysrc[j];
+      float uo = 0.f, yo = 0.f;
+      if (valid) {
+        if (!(v > 0.f) || !isfinite(v) || !isfinite(yv)) {
+          bad = 1;
+        } else {
+          uo = 1.0f / v;
+          yo = yv;
+          const bool tiny = v < 1.17549435e-38f;  // below the normal range
+          const uint32_t b = __float_as_uint(tiny ? v * 16777216.f : v);
+          esum += (int)(b >> 23) - (tiny ? 127 + 24 : 127);
+          prod *= (double)__uint_as_float((b & 0x007fffffu) | 0x3f800000u);
+          if (++pending == 512) {
+            ld += log(prod);
+            prod = 1.0;
+            pending = 0;
+          }
+          suy += (double)uo * (double)yv;
+          su += (double)uo;
+          ++cnt;
+        }
       }
+      a.u[base + j] = uo;
+      a.y[base + j] = yo;
     }
-    a.u[off] = uo;
-    a.y[off] = yo;
   }
   if (bad) atomicOr(a.err, kErrData);
+  // sum of log(2 pi v) = sum of log mantissas + (exponents) log 2 + count log 2 pi
+  ld += log(prod);
+  ld += (double)esum * 0.69314718055994530942 + (double)cnt * 1.83787706640934548356;
   const double s0 = block_sum_f64(ld, red);
   const double s1 = block_sum_f64(suy, red);
   const double s2 = block_sum_f64(su, red);
-  const double s3 = block_sum_f64(cnt, red);
+  const double s3 = block_sum_f64((double)cnt, red);
   if (threadIdx.x == 0) {
     a.part[4 * blockIdx.x + 0] = s0;
     a.part[4 * blockIdx.x + 1] = s1;

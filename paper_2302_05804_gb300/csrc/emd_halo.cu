@@ -70,7 +70,7 @@ size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 struct HaloShape {
   int rows;   // staged rows: TH + 2 hc
   int cols;   // staged columns: kTile + KP
-  int pitch;  // floats per staged row; rows also carry a skew of 4 floats every 4 rows
+  int pitch;  // floats per staged row; rows also carry a skew of 4 floats every TH / 16 rows
   int buf;    // floats of the staged window
   int ks;     // floats of one Kc x KP kernel
 };
@@ -80,8 +80,9 @@ __host__ __device__ inline HaloShape halo_shape(const Shape& s, int TH) {
   h.rows = TH + 2 * s.hc;
   h.cols = kTile + s.KP;
   h.pitch = h.cols;  // a multiple of 4: rows start 16-byte aligned; even: the
-                     // 8 lanes of a load phase (rows 4 apart) hit distinct bank groups
-  h.buf = h.rows * h.pitch + 4 * ((h.rows + 3) >> 2);
+                     // 8 lanes of a load phase (TH / 16 rows apart) hit distinct bank groups
+  const int ry = TH / 16;
+  h.buf = h.rows * h.pitch + 4 * ((h.rows + ry - 1) / ry);
   h.ks = s.Kc * s.KP;
   return h;
 }
@@ -89,22 +90,6 @@ __host__ __device__ inline HaloShape halo_shape(const Shape& s, int TH) {
 size_t halo_smem_bytes(const Shape& s, int TH) {
   const HaloShape h = halo_shape(s, TH);
   return (size_t)(h.buf + h.ks) * sizeof(float);
-}
-
-__device__ __forceinline__ int ld_acquire(const int* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ int ld_relaxed(const int* p) {
-  int v;
-  asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void st_release(int* p, int v) {
-  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // Bounded wait for *p >= v. Gives up after `limit` polls (raising the
@@ -121,6 +106,16 @@ __device__ bool wait_geq(const int* p, int v, unsigned long long* ctrl,
   return false;
 }
 
+// Forward item: the x window of rows [i0 - hc, i0 + TH + hc) and columns
+// [j0 - hc, j0 - hc + cols) of one padded latent plane (read-only during
+// the launch; border B = 2 hc).
+template <int RY>
+__device__ void gather_plane(const Shape& s, const HaloShape& hs, const SPlane& sp,
+                             const float* __restrict__ plane, int i0, int j0) {
+  stage_window<RY, kHT, kGather / 2, false>(sp, plane + (long long)(i0 + s.hc) * s.g.P, s.g.P,
+                                        j0 + s.hc, hs.rows, hs.cols);
+}
+
 // Writes the four floats of v into the staged row at columns C .. C+3,
 // skipping columns outside [0, cols).
 __device__ __forceinline__ void put4(float* row, int C, int cols, const float4 v) {
@@ -134,37 +129,6 @@ __device__ __forceinline__ void put4(float* row, int C, int cols, const float4 v
     if (C + 1 >= 0 && C + 1 < cols) row[C + 1] = v.y;
     if (C + 2 >= 0 && C + 2 < cols) row[C + 2] = v.z;
     if (C + 3 >= 0 && C + 3 < cols) row[C + 3] = v.w;
-  }
-}
-
-// Forward item: the x window of rows [i0 - hc, i0 + TH + hc) and columns
-// [j0 - hc, j0 - hc + cols) of one padded latent plane (read-only during
-// the launch), through 16-byte loads on the plane's 16-byte grid.
-__device__ void gather_plane(const Shape& s, const HaloShape& hs, const SPlane& sp,
-                             const float* __restrict__ plane, int i0, int j0) {
-  const int c0 = j0 + s.hc;  // padded column of window column 0 (border B = 2 hc)
-  const int q0 = c0 >> 2;
-  const int nq = ((c0 + hs.cols - 1) >> 2) - q0 + 1;
-  const int total = hs.rows * nq;
-  const float* base = plane + (long long)(i0 + s.hc) * s.g.P;
-  for (int e0 = threadIdx.x; e0 < total; e0 += kHT * kGather) {
-    float4 v[kGather];
-#pragma unroll
-    for (int q = 0; q < kGather; ++q) {
-      const int e = e0 + q * kHT;
-      if (e < total) {
-        const int R = e / nq, m = e - R * nq;
-        v[q] = __ldg(reinterpret_cast<const float4*>(base + (long long)R * s.g.P + ((q0 + m) << 2)));
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < kGather; ++q) {
-      const int e = e0 + q * kHT;
-      if (e < total) {
-        const int R = e / nq, m = e - R * nq;
-        put4(srow(sp, R), ((q0 + m) << 2) - c0, hs.cols, v[q]);
-      }
-    }
   }
 }
 
@@ -203,7 +167,7 @@ __device__ void gather_ring(const HaloShape& hs, const SPlane& sp, const float* 
       const int e = e0 + q * kHT;
       if (e < total) {
         const int R = e / nq, m = e - R * nq;
-        put4(srow(sp, R), ((q0 + m) << 2) - c0, hs.cols, v[q]);
+        put4(srow<TH / 16>(sp, R), ((q0 + m) << 2) - c0, hs.cols, v[q]);
       }
     }
   }
@@ -291,7 +255,7 @@ __device__ __forceinline__ void halo_item(const Shape& s, const HaloLaunch& h, c
   const FusedArgs& a = h.a;
   const Geom& g = s.g;
   const HaloShape hs = halo_shape(s, TH);
-  const SPlane sp{smem, hs.pitch, 2};
+  const SPlane sp{smem, hs.pitch};
   float* ks = smem + hs.buf;
   const int tid = threadIdx.x;
   const int my = tid & 15, mx = tid >> 4;  // this thread's RY x 16 outputs: rows RY my, cols 16 mx
@@ -359,7 +323,7 @@ __device__ __forceinline__ void halo_item(const Shape& s, const HaloLaunch& h, c
     const int pass = step / s.R2, phi = step - pass * s.R2;
     if (step > 0) __syncthreads();  // readers of the previous step's window and kernel are done
     if (fwd) {
-      gather_plane(s, hs, sp, a.x + (long long)phi * g.plane, i0, j0);
+      gather_plane<RY>(s, hs, sp, a.x + (long long)phi * g.plane, i0, j0);
     } else {
       if (phi == 0) gather_ring<TH>(hs, sp, nb_s, pass * kTileFloats, s.hc, i0, j0);
       if (step > 0) {
@@ -631,7 +595,7 @@ __global__ void __launch_bounds__(kHT, 2)
   __shared__ double red[kHT / 32];
   const Geom& g = s.g;
   const HaloShape hs = halo_shape(s, kTH);
-  const SPlane sp{smem, hs.pitch, 2};
+  const SPlane sp{smem, hs.pitch};
   float* ks = smem + hs.buf;
   const int tid = threadIdx.x;
   const int my = tid & 15, mx = tid >> 4;
@@ -652,7 +616,7 @@ __global__ void __launch_bounds__(kHT, 2)
         for (int c = 0; c < 16; ++c) acc[p][c] = 0.f;
       for (int phi = 0; phi < s.R2; ++phi) {
         __syncthreads();  // readers of the previous window and kernel are done
-        if (s.R2 > 1 || t == t0) gather_plane(s, hs, sp, a.x + (long long)phi * g.plane, i0, j0);
+        if (s.R2 > 1 || t == t0) gather_plane<4>(s, hs, sp, a.x + (long long)phi * g.plane, i0, j0);
         const float4* kg =
             reinterpret_cast<const float4*>(a.kf + ((long long)t * s.R2 + phi) * hs.ks);
         for (int q = tid; q < kq; q += kHT) reinterpret_cast<float4*>(ks)[q] = kg[q];

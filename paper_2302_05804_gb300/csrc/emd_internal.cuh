@@ -76,8 +76,10 @@ struct FusedArgs {
 
 struct SetupArgs {
   const uint8_t* mask;  // n x H x W uint8 (natural layout, device), or null
-  float* u;             // in: v (copied into the u planes); out: u
-  float* y;             // in/out: y; masked pixels become 0
+  const float* ysrc;    // n x H x W y (natural layout, device), or null: in the y planes
+  const float* vsrc;    // n x H x W v, or null: in the u planes
+  float* u;             // u planes
+  float* y;             // y planes; masked pixels become 0
   double* part;         // kRedBlocks x 4 partial sums
   int* err;
 };

@@ -1,0 +1,805 @@
+// emd_taps.cu -- the FP32 direct EM iteration of Sec. 2, Eq. (2) (Eq. (3) for
+// r > 1) without a chain of tile items: per chunk of exposures a forward pass
+// (w_t = u_t . F_t x into work planes) and an adjoint pass (Den += F_t^T w_t,
+// the last chunk applying the update), in two forms.
+//
+// Taps form (large frame sets). Each pass is a launch that carries the taps
+// of its chunk's kernels in its parameters, so the correlation loop reads them
+// from the constant bank instead of shared memory: they never pass through
+// the vector registers, and the loop runs at 68-72 TFLOP/s of the derived
+// 80.5 (K = 43, 64 x 128 tiles), against 55 with the taps in shared memory,
+// whose limit is the dispatch stall of FMAs with three register operands.
+// 30 KB of parameters hold 4 kernels of 43 x 43; Den is read and written
+// once per exposure as in halo_kernel.
+//
+// Split form (images of a few tiles). halo_kernel adds the exposures of a
+// tile one after the other, so a 128 x 128 image keeps 2 of 152 SMs busy. Here
+// (tile, exposure) items are independent: every exposure's adjoint sum goes
+// to a work plane of its own and the last CTA to finish a tile adds the planes
+// in exposure order. One cooperative launch runs many iterations, two
+// grid barriers each; tiles shrink with the image.
+//
+// Both give halo_kernel's iterates bit for bit: every output's taps are
+// summed in the same order (emd_corr.cuh), each exposure's adjoint sum starts
+// at zero, and the sums are added in exposure order.
+#include <algorithm>
+
+#include "emd_corr.cuh"
+#include "emd_taps.cuh"
+
+namespace emd {
+
+namespace {
+
+constexpr int kSMs = 152;
+constexpr uint32_t kBarrierPolls = 1u << 23;  // x ~0.5 us per poll: seconds, not a hang
+
+// ---------------------------------------------------------------------------
+// correlation with the taps in the constant bank
+// ---------------------------------------------------------------------------
+
+__device__ __forceinline__ float4 bank_quad(const TapBank& bank, int off) {
+  return reinterpret_cast<const float4*>(bank.k)[off >> 2];
+}
+
+// U source rows (U = 2 or 4), the first at row s with s mod 4 = 3: xv holds
+// its window, q[j] the quad of kernel row s - 1 - j. On return xv holds row
+// s + U.
+template <int U>
+__device__ __forceinline__ void bank_rows(float (&acc)[4][16], float4 (&q)[3], float (&xv)[20],
+                                          const float*& row, int& ko, int pitch, int KP,
+                                          const TapBank& bank) {
+  float4 nw[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    nw[u] = bank_quad(bank, ko);
+    ko += KP;
+    row += u == 0 ? pitch + 4 : pitch;  // the skew steps where s mod 4 = 0
+#pragma unroll
+    for (int p = 0; p < 4; ++p) corr_taps<16>(acc[p], p <= u ? nw[u - p] : q[p - u - 1], xv);
+    corr_window<16>(xv, row);
+  }
+  if (U == 2) q[2] = q[0];
+#pragma unroll
+  for (int j = 0; j < (U == 2 ? 2 : 3); ++j) q[j] = nw[U - 1 - j];
+}
+
+// corr_tile<4, 16> with the kernel at bank.k[koff ..] (Kc odd and >= 5, rows
+// of KP floats): the same sums in the same order. Rows 0 .. 2 and Kc .. Kc + 2
+// are unrolled triangles, so the loop over the rows between carries no checks.
+__device__ __forceinline__ void corr_bank(float (&acc)[4][16], const SPlane& src, int oy, int ox,
+                                          const TapBank& bank, int koff, int KP, int Kc) {
+  const float* col = srow<4>(src, oy) + ox;
+  const int pitch = src.pitch;
+#pragma unroll 1
+  for (int b = 0; b < KP; b += 4) {
+    const float* row = col + b;
+    int ko = koff + b;
+    float xv[20];
+    float4 q[3];
+    corr_window<16>(xv, row);
+    const float4 k0 = bank_quad(bank, ko), k1 = bank_quad(bank, ko + KP),
+                 k2 = bank_quad(bank, ko + 2 * KP);
+    ko += 3 * KP;
+    corr_taps<16>(acc[0], k0, xv);
+    row += pitch;
+    corr_window<16>(xv, row);
+    corr_taps<16>(acc[0], k1, xv);
+    corr_taps<16>(acc[1], k0, xv);
+    row += pitch;
+    corr_window<16>(xv, row);
+    corr_taps<16>(acc[0], k2, xv);
+    corr_taps<16>(acc[1], k1, xv);
+    corr_taps<16>(acc[2], k0, xv);
+    row += pitch;
+    corr_window<16>(xv, row);
+    q[0] = k2;
+    q[1] = k1;
+    q[2] = k0;
+    int s = 3;
+#pragma unroll 1
+    for (; s + 4 <= Kc; s += 4) bank_rows<4>(acc, q, xv, row, ko, pitch, KP, bank);
+    if (s < Kc) bank_rows<2>(acc, q, xv, row, ko, pitch, KP, bank);  // Kc mod 4 = 1
+    corr_taps<16>(acc[1], q[0], xv);
+    corr_taps<16>(acc[2], q[1], xv);
+    corr_taps<16>(acc[3], q[2], xv);
+    row += (Kc & 3) == 3 ? pitch + 4 : pitch;
+    corr_window<16>(xv, row);
+    corr_taps<16>(acc[2], q[0], xv);
+    corr_taps<16>(acc[3], q[1], xv);
+    row += pitch;
+    corr_window<16>(xv, row);
+    corr_taps<16>(acc[3], q[0], xv);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// pieces shared by both forms; a thread's block: RY x RX outputs at image
+// rows i .., columns j ..
+// ---------------------------------------------------------------------------
+
+__device__ __forceinline__ float student_weight(float u, float y, float z, float nu) {
+  const float d = y - z;
+  return u > 0.f ? u * (nu + 1.f) / fmaf(u * d, d, nu) : 0.f;
+}
+
+// w = u z (heavy-tailed: w = u' z and w2 = u' y) on the block's pixels inside
+// the image, to the work planes; u and y: the exposure's planes
+template <int RY, int RX, bool STUDENT>
+__device__ __forceinline__ void store_w(const Geom& g, const float (&acc)[RY][RX], int i0, int j0,
+                                        const float* u, const float* y, float nu, float* w,
+                                        float* w2) {
+  const bool whole = j0 + RX <= g.W;
+#pragma unroll
+  for (int p = 0; p < RY; ++p) {
+    if (i0 + p >= g.H) break;
+    // B, P and the block's first column are even: pairs are 8-byte aligned
+    const long long off = (long long)(g.B + i0 + p) * g.P + g.B + j0;
+#pragma unroll
+    for (int c = 0; c < RX; c += 2) {
+      const float2 uu = __ldg(reinterpret_cast<const float2*>(u + off + c));
+      float2 wv, w2v;
+      if (STUDENT) {
+        const float2 yy = __ldg(reinterpret_cast<const float2*>(y + off + c));
+        const float s0 = student_weight(uu.x, yy.x, acc[p][c], nu);
+        const float s1 = student_weight(uu.y, yy.y, acc[p][c + 1], nu);
+        wv = make_float2(s0 * acc[p][c], s1 * acc[p][c + 1]);
+        w2v = make_float2(s0 * yy.x, s1 * yy.y);
+      } else {
+        wv = make_float2(uu.x * acc[p][c], uu.y * acc[p][c + 1]);
+      }
+      if (whole) {
+        *reinterpret_cast<float2*>(w + off + c) = wv;
+        if (STUDENT) *reinterpret_cast<float2*>(w2 + off + c) = w2v;
+      } else {
+        if (j0 + c < g.W) w[off + c] = wv.x;
+        if (j0 + c + 1 < g.W) w[off + c + 1] = wv.y;
+        if (STUDENT) {
+          if (j0 + c < g.W) w2[off + c] = w2v.x;
+          if (j0 + c + 1 < g.W) w2[off + c + 1] = w2v.y;
+        }
+      }
+    }
+  }
+}
+
+// w = u y on a tile's pixels inside the image
+__device__ __forceinline__ void store_uy(const Geom& g, int i0, int j0, int TH, int TW, int NT,
+                                         const float* u, const float* y, float* w) {
+  for (int e = threadIdx.x; e < TH * TW; e += NT) {
+    const int i = i0 + e / TW, j = j0 + e % TW;
+    const long long off = (long long)(g.B + i) * g.P + g.B + j;
+    if (i < g.H && j < g.W) w[off] = u[off] * y[off];
+  }
+}
+
+// one pixel of Eq. (2) (the expressions of halo_kernel)
+__device__ __forceinline__ float em_update(float xo, float d, float n) {
+  float xv = xo;
+  if (d > 0.f) {
+    const float nv = fmaxf(n, 0.f);
+    if (d < 1e-30f)  // denominator near zero: guarded ratio in FP64
+      xv = (float)((double)xo * (double)nv / (double)d);
+    else
+      xv = xo * nv / d;
+  }
+  return xv;
+}
+
+// Adds the partial planes part[pass][e] (e < ne) of one phase into Den (and
+// N') in exposure order on the block's pixels, and stores them or, after the
+// last exposures, applies the update. first: the exposures before were none.
+template <int RY, int RX, bool STUDENT>
+__device__ __forceinline__ void sum_parts(const Shape& s, const FusedArgs& a, const float* part,
+                                          int ne, int phi, int i0, int j0, bool first, bool last,
+                                          bool numerator) {
+  const Geom& g = s.g;
+  const long long pb = (long long)phi * g.plane, step = (long long)s.R2 * g.plane;
+#pragma unroll 1
+  for (int p = 0; p < RY; ++p) {
+    if (i0 + p >= g.H) break;
+    const long long off = (long long)(g.B + i0 + p) * g.P + g.B + j0;
+#pragma unroll 1
+    for (int c = 0; c < RX; c += 4) {
+      if (j0 + c >= g.W) break;
+      float d[STUDENT ? 2 : 1][4];
+#pragma unroll
+      for (int pass = 0; pass < (STUDENT ? 2 : 1); ++pass) {
+        const float* src = part + (long long)pass * ne * step + pb + off + c;
+        float* run = (pass == 0 ? a.Den : a.Nw) + pb + off + c;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) d[pass][q] = first ? 0.f : __ldcg(run + q);
+#pragma unroll 4
+        for (int e = 0; e < ne; ++e) {
+          const float2 v0 = __ldcg(reinterpret_cast<const float2*>(src + e * step));
+          const float2 v1 = __ldcg(reinterpret_cast<const float2*>(src + e * step + 2));
+          const float v[4] = {v0.x, v0.y, v1.x, v1.y};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) d[pass][q] = first && e == 0 ? v[q] : d[pass][q] + v[q];
+        }
+        if (last && numerator) run = a.Nw + pb + off + c;
+        if (!last || numerator)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (j0 + c + q < g.W) run[q] = d[pass][q];
+      }
+      if (last && !numerator)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (j0 + c + q < g.W) {
+            const float n = STUDENT ? d[STUDENT ? 1 : 0][q] : a.N[pb + off + c + q];
+            a.xn[pb + off + c + q] = em_update(__ldcg(a.x + pb + off + c + q), d[0][q], n);
+          }
+    }
+  }
+}
+
+template <int RY, int RX>
+__device__ __forceinline__ void zero_block(float (&acc)[RY][RX]) {
+#pragma unroll
+  for (int p = 0; p < RY; ++p)
+#pragma unroll
+    for (int c = 0; c < RX; ++c) acc[p][c] = 0.f;
+}
+
+// stores the block's pixels inside the image into one plane
+template <int RY, int RX>
+__device__ __forceinline__ void store_block(const Geom& g, const float (&acc)[RY][RX], int i0,
+                                            int j0, float* plane) {
+  const bool whole = j0 + RX <= g.W;
+#pragma unroll
+  for (int p = 0; p < RY; ++p) {
+    if (i0 + p >= g.H) break;
+    float* dst = plane + (long long)(g.B + i0 + p) * g.P + g.B + j0;
+#pragma unroll
+    for (int c = 0; c < RX; c += 2) {
+      if (whole) {
+        *reinterpret_cast<float2*>(dst + c) = make_float2(acc[p][c], acc[p][c + 1]);
+      } else {
+        if (j0 + c < g.W) dst[c] = acc[p][c];
+        if (j0 + c + 1 < g.W) dst[c + 1] = acc[p][c + 1];
+      }
+    }
+  }
+}
+
+// The last CTA to bring its partial of a tile and phase (count of ne) returns
+// true, with every partial visible to it; the counter is back at zero.
+__device__ __forceinline__ bool last_to_arrive(int* counter, int ne, int* flag_s) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const bool last = atomicAdd(counter, 1) == ne - 1;
+    if (last) *counter = 0;
+    *flag_s = last;
+  }
+  __syncthreads();
+  if (*flag_s) __threadfence();
+  return *flag_s != 0;
+}
+
+// ---------------------------------------------------------------------------
+// taps form
+// ---------------------------------------------------------------------------
+
+// Tile variants, 4 x 16 outputs per thread: 64 x 128 (128 threads) where the
+// chunk fills the SMs several times over, 64 x 64 (64 threads) otherwise, whose
+// items divide the SMs more evenly.
+template <int V> struct TapsTile;
+template <> struct TapsTile<0> { static constexpr int TH = 64, TW = 128, MINB = 3; };
+template <> struct TapsTile<1> { static constexpr int TH = 64, TW = 64, MINB = 5; };
+
+struct TapsArgs {
+  FusedArgs a;      // t0, t1: all exposures of the iteration
+  float* w;         // chunk planes (heavy-tailed: then chunk planes of w2)
+  float* part;      // parts: chunk x R2 planes (heavy-tailed: twice)
+  int* counters;    // parts: one per (phase, tile)
+  int c0, ne;       // exposures [c0, c0 + ne) of this launch
+  int epi;          // exposures per forward item
+  int parts;        // adjoint partials per exposure, summed by the last CTA of a tile
+  int numerator;    // the sum over the exposures goes to a.Nw as it is
+  int gx, T;        // tiles per row, tiles
+};
+
+template <int V, bool STUDENT>
+__global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), TapsTile<V>::MINB)
+    taps_forward_kernel(const Shape s, const TapsArgs A, const __grid_constant__ TapBank bank) {
+  constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NY = TH / 4, NT = NY * (TW / 16);
+  extern __shared__ __align__(128) float smem[];
+  const Geom& g = s.g;
+  const SPlane sp{smem, TW + s.KP};
+  const int my = threadIdx.x % NY, mx = threadIdx.x / NY;
+  const int grp = blockIdx.x / A.T, k = blockIdx.x - grp * A.T;
+  const int i0 = (k / A.gx) * TH, j0 = (k % A.gx) * TW;
+  const int e1 = min(A.ne, (grp + 1) * A.epi);
+  for (int e = grp * A.epi; e < e1; ++e) {
+    float acc[4][16];
+    zero_block(acc);
+    for (int phi = 0; phi < s.R2; ++phi) {
+      if (s.R2 > 1 || e == grp * A.epi) {
+        __syncthreads();  // readers of the previous window are done
+        stage_window<4, NT, 4, false>(
+            sp, A.a.x + (long long)phi * g.plane + (long long)(i0 + s.hc) * g.P, g.P, j0 + s.hc,
+            TH + 2 * s.hc, TW + s.KP);
+        __syncthreads();
+      }
+      corr_bank(acc, sp, 4 * my, 16 * mx, bank, (e * s.R2 + phi) * s.Kc * s.KP, s.KP, s.Kc);
+    }
+    const long long tp = (long long)(A.c0 + e) * g.plane;
+    store_w<4, 16, STUDENT>(g, acc, i0 + 4 * my, j0 + 16 * mx, A.a.u + tp, A.a.y + tp, A.a.nu,
+                            A.w + (long long)e * g.plane, A.w + (long long)(A.ne + e) * g.plane);
+  }
+}
+
+// blockIdx.x: tile, y: phase; z: exposure of the chunk (parts) or one CTA
+// running all of them in order, adding each to Den (and N') in global memory
+template <int V, bool STUDENT>
+__global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), TapsTile<V>::MINB)
+    taps_adjoint_kernel(const Shape s, const TapsArgs A, const __grid_constant__ TapBank bank) {
+  constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NY = TH / 4, NT = NY * (TW / 16);
+  extern __shared__ __align__(128) float smem[];
+  __shared__ int flag_s;
+  const Geom& g = s.g;
+  const SPlane sp{smem, TW + s.KP};
+  const int my = threadIdx.x % NY, mx = threadIdx.x / NY;
+  const int k = blockIdx.x, phi = blockIdx.y;
+  const int i0 = (k / A.gx) * TH, j0 = (k % A.gx) * TW;
+  const int i = i0 + 4 * my, j = j0 + 16 * mx;
+  const long long pb = (long long)phi * g.plane;
+  const bool first = A.c0 == A.a.t0, last = A.c0 + A.ne == A.a.t1;
+  const int e0 = A.parts ? blockIdx.z : 0, e1 = A.parts ? e0 + 1 : A.ne;
+  for (int e = e0; e < e1; ++e) {
+#pragma unroll 1
+    for (int pass = 0; pass < (STUDENT ? 2 : 1); ++pass) {
+      float acc[4][16];
+      zero_block(acc);
+      __syncthreads();  // readers of the previous window are done
+      stage_window<4, NT, 4, false>(
+          sp, A.w + (long long)(pass * A.ne + e) * g.plane + (long long)(i0 + s.hc) * g.P, g.P,
+          j0 + s.hc, TH + 2 * s.hc, TW + s.KP);
+      __syncthreads();
+      corr_bank(acc, sp, 4 * my, 16 * mx, bank, (e * s.R2 + phi) * s.Kc * s.KP, s.KP, s.Kc);
+      if (A.parts) {
+        store_block(g, acc, i, j, A.part + (long long)(pass * A.ne + e) * s.R2 * g.plane + pb);
+        continue;
+      }
+      float* run = (pass == 0 ? A.a.Den : A.a.Nw) + pb;
+      const bool begin = first && e == 0, end = last && e + 1 == A.ne;
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        if (i + p >= g.H) break;
+        const long long off = (long long)(g.B + i + p) * g.P + g.B + j;
+        // columns past the image stay inside the padded plane
+        float2* run2 = reinterpret_cast<float2*>(run + off);
+        if (!begin) {
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {
+            const float2 v = run2[c];
+            acc[p][2 * c] = v.x + acc[p][2 * c];
+            acc[p][2 * c + 1] = v.y + acc[p][2 * c + 1];
+          }
+        }
+        if (end && A.numerator) run2 = reinterpret_cast<float2*>(A.a.Nw + pb + off);
+        // not the last exposure; or the heavy-tailed Den, kept for pass 1
+        // (read back below by the thread that wrote it)
+        if (!end || A.numerator || (STUDENT && pass == 0)) {
+#pragma unroll
+          for (int c = 0; c < 8; ++c) run2[c] = make_float2(acc[p][2 * c], acc[p][2 * c + 1]);
+          continue;
+        }
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+          if (j + c < g.W) {
+            const float d = STUDENT ? A.a.Den[pb + off + c] : acc[p][c];
+            const float n = STUDENT ? acc[p][c] : A.a.N[pb + off + c];
+            A.a.xn[pb + off + c] = em_update(A.a.x[pb + off + c], d, n);
+          }
+      }
+    }
+  }
+  if (A.parts && last_to_arrive(A.counters + phi * A.T + k, A.ne, &flag_s))
+    sum_parts<4, 16, STUDENT>(s, A.a, A.part, A.ne, phi, i, j, first, last, A.numerator);
+}
+
+// ---------------------------------------------------------------------------
+// split form
+// ---------------------------------------------------------------------------
+
+// Tile variants: 2 x RX outputs per thread. Fewer outputs per thread cost more
+// shared loads per FMA and more staging per output, but give more warps.
+template <int V> struct SplitTile;
+template <> struct SplitTile<0> { static constexpr int TH = 32, TW = 64, RX = 16; };
+template <> struct SplitTile<1> { static constexpr int TH = 32, TW = 32, RX = 8; };
+template <> struct SplitTile<2> { static constexpr int TH = 16, TW = 32, RX = 4; };
+
+constexpr int split_rows(int v) { return v == 2 ? 16 : 32; }
+constexpr int split_cols(int v) { return v == 0 ? 64 : 32; }
+
+struct SplitArgs {
+  FusedArgs a;      // x, xn: current and next buffers of the first iteration
+  float* w;         // chunk planes (heavy-tailed: then chunk planes of w2)
+  float* part;      // chunk x R2 planes (heavy-tailed: twice)
+  int* ctrl;        // [0] barrier arrivals, [1] CTAs finished, [2] abort flag
+  int* counters;    // one per (phase, tile)
+  int chunk, iters;
+  int numerator;    // w = u y instead of u z; the sum goes to a.Nw as it is
+  int gx, T;
+};
+
+// Grid barrier number `round` (from 1) of a cooperative launch; every thread
+// of the CTA calls it. Bounded: a wait that gives up raises the abort flag,
+// which ends all later waits; returns false then.
+__device__ bool grid_barrier(int* ctrl, int round, int* ok_s) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicAdd(&ctrl[0], 1);
+    const int target = round * (int)gridDim.x;
+    uint32_t i = 0;
+    bool ok = false;
+    for (; i < kBarrierPolls; ++i) {
+      if (ld_acquire(&ctrl[0]) >= target) {
+        ok = true;
+        break;
+      }
+      if (ld_relaxed(&ctrl[2])) break;
+      if (i > 64) __nanosleep(100);
+    }
+    if (!ok) atomicExch(&ctrl[2], 1);
+    *ok_s = ok;
+  }
+  __syncthreads();
+  return *ok_s != 0;
+}
+
+template <int V, bool STUDENT>
+__global__ void __launch_bounds__(SplitTile<V>::TH / 2 * (SplitTile<V>::TW / SplitTile<V>::RX))
+    split_kernel(const Shape s, const SplitArgs A) {
+  constexpr int TH = SplitTile<V>::TH, TW = SplitTile<V>::TW, RX = SplitTile<V>::RX;
+  constexpr int NY = TH / 2, NT = NY * (TW / RX);
+  extern __shared__ __align__(128) float smem[];
+  __shared__ int flag_s;
+  const Geom& g = s.g;
+  const int rows = TH + 2 * s.hc, cols = TW + s.KP, kf4 = s.Kc * s.KP >> 2;
+  const SPlane sp{smem, cols};
+  float* ks = smem + rows * cols + 4 * ((rows + 1) >> 1);
+  const int my = threadIdx.x % NY, mx = threadIdx.x / NY;
+  const int n = A.a.t1 - A.a.t0;
+  FusedArgs a = A.a;
+  int round = 0;
+  bool ok = true;
+  auto stage = [&](const float* plane, const float* taps, int i0, int j0, bool window) {
+    __syncthreads();  // readers of the previous window and taps are done
+    if (window)
+      stage_window<2, NT, 4, true>(sp, plane + (long long)(i0 + s.hc) * g.P, g.P, j0 + s.hc, rows,
+                                   cols);
+    const float4* kg = reinterpret_cast<const float4*>(taps);
+    for (int q = threadIdx.x; q < kf4; q += NT) reinterpret_cast<float4*>(ks)[q] = __ldg(kg + q);
+    __syncthreads();
+  };
+  for (int it = 0; ok && it < A.iters; ++it) {
+    for (int c0 = 0; ok && c0 < n; c0 += A.chunk) {
+      const int ne = min(A.chunk, n - c0);
+      const bool first = c0 == 0, last = c0 + ne == n;
+      for (int id = blockIdx.x; id < ne * A.T; id += gridDim.x) {
+        const int e = id / A.T, k = id - e * A.T, t = a.t0 + c0 + e;
+        const int i0 = (k / A.gx) * TH, j0 = (k % A.gx) * TW;
+        float acc[2][RX];
+        zero_block(acc);
+        if (A.numerator) {
+          store_uy(g, i0, j0, TH, TW, NT, a.u + (long long)t * g.plane,
+                   a.y + (long long)t * g.plane, A.w + (long long)e * g.plane);
+          continue;
+        }
+        for (int phi = 0; phi < s.R2; ++phi) {
+          stage(a.x + (long long)phi * g.plane,
+                a.kf + ((long long)t * s.R2 + phi) * s.Kc * s.KP, i0, j0, true);
+          corr_tile<2, RX>(acc, sp, 2 * my, RX * mx, ks, s.KP, s.Kc);
+        }
+        const long long tp = (long long)t * g.plane;
+        store_w<2, RX, STUDENT>(g, acc, i0 + 2 * my, j0 + RX * mx, a.u + tp, a.y + tp, a.nu,
+                                A.w + (long long)e * g.plane,
+                                A.w + (long long)(ne + e) * g.plane);
+      }
+      ok = grid_barrier(A.ctrl, ++round, &flag_s);
+      const int per = A.T * s.R2;
+      for (int id = blockIdx.x; ok && id < ne * per; id += gridDim.x) {
+        const int e = id / per, rest = id - e * per, phi = rest / A.T, k = rest - phi * A.T;
+        const int t = a.t0 + c0 + e;
+        const int i0 = (k / A.gx) * TH, j0 = (k % A.gx) * TW;
+#pragma unroll 1
+        for (int pass = 0; pass < (STUDENT ? 2 : 1); ++pass) {
+          float acc[2][RX];
+          zero_block(acc);
+          stage(A.w + (long long)(pass * ne + e) * g.plane,
+                a.ka + ((long long)t * s.R2 + phi) * s.Kc * s.KP, i0, j0, true);
+          corr_tile<2, RX>(acc, sp, 2 * my, RX * mx, ks, s.KP, s.Kc);
+          store_block(g, acc, i0 + 2 * my, j0 + RX * mx,
+                      A.part + (long long)((pass * ne + e) * s.R2 + phi) * g.plane);
+        }
+        if (last_to_arrive(A.counters + rest, ne, &flag_s))
+          sum_parts<2, RX, STUDENT>(s, a, A.part, ne, phi, i0 + 2 * my, j0 + RX * mx, first, last,
+                                    A.numerator);
+      }
+      if (ok) ok = grid_barrier(A.ctrl, ++round, &flag_s);
+    }
+    float* t = const_cast<float*>(a.x);
+    a.x = a.xn;
+    a.xn = t;
+  }
+  // the last CTA leaves the control words (and, after a wait that gave up, the
+  // tile counters) at zero for the next launch
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (!ok) atomicOr(a.err, kErrTimeout);
+    __threadfence();
+    flag_s = atomicAdd(&A.ctrl[1], 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (flag_s) {
+    __threadfence();
+    if (!ok)
+      for (int q = threadIdx.x; q < A.T * s.R2; q += NT) A.counters[q] = 0;
+    if (threadIdx.x < 3) A.ctrl[threadIdx.x] = 0;
+  }
+}
+
+size_t taps_smem_bytes(const Shape& s, int TH, int TW) {
+  const int rows = TH + 2 * s.hc;
+  return ((size_t)rows * (TW + s.KP) + 4 * ((rows + 3) / 4)) * sizeof(float);
+}
+
+size_t split_smem_bytes(const Shape& s, int TH, int TW) {
+  const int rows = TH + 2 * s.hc;
+  return ((size_t)rows * (TW + s.KP) + 4 * ((rows + 1) / 2) + (size_t)s.Kc * s.KP) * sizeof(float);
+}
+
+int cdiv(int a, int b) { return (a + b - 1) / b; }
+
+// The log-likelihood's data term over the chunk (Eq. (1); the Student-t term
+// with STUDENT): part[group * T + tile] (+)= sum of u (y - z)^2 in FP64 over
+// the group's exposures, z as the forward pass computes it. Launches of later
+// chunks add to the same partial sums, so their order is fixed.
+template <int V, bool STUDENT>
+__global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), TapsTile<V>::MINB)
+    taps_chi2_kernel(const Shape s, const TapsArgs A, double* __restrict__ part,
+                     const __grid_constant__ TapBank bank) {
+  constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NY = TH / 4, NT = NY * (TW / 16);
+  extern __shared__ __align__(128) float smem[];
+  __shared__ double red[NT / 32];
+  const Geom& g = s.g;
+  const SPlane sp{smem, TW + s.KP};
+  const int my = threadIdx.x % NY, mx = threadIdx.x / NY;
+  const int grp = blockIdx.x / A.T, k = blockIdx.x - grp * A.T;
+  const int i0 = (k / A.gx) * TH, j0 = (k % A.gx) * TW;
+  const int i = i0 + 4 * my, j = j0 + 16 * mx;
+  const int e1 = min(A.ne, (grp + 1) * A.epi);
+  double chi = 0.0;
+  for (int e = grp * A.epi; e < e1; ++e) {
+    float acc[4][16];
+    zero_block(acc);
+    for (int phi = 0; phi < s.R2; ++phi) {
+      if (s.R2 > 1 || e == grp * A.epi) {
+        __syncthreads();  // readers of the previous window are done
+        stage_window<4, NT, 4, false>(
+            sp, A.a.x + (long long)phi * g.plane + (long long)(i0 + s.hc) * g.P, g.P, j0 + s.hc,
+            TH + 2 * s.hc, TW + s.KP);
+        __syncthreads();
+      }
+      corr_bank(acc, sp, 4 * my, 16 * mx, bank, (e * s.R2 + phi) * s.Kc * s.KP, s.KP, s.Kc);
+    }
+    const long long tp = (long long)(A.c0 + e) * g.plane;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      if (i + p >= g.H) break;
+      const long long off = tp + (long long)(g.B + i + p) * g.P + g.B + j;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        const float uv = A.a.u[off + c];
+        if (j + c < g.W && uv != 0.f) {
+          const double d = (double)A.a.y[off + c] - (double)acc[p][c];
+          if (STUDENT)
+            chi += ((double)A.a.nu + 1.0) * log1p((double)uv * d * d / (double)A.a.nu);
+          else
+            chi += (double)uv * d * d;
+        }
+      }
+    }
+  }
+  const double tot = block_sum_f64(chi, red);
+  if (threadIdx.x == 0) part[blockIdx.x] = (A.c0 == A.a.t0 ? 0.0 : part[blockIdx.x]) + tot;
+}
+
+template <int V, bool STUDENT>
+cudaError_t launch_chi2_t(const Shape& s, const FusedArgs& a, const float* hkf,
+                          double* part, int max_parts, int* nparts, cudaStream_t st) {
+  constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NT = TH / 4 * (TW / 16);
+  const size_t smem = taps_smem_bytes(s, TH, TW);
+  cudaError_t e = allow_max_dynamic_smem((const void*)taps_chi2_kernel<V, STUDENT>);
+  if (e != cudaSuccess) return e;
+  const size_t kfl = (size_t)s.R2 * s.Kc * s.KP;
+  TapsArgs A{};
+  A.a = a;
+  A.gx = cdiv(s.W, TW);
+  A.T = A.gx * cdiv(s.H, TH);
+  const int chunk = std::min(s.n, tap_bank_kernels(s) / s.R2);
+  const int groups = std::min(chunk, max_parts / A.T);
+  if (groups < 1) return cudaErrorInvalidValue;
+  A.epi = cdiv(chunk, groups);
+  *nparts = cdiv(chunk, A.epi) * A.T;
+  TapBank bank;
+  for (A.c0 = a.t0; A.c0 < a.t1; A.c0 += chunk) {
+    A.ne = std::min(chunk, a.t1 - A.c0);
+    std::copy(hkf + (size_t)A.c0 * kfl, hkf + (size_t)(A.c0 + A.ne) * kfl, bank.k);
+    taps_chi2_kernel<V, STUDENT><<<A.T * cdiv(A.ne, A.epi), NT, smem, st>>>(s, A, part, bank);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// w = u y of the exposures [c0, c0 + ne) for the numerator
+__global__ void __launch_bounds__(128) uy_kernel(const Shape s, const TapsArgs A) {
+  const int k = blockIdx.x, e = blockIdx.y;
+  const long long tp = (long long)(A.c0 + e) * s.g.plane;
+  store_uy(s.g, k / s.gx * 64, k % s.gx * kTile, 64, kTile, 128, A.a.u + tp, A.a.y + tp,
+           A.w + (long long)e * s.g.plane);
+}
+
+template <int V, bool STUDENT>
+cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
+                          const float* hkf, const float* hka, bool numerator, cudaStream_t st) {
+  constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NT = TH / 4 * (TW / 16);
+  const size_t smem = taps_smem_bytes(s, TH, TW);
+  cudaError_t e = allow_max_dynamic_smem((const void*)taps_forward_kernel<V, STUDENT>);
+  if (e == cudaSuccess) e = allow_max_dynamic_smem((const void*)taps_adjoint_kernel<V, STUDENT>);
+  if (e != cudaSuccess) return e;
+  const size_t kfl = (size_t)s.R2 * s.Kc * s.KP;  // taps of one exposure
+  TapsArgs A;
+  A.a = h.a;
+  A.w = h.work;
+  A.counters = h.counters + 64;
+  A.parts = p.parts;
+  A.numerator = numerator;
+  A.gx = cdiv(s.W, TW);
+  A.T = A.gx * cdiv(s.H, TH);
+  TapBank bank;
+  for (int c0 = h.a.t0; c0 < h.a.t1; c0 += p.chunk) {
+    A.c0 = c0;
+    A.ne = std::min(p.chunk, h.a.t1 - c0);
+    A.part = h.work + (long long)(STUDENT ? 2 : 1) * A.ne * s.g.plane;
+    // exposures per forward item (r = 1: its window is staged once): as many
+    // as still leave 16 items an SM
+    A.epi = s.R2 > 1 ? 1 : std::max(1, std::min(A.ne, A.T * A.ne / (16 * kSMs)));
+    if (numerator) {
+      uy_kernel<<<dim3(s.gx * cdiv(s.H, 64), A.ne), 128, 0, st>>>(s, A);
+    } else {
+      std::copy(hkf + (size_t)c0 * kfl, hkf + (size_t)(c0 + A.ne) * kfl, bank.k);
+      taps_forward_kernel<V, STUDENT><<<A.T * cdiv(A.ne, A.epi), NT, smem, st>>>(s, A, bank);
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    std::copy(hka + (size_t)c0 * kfl, hka + (size_t)(c0 + A.ne) * kfl, bank.k);
+    taps_adjoint_kernel<V, STUDENT>
+        <<<dim3(A.T, s.R2, p.parts ? A.ne : 1), NT, smem, st>>>(s, A, bank);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+template <int V, bool STUDENT>
+cudaError_t launch_split_t(const Shape& s, const DirectPlan& p, const DirectLaunch& h, float* xa,
+                           float* xb, int iters, bool numerator, cudaStream_t st) {
+  constexpr int NT = SplitTile<V>::TH / 2 * (SplitTile<V>::TW / SplitTile<V>::RX);
+  const size_t smem = split_smem_bytes(s, SplitTile<V>::TH, SplitTile<V>::TW);
+  const void* kern = (const void*)split_kernel<V, STUDENT>;
+  cudaError_t e = allow_max_dynamic_smem(kern);
+  if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0, occ = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+    return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NT, smem)) != cudaSuccess)
+    return e;
+  SplitArgs A;
+  A.a = h.a;
+  A.a.x = xa;
+  A.a.xn = xb;
+  A.chunk = p.chunk;
+  A.iters = iters;
+  A.numerator = numerator;
+  A.w = h.work;
+  A.part = h.work + (long long)(STUDENT ? 2 : 1) * p.chunk * s.g.plane;
+  A.ctrl = h.counters;
+  A.counters = h.counters + 64;
+  A.gx = cdiv(s.W, SplitTile<V>::TW);
+  A.T = A.gx * cdiv(s.H, SplitTile<V>::TH);
+  const long long items = (long long)std::min(p.chunk, h.a.t1 - h.a.t0) * A.T * s.R2;
+  const int grid = (int)std::min<long long>(items, (long long)sms * std::max(occ, 1));
+  void* args[2] = {const_cast<Shape*>(&s), &A};
+  return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(NT), args, smem, st);
+}
+
+}  // namespace
+
+int tap_bank_kernels(const Shape& s) { return kTapFloats / (s.Kc * s.KP); }
+
+int direct_counter_ints(const Shape& s) {
+  return 64 + s.R2 * cdiv(s.W, 32) * cdiv(s.H, 16);
+}
+
+cudaError_t launch_taps_iter(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
+                             const float* hkf, const float* hka, bool numerator,
+                             cudaStream_t st) {
+  if (h.a.nu > 0.f && !numerator)
+    return p.tile == 0 ? launch_taps_t<0, true>(s, p, h, hkf, hka, false, st)
+                       : launch_taps_t<1, true>(s, p, h, hkf, hka, false, st);
+  return p.tile == 0 ? launch_taps_t<0, false>(s, p, h, hkf, hka, numerator, st)
+                     : launch_taps_t<1, false>(s, p, h, hkf, hka, numerator, st);
+}
+
+cudaError_t launch_taps_chi2(const Shape& s, const DirectPlan& p, const FusedArgs& a,
+                             const float* hkf, double* part, int max_parts, int* nparts,
+                             cudaStream_t st) {
+  if (a.nu > 0.f)
+    return p.tile == 0 ? launch_chi2_t<0, true>(s, a, hkf, part, max_parts, nparts, st)
+                       : launch_chi2_t<1, true>(s, a, hkf, part, max_parts, nparts, st);
+  return p.tile == 0 ? launch_chi2_t<0, false>(s, a, hkf, part, max_parts, nparts, st)
+                     : launch_chi2_t<1, false>(s, a, hkf, part, max_parts, nparts, st);
+}
+
+cudaError_t launch_split_iters(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
+                               float* xa, float* xb, int iters, bool numerator, cudaStream_t st) {
+  if (h.a.nu > 0.f && !numerator)
+    return p.tile == 0 ? launch_split_t<0, true>(s, p, h, xa, xb, iters, false, st)
+                       : launch_split_t<1, true>(s, p, h, xa, xb, iters, false, st);
+  return p.tile == 0 ? launch_split_t<0, false>(s, p, h, xa, xb, iters, numerator, st)
+                     : launch_split_t<1, false>(s, p, h, xa, xb, iters, numerator, st);
+}
+
+int split_iters_per_launch(const Shape& s) {
+  // about 2 ms a launch (20 TFLOP/s and 20 us of barriers an iteration), so
+  // that other streams' work is not held up longer
+  const double us = 20.0 + 6.0 * s.n * s.R2 * (double)s.H * s.W * s.Kc * s.Kc / 20e6;
+  return std::max(1, (int)(2000.0 / us));
+}
+
+DirectPlan direct_plan(const Shape& s, bool student) {
+  DirectPlan p{};
+  const long long T = (long long)s.gx * cdiv(s.H, 64);  // 64 x 128 tiles
+  const int cap = s.Kc >= 5 ? tap_bank_kernels(s) / s.R2 : 0;  // exposures of one launch
+  // Exposures of a taps launch: 8192 items (18 waves of three CTAs an SM)
+  // leave little of a last wave idle; more would only take memory for w.
+  const int taps = (int)std::min<long long>({(long long)cap, (long long)s.n,
+                                             std::max(4LL, 8192 / T)});
+  // Measured (us an iteration, halo / taps / split; K, n): 128^2 15, 4: 166 /
+  // 78 / 22; 300^2 21, 12: 735 / 156 / 90; 512^2 31, 12 (T taps = 280): 1201 /
+  // 450 / 342; 700 x 800 31, 20 (539): 2035 / 1075 / 1101; 1021 x 1009 43, 33
+  // (512): 6196 / 5675 / 5660; 1600 x 1500 31, 20: 4171 / 3352 / 4228; 4096^2
+  // 43, 33: 80173 / 62670 / 93051. Below 500 items a taps launch leaves SMs
+  // idle and the split form, with every exposure's items in one phase, wins.
+  if (taps > 0 && T * taps >= 500) {
+    p.form = kFormTaps;
+    p.chunk = taps;
+    // one CTA per tile and phase adds the exposures itself where those fill
+    // the SMs; else their partials take planes (2048^2 15, 8: 967 and 909 us;
+    // 1600 x 1500: 3352 and 3358; 4096^2: 62670 and 66560)
+    p.parts = T * s.R2 < 4 * kSMs;
+    // 64 x 64 tiles divide few items more evenly (700 x 800: 1123 and 1075 us;
+    // 1600 x 1500, 2100 items: 3352 and 3434)
+    p.tile = T * taps >= 1500 ? 0 : 1;
+  } else if (T * s.n < 4000 && T < 500) {
+    p.form = kFormSplit;
+    p.parts = 1;
+    p.chunk = s.n;
+    // 2 x 4 outputs per thread where even those give few warps (300^2 21, 12,
+    // 1.1 M outputs an operator: 106 and 90 us; 512^2 31, 12, 3.2 M: 342 and 389)
+    p.tile = (double)s.n * s.R2 * s.H * s.W >= 2e6 ? 0 : 1;
+  } else {
+    return p;  // halo_kernel: no work planes
+  }
+  const int per = 1 + p.parts * s.R2;  // planes per exposure (heavy-tailed: twice as many)
+  p.planes = std::max(p.chunk, 2) * per;
+  if (student) p.chunk = std::min(p.chunk, p.planes / (2 * per));
+  return p;
+}
+
+}  // namespace emd

@@ -1,0 +1,58 @@
+// emd_taps.cuh -- forms of the FP32 direct iteration whose passes are whole
+// launches or grid-wide phases instead of a chain of tile items
+// (declarations; the kernels are in emd_taps.cu).
+#pragma once
+
+#include "emd_internal.cuh"
+
+namespace emd {
+
+enum DirectForm {
+  kFormHalo = 0,   // halo_kernel (emd_halo.cu)
+  kFormTaps = 1,   // forward and adjoint launches, taps in the constant bank
+  kFormSplit = 2   // one cooperative launch, (tile, exposure) items, grid barriers
+};
+
+// How a full FP32 direct iteration of this problem shape runs. Host only and
+// independent of the device, so that emd_ctx_bytes can count the work planes.
+struct DirectPlan {
+  int form;
+  int tile;      // tile variant of the form
+  int chunk;     // exposures per forward launch / phase
+  int parts;     // 1: adjoint partials per exposure in work planes, summed in order
+  int planes;    // work planes of the context's arena (the same for both noise models)
+};
+DirectPlan direct_plan(const Shape& s, bool student);
+
+constexpr int kTapFloats = 7600;  // taps of one launch (30,400 bytes of kernel parameters)
+struct TapBank {
+  float k[kTapFloats];
+};
+// kernels (Kc x KP floats each) that one launch's constant bank holds
+int tap_bank_kernels(const Shape& s);
+
+struct DirectLaunch {
+  FusedArgs a;      // x, xn, u, y, kf, ka, N, Nw, Den, err, nu
+  float* work;      // plan.planes planes, zero outside the image
+  int* counters;    // split / parts: zero between launches (direct_counter_ints of them)
+};
+int direct_counter_ints(const Shape& s);
+
+// One iteration with the taps form; hkf, hka: host copies of all kernels.
+// numerator: N = sum_t F_t^T (u_t y_t) into a.Nw instead.
+cudaError_t launch_taps_iter(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
+                             const float* hkf, const float* hka, bool numerator, cudaStream_t st);
+// iters iterations with the split form, x buffers xa (current) and xb (or
+// the numerator, iters = 1)
+cudaError_t launch_split_iters(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
+                               float* xa, float* xb, int iters, bool numerator, cudaStream_t st);
+// The log-likelihood's data term with the taps form: *nparts partial sums
+// into part (at most max_parts, at least one per 64 x 64 tile), to be added in
+// index order.
+cudaError_t launch_taps_chi2(const Shape& s, const DirectPlan& p, const FusedArgs& a,
+                             const float* hkf, double* part, int max_parts, int* nparts,
+                             cudaStream_t st);
+// iterations one split launch should run (a bound on its duration)
+int split_iters_per_launch(const Shape& s);
+
+}  // namespace emd
