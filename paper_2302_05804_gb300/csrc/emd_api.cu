@@ -123,13 +123,8 @@ struct emd_ctx {
   // FFT path (allocated when EMD_PREC_FFT_FP32 is first selected)
   char* fft_arena = nullptr;
   size_t fft_bytes = 0;
-  float2* fft_spec = nullptr;
-  float* fft_w = nullptr;
-  float* fft_w2 = nullptr;
-  float2* fft_scratch = nullptr;
-  float2* fft_partials = nullptr;  // split launch (r = 1 Gaussian): partial accumulators
-  int* fft_counters = nullptr;     // and per-tile flags
-  size_t fft_counters_bytes = 0;
+  emd::FftLaunch fft{};            // the arena's buffers (x and xn per launch)
+  size_t fft_counters_bytes = 0;   // per-tile flags of the split launch and the groups
   int fft_split_ctas = 0;          // persistent CTAs of the split launch (one per SM)
   int fft_bound = -1;              // noise model the pointers are laid out for (-1: none)
   bool fft_ready = false;
@@ -211,7 +206,8 @@ int check_device_error(emd_ctx* c) {
   if (h & emd::kErrTimeout) {
     // a split FFT launch whose wait gave up may have left tile flags raised:
     // clear them so that the next launch starts from a clean state
-    if (c->fft_counters) CK(cudaMemsetAsync(c->fft_counters, 0, c->fft_counters_bytes, c->st));
+    if (c->fft_bound >= 0 && c->fft_counters_bytes)
+      CK(cudaMemsetAsync(c->fft.counters, 0, c->fft_counters_bytes, c->st));
     set_err("a bounded device-side wait gave up");
     return EMD_ETIMEOUT;
   }
@@ -343,7 +339,7 @@ size_t emd_ctx_bytes_precision(int H, int W, int n, int psf_k, int r, int mode) 
   if (mode == EMD_PREC_FP32) return base + emd::halo_buffer_bytes(s, false);
   if (mode == EMD_PREC_FP32_PAIR) return base;
   if (mode == EMD_PREC_FFT_FP32)
-    return base + emd::fft_buffer_bytes(s, false, current_device_sms());
+    return base + emd::fft_layout(s, false, current_device_sms()).total;
   if (mode < EMD_PREC_FP32 || mode > EMD_PREC_FFT_FP32) return 0;
   emd::TcShape t;
   if (!emd::make_tc_shape(s, mode, &t, &why)) return 0;
@@ -432,16 +428,14 @@ int emd_set_stream(emd_ctx* c, void* stream) {
 namespace {
 
 // the FFT form's buffers, sized and laid out for the context's noise model
-// (the heavy-tailed form adds the w2 planes and a larger per-tile scratch;
-// r = 1 Gaussian adds the split launch's partial accumulators, one per SM,
-// and per-tile flags); a buffer that grows is re-made, one whose layout
-// changes is re-bound (its flags cleared), and either way the PSF spectra
-// are recomputed
+// (emd::FftLayout); a buffer that grows is re-made, one whose layout changes is
+// re-bound (its flags cleared), and either way the PSF spectra are
+// recomputed
 int ensure_fft_arena(emd_ctx* c) {
   const bool student = c->noise == EMD_NOISE_STUDENT_T;
   if (c->fft_split_ctas == 0) c->fft_split_ctas = current_device_sms();
-  const size_t need = emd::fft_buffer_bytes(c->s, student, c->fft_split_ctas);
-  if (!c->fft_arena || c->fft_bytes < need) {
+  const emd::FftLayout F = emd::fft_layout(c->s, student, c->fft_split_ctas);
+  if (!c->fft_arena || c->fft_bytes < F.total) {
     if (c->fft_arena) {
       CK(cudaStreamSynchronize(c->st));
       cudaFree(c->fft_arena);
@@ -449,37 +443,45 @@ int ensure_fft_arena(emd_ctx* c) {
       c->fft_bytes = 0;
     }
     void* p = nullptr;
-    if (cudaMalloc(&p, need) != cudaSuccess) {
+    if (cudaMalloc(&p, F.total) != cudaSuccess) {
       cudaGetLastError();
-      set_err("cudaMalloc(%zu) for the FFT path failed", need);
+      set_err("cudaMalloc(%zu) for the FFT path failed", F.total);
       return EMD_ENOMEM;
     }
-    CK(cudaMemsetAsync(p, 0, need, c->st));
+    CK(cudaMemsetAsync(p, 0, F.total, c->st));
     c->fft_arena = static_cast<char*>(p);
-    c->fft_bytes = need;
+    c->fft_bytes = F.total;
     c->fft_bound = -1;
   }
   if (c->fft_bound == (int)student) return EMD_OK;
-  const size_t spec =
-      ((size_t)c->s.n * c->s.R2 * 128 * 65 * sizeof(float2) + 255) & ~(size_t)255;
-  c->fft_spec = reinterpret_cast<float2*>(c->fft_arena);
-  c->fft_w = reinterpret_cast<float*>(c->fft_arena + spec);
-  c->fft_w2 = student ? reinterpret_cast<float*>(c->fft_arena + emd::fft_w2_offset(c->s)) : nullptr;
-  c->fft_scratch =
-      reinterpret_cast<float2*>(c->fft_arena + emd::fft_scratch_offset(c->s, student));
-  const bool parts = emd::fft_buffer_bytes(c->s, student, c->fft_split_ctas) >
-                     emd::fft_buffer_bytes(c->s, student, 0);
-  c->fft_partials =
-      parts ? reinterpret_cast<float2*>(c->fft_arena + emd::fft_split_offset(c->s, student))
-            : nullptr;
-  c->fft_counters = parts ? reinterpret_cast<int*>(c->fft_arena + emd::fft_counters_offset(
-                                                                      c->s, student, c->fft_split_ctas))
-                          : nullptr;
-  c->fft_counters_bytes =
-      c->fft_counters ? need - emd::fft_counters_offset(c->s, student, c->fft_split_ctas) : 0;
-  if (c->fft_counters) CK(cudaMemsetAsync(c->fft_counters, 0, c->fft_counters_bytes, c->st));
+  auto at = [&](size_t off) { return reinterpret_cast<float2*>(c->fft_arena + off); };
+  c->fft = emd::FftLaunch{};
+  c->fft.N = c->N;
+  c->fft.u = c->u;
+  c->fft.y = c->y;
+  c->fft.err = c->err;
+  c->fft.spec = at(F.spec);
+  c->fft.spec1 = student ? at(F.spec1) : nullptr;
+  c->fft.w = at(F.w);
+  c->fft.scratch = at(F.scratch);
+  c->fft.partials = at(F.partials);
+  c->fft.counters = reinterpret_cast<int*>(c->fft_arena + F.counters);
+  c->fft.groups = emd::fft_groups(c->s);
+  c->fft.split_ctas = c->fft_split_ctas;
+  c->fft_counters_bytes = F.total - F.counters;
+  if (c->fft_counters_bytes)
+    CK(cudaMemsetAsync(c->fft.counters, 0, c->fft_counters_bytes, c->st));
   c->fft_bound = (int)student;
   c->fft_ready = false;
+  return EMD_OK;
+}
+
+// the PSF spectra, once per frame set
+int ensure_fft_spectra(emd_ctx* c) {
+  if (c->fft_ready) return EMD_OK;
+  CK(emd::launch_fft_spectra(c->s, c->ka, const_cast<float2*>(c->fft.spec),
+                             const_cast<float2*>(c->fft.spec1), c->st));
+  c->fft_ready = true;
   return EMD_OK;
 }
 
@@ -814,28 +816,12 @@ int emd_iterate(emd_ctx* c, int k) {
   DeviceGuard dg(c->device);
   if (c->prec == EMD_PREC_FFT_FP32 && k > 0) {
     if (int rc = ensure_fft_arena(c)) return rc;  // grows if the noise model changed
-    if (!c->fft_ready) {
-      CK(emd::launch_fft_spectra(c->s, c->ka, c->fft_spec, c->st));
-      c->fft_ready = true;
-    }
+    if (int rc = ensure_fft_spectra(c)) return rc;
     for (int it = 0; it < k; ++it) {
-      emd::FftLaunch L{};
+      emd::FftLaunch L = c->fft;
       L.x = c->x[c->cur];
       L.xn = c->x[c->cur ^ 1];
-      L.N = c->N;
-      L.u = c->u;
-      L.w = c->fft_w;
-      L.spec = c->fft_spec;
-      L.scratch = c->fft_scratch;
-      L.partials = c->fft_partials;
-      L.counters = c->fft_counters;
-      L.split_ctas = c->fft_split_ctas;
-      L.err = c->err;
-      if (c->noise == EMD_NOISE_STUDENT_T) {
-        L.y = c->y;
-        L.w2 = c->fft_w2;
-        L.nu = (float)c->nu;
-      }
+      L.nu = c->noise == EMD_NOISE_STUDENT_T ? (float)c->nu : 0.f;
       CK(emd::launch_fft_iter(c->s, L, c->st));
       c->cur ^= 1;
     }
@@ -1290,20 +1276,16 @@ int upload_table(emd_batch* b) {
       emd::FftBatchJob& F = ftab[i];
       F.s = c->s;
       for (int k = 0; k < 2; ++k) {
-        emd::FftLaunch& L = F.a[k];
-        L.x = c->x[k];
-        L.xn = c->x[k ^ 1];
-        L.N = c->N;
-        L.u = c->u;
-        L.w = c->fft_w;
-        L.spec = c->fft_spec;
-        L.scratch = c->fft_scratch;
+        F.a[k] = c->fft;
+        F.a[k].x = c->x[k];
+        F.a[k].xn = c->x[k ^ 1];
       }
       F.cur = c->cur;
       F.remaining = b->remaining[i];
       F.gxt = emd::fft_tiles_x(c->s);
       if (F.remaining > 0)
-        for (int t = 0; t < emd::fft_tiles_total(c->s); ++t) fitems.push_back(make_int2((int)i, t));
+        for (int t = 0; t < emd::fft_tiles_total(c->s) * c->fft.groups; ++t)
+          fitems.push_back(make_int2((int)i, t));
       continue;  // not in the direct table (remaining 0 there)
     }
     if (c->prec == EMD_PREC_FP32 && b->cur.form == 0 && c->halo_arena && b->remaining[i] > 0) {
@@ -1580,9 +1562,10 @@ int emd_batch_add(emd_batch* b, emd_ctx* c, int iterations) {
       // the job's own stream work (set_frames, set_x, its PSF spectra) must
       // be done first
       DeviceGuard dg(c->device);
-      if (c->prec == EMD_PREC_FFT_FP32 && !c->fft_ready) {
-        CK(emd::launch_fft_spectra(c->s, c->ka, c->fft_spec, c->st));
-        c->fft_ready = true;
+      if (c->prec == EMD_PREC_FFT_FP32) {
+        // (re-binds the buffers if the noise model changed since)
+        if (int rc = ensure_fft_arena(c)) return rc;
+        if (int rc = ensure_fft_spectra(c)) return rc;
       }
       if (c->prec == EMD_PREC_FP32) {
         bool ok = false;  // without a ring (too many items) the job runs the CTA-pair form

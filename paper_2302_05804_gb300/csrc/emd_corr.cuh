@@ -183,6 +183,35 @@ __device__ __forceinline__ void st_release(int* p, int v) {
   asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+constexpr uint32_t kBarrierPolls = 1u << 23;  // x ~0.5 us per poll: seconds, not a hang
+
+// Grid barrier number `round` (from 1) of a cooperative launch; every thread
+// of the CTA calls it. Bounded: a wait that gives up raises the abort flag,
+// which ends all later waits; returns false then. ctrl: [0] arrivals, [1] CTAs
+// finished, [2] abort flag.
+__device__ __forceinline__ bool grid_barrier(int* ctrl, int round, int* ok_s) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicAdd(&ctrl[0], 1);
+    const int target = round * (int)gridDim.x;
+    uint32_t i = 0;
+    bool ok = false;
+    for (; i < kBarrierPolls; ++i) {
+      if (ld_acquire(&ctrl[0]) >= target) {
+        ok = true;
+        break;
+      }
+      if (ld_relaxed(&ctrl[2])) break;
+      if (i > 64) __nanosleep(100);
+    }
+    if (!ok) atomicExch(&ctrl[2], 1);
+    *ok_s = ok;
+  }
+  __syncthreads();
+  return *ok_s != 0;
+}
+
 // Sum of v over the CTA, in FP64 (warp shuffles, then the warps in order).
 __device__ __forceinline__ double block_sum_f64(double v, double* red /* >= 8 */) {
 #pragma unroll

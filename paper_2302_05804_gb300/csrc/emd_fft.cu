@@ -1,6 +1,6 @@
 // emd_fft.cu -- the forward model and the adjoint of Eq. (2) by FFT
 // (overlap-save on 128 x 128 tiles), an alternative to the direct FP32
-// kernel. Same arithmetic type (FP32), different rounding. For r > 1 every
+// kernels. Same arithmetic type (FP32), different rounding. For r > 1 every
 // operator below acts on the polyphase planes with the Kc x Kc phase
 // kernels (hc in place of h), summed over the phases in the forward model.
 //
@@ -10,52 +10,67 @@
 // 128 x 128 array, the circular convolution of the region with k holds
 // z(i0 + p, j0 + q) at circular index (p + 2hc, q + 2hc), and the circular
 // correlation of the w region with k holds Den(i0 + p, j0 + q) at (p, q),
-// for p, q < B: no wrapped term reaches those indices. In Fourier space the
-// convolution multiplies by k^ and the correlation by conj(k^) (k is real).
+// for p, q < B: no wrapped term reaches those indices.
 //
-// 2D real transforms in shared memory, in place, each 128-point FFT done by
-// one warp in registers (radix-2 butterflies; four values per lane; the
-// cross-lane stages exchange half of a lane's values with its partner lane):
-//   forward (R2C): two real rows packed as one complex row; 64 row FFTs by
-//     decimation in frequency (natural in; frequency 32 q + rev5(l) out in
-//     slot q of lane l, stored at 32 q + l); the packed spectra split into
-//     the half spectra (65 bins) of the two rows; 65 column FFTs, again by
-//     decimation in frequency, stored the same way. Result: row frequency
-//     permuted, column frequency 0..64 natural. The PSF spectra are made by
-//     the same code, so products never need a reordering.
-//   inverse (C2R): 65 column FFTs by decimation in time with conjugate
-//     twiddles (the permuted order in, natural out); the half spectra of row
-//     pairs merged into one packed full spectrum (Hermitian symmetry),
-//     written in the permuted order; 64 row FFTs by decimation in time; real
-//     part = even row, imaginary part = odd row; scaled by 1/128^2 (exact).
-// A half-spectrum buffer is 128 rows x kFP complex; the packed row pair k
-// occupies the 2 kFP slots from 2k kFP, so splitting and merging stay in
-// place (each pair is one warp's, with a warp barrier between its reads and
-// its writes).
+// Two exposures share one complex transform, without splitting or merging.
+// With the complex kernel k = k_a + i k_b:
+//   forward  IFFT(x^ k^) = z_a + i z_b;
+//   adjoint  the real part of IFFT(FFT(w_a + i w_b) conj(k^)) is
+//            corr(w_a, k_a) + corr(w_b, k_b), which is all Den needs (the
+//            imaginary part holds cross terms and is dropped).
+// Heavy-tailed noise packs the two images of one exposure instead: with the
+// real kernel k_t, IFFT(FFT(w + i w2) conj(k_t^)) = Den_t + i N'_t.
+// x is real, so x^(-m, -f) = conj(x^(m, f)): 64 column slots (m = 1 .. 63, and
+// columns 0 and 64 in slot 0) stand for the 128 columns. Slot m serves the
+// columns m and 128 - m, the second by conjugation:
+//   forward  column 128 - m after the inverse transform over f is
+//            conj(IFFT_f(x^(m, f) S2(m, f))), S2(m, f) = conj(k^(128-m, -f));
+//   adjoint  the Hermitian part of the product, H(m, f) = Z(m, f) conj(S1(m, f))
+//            + FFT_f(conj(column 128 - m)) conj(S2(m, f)), S1 = k^.
+// So a slot's spectrum values, x^ or the accumulator H, are 16 complex
+// registers per thread for all exposures, and the tables S1 and S2 are
+// read once per pair.
 //
-// Per iteration: fft_forward_kernel (per tile: x^ once, then for each
-// exposure z = IFFT(x^ k_t^), w_t = u_t z written to a plane) and
-// fft_adjoint_kernel (per tile: sum_t FFT(w_t) conj(k_t^), one inverse
-// transform, the update of Eq. (2)), one CTA per tile; or, for r = 1
-// Gaussian with at least as many tiles as SMs, their split forms
-// (fft_forward_split_kernel, fft_adjoint_split_kernel: one persistent CTA
-// per SM, whole waves of tiles, then the last wave's tiles cut into
-// exposure ranges across all CTAs).
+// A 128-point FFT is eight lanes' work, 16 values each: a 16-point DFT in
+// registers (inputs j + 8 i of lane j), twiddles, one exchange through the
+// row's or column's own shared memory, two 8-point DFTs. Frequencies 2 t + 16 q
+// and 2 t + 1 + 16 q end in lane t (adjacent: rows move them as 16-byte words);
+// the inverse takes them there and runs the stages in reverse. The exchange
+// positions, the row pitch of 130 complex and the choice of a warp's four rows
+// and columns (Lane) keep every access free of bank conflicts.
+//
+// Against the form before (radix-2 stages across the 32 lanes of a warp,
+// two real rows per complex row, accumulators in shared memory) a transform
+// takes half the instructions and two thirds of the shared-memory passes.
+//
+// Per iteration: the forward kernel (per tile: x^ once, then per pair of
+// exposures z, w_t = u_t z_t to the w planes) and the adjoint kernel (per
+// tile: the sum over pairs, one inverse transform, the update of Eq. (2)). Work
+// items are (tile, group of exposures): images with fewer tiles than SMs
+// split the exposures into groups (fft_groups), whose accumulators the last
+// CTA of a tile adds in group order. For r = 1 Gaussian with at least as many
+// tiles as SMs the split forms run one persistent CTA per SM: whole waves of
+// tiles, then the last wave's tiles cut into exposure ranges across all CTAs.
 #include <math.h>
 
-#include "emd_internal.cuh"
+#include <algorithm>
+
+#include "emd_corr.cuh"
 #include "emd_fft.cuh"
+#include "emd_internal.cuh"
 
 namespace emd {
 namespace {
 
 constexpr int kFT = 128;                 // tile side
-constexpr int kFP = 67;                  // half-spectrum row pitch (complex, odd:
-                                         // a warp's column loads hit distinct banks)
-constexpr int kFBins = 65;               // half-spectrum columns
-constexpr int kFBuf = kFT * kFP;         // float2 per transform buffer
-constexpr int kFThreads = 512;
+constexpr int kFP = 130;                 // row pitch in shared memory (complex)
+constexpr int kFBuf = kFT * kFP;         // float2 of the transform buffer
+constexpr int kFThreads = 512;           // 64 groups of eight lanes
+constexpr int kSlots = 64 * kFT;         // float2 of the 64 column slots
+constexpr int kCol = kSlots + kFT;       // the slots, then column 64
+constexpr int kPairSpec = 2 * kSlots;    // S1, then S2 (slot 0 of S2: column 64)
 constexpr float kFScale = 1.0f / (kFT * kFT);
+constexpr int kSMs = 152;
 
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
@@ -65,976 +80,724 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {  // a conj(b)
   return make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
-__device__ __forceinline__ float2 conjf2(float2 a) { return make_float2(a.x, -a.y); }
-__device__ __forceinline__ int rev5(int m) { return (int)(__brev((unsigned)m) >> 27); }
+// a + b conj(c)
+__device__ __forceinline__ float2 cfmac(float2 a, float2 b, float2 c) {
+  a.x = fmaf(b.x, c.x, a.x);
+  a.y = fmaf(b.y, c.x, a.y);
+  a.x = fmaf(b.y, c.y, a.x);
+  a.y = fmaf(-b.x, c.y, a.y);
+  return a;
+}
+// a + b c
+__device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 c) {
+  a.x = fmaf(b.x, c.x, a.x);
+  a.y = fmaf(b.x, c.y, a.y);
+  a.x = fmaf(-b.y, c.y, a.x);
+  a.y = fmaf(b.y, c.x, a.y);
+  return a;
+}
 
-// Twiddles exp(-2 pi i k / 128), laid out so that the 32 lanes of a warp
-// read consecutive entries at every stage (no bank conflicts):
-//   w[k]        k < 64 (first stage: lane l, value q reads w[32 q + l])
-//   lane2[l]    w[2 l] (second stage)
-//   xs[k][l]    the twiddle of the cross-lane stage on lane bit k (span
-//               2^k): w[(l mod 2^k) 64 / 2^k], negated on the lanes whose bit
-//               k is set (see warp_fft_dif and warp_ifft_dit)
-struct TwTab {
-  float2 w[64];
-  float2 lane2[32];
-  float2 xs[5][32];
+// ---------------------------------------------------------------------------
+// DFTs in registers (INV: conjugate twiddles, unscaled)
+// ---------------------------------------------------------------------------
+
+// a * exp(-+ i pi / 2)
+template <bool INV>
+__device__ __forceinline__ float2 rot(float2 a) {
+  return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+}
+
+template <bool INV>
+__device__ __forceinline__ void dft4(float2& a, float2& b, float2& c, float2& d) {
+  const float2 s0 = cadd(a, c), s1 = csub(a, c), s2 = cadd(b, d), s3 = rot<INV>(csub(b, d));
+  a = cadd(s0, s2);
+  b = cadd(s1, s3);
+  c = csub(s0, s2);
+  d = csub(s1, s3);
+}
+
+// a * (wr -+ i wi): wr, wi the cosine and sine of the (positive) angle
+template <bool INV>
+__device__ __forceinline__ float2 cmulk(float2 a, float wr, float wi) {
+  return INV ? make_float2(a.x * wr - a.y * wi, a.y * wr + a.x * wi)
+             : make_float2(a.x * wr + a.y * wi, a.y * wr - a.x * wi);
+}
+
+constexpr float kR2 = 0.70710678118654752440f;   // cos(pi/4)
+constexpr float kC8 = 0.92387953251128675613f;   // cos(pi/8)
+constexpr float kS8 = 0.38268343236508977173f;   // sin(pi/8)
+
+// eight points at v[0], v[1], ..., natural in and out
+template <bool INV>
+__device__ __forceinline__ void dft8(float2* v) {
+  float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
+  dft4<INV>(e0, e1, e2, e3);
+  dft4<INV>(o0, o1, o2, o3);
+  // o1 w, o2 w^2, o3 w^3 with w = exp(-+ i pi / 4)
+  o1 = INV ? make_float2(kR2 * (o1.x - o1.y), kR2 * (o1.x + o1.y))
+           : make_float2(kR2 * (o1.x + o1.y), kR2 * (o1.y - o1.x));
+  o2 = rot<INV>(o2);
+  o3 = INV ? make_float2(-kR2 * (o3.x + o3.y), kR2 * (o3.x - o3.y))
+           : make_float2(kR2 * (o3.y - o3.x), -kR2 * (o3.x + o3.y));
+  v[0] = cadd(e0, o0);
+  v[4] = csub(e0, o0);
+  v[1] = cadd(e1, o1);
+  v[5] = csub(e1, o1);
+  v[2] = cadd(e2, o2);
+  v[6] = csub(e2, o2);
+  v[3] = cadd(e3, o3);
+  v[7] = csub(e3, o3);
+}
+
+// sixteen points, natural in and out
+template <bool INV>
+__device__ __forceinline__ void dft16(float2 (&v)[16]) {
+#pragma unroll
+  for (int b = 0; b < 4; ++b) dft4<INV>(v[b], v[4 + b], v[8 + b], v[12 + b]);  // v[4 k + b]: y_b[k]
+  v[5] = cmulk<INV>(v[5], kC8, kS8);                                      // w^1
+  v[6] = INV ? make_float2(kR2 * (v[6].x - v[6].y), kR2 * (v[6].x + v[6].y))
+             : make_float2(kR2 * (v[6].x + v[6].y), kR2 * (v[6].y - v[6].x));  // w^2
+  v[7] = cmulk<INV>(v[7], kS8, kC8);                                      // w^3
+  v[9] = INV ? make_float2(kR2 * (v[9].x - v[9].y), kR2 * (v[9].x + v[9].y))
+             : make_float2(kR2 * (v[9].x + v[9].y), kR2 * (v[9].y - v[9].x));  // w^2
+  v[10] = rot<INV>(v[10]);                                                // w^4
+  v[11] = INV ? make_float2(-kR2 * (v[11].x + v[11].y), kR2 * (v[11].x - v[11].y))
+              : make_float2(kR2 * (v[11].y - v[11].x), -kR2 * (v[11].x + v[11].y));  // w^6
+  v[13] = cmulk<INV>(v[13], kS8, kC8);                                    // w^3
+  v[14] = INV ? make_float2(-kR2 * (v[14].x + v[14].y), kR2 * (v[14].x - v[14].y))
+              : make_float2(kR2 * (v[14].y - v[14].x), -kR2 * (v[14].x + v[14].y));  // w^6
+  v[15] = cmulk<INV>(v[15], -kC8, -kS8);                                  // w^9
+#pragma unroll
+  for (int k = 0; k < 4; ++k) dft4<INV>(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+  // v[4 k1 + k2] holds X[k1 + 4 k2]: transpose the register names
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = a + 1; b < 4; ++b) {
+      const float2 t = v[4 * a + b];
+      v[4 * a + b] = v[4 * b + a];
+      v[4 * b + a] = t;
+    }
+}
+
+// (exp(-2 pi i j 2k / 128), exp(-2 pi i j (2k + 1) / 128)) at tw[8 k + j]
+__device__ __forceinline__ void init_twiddles(float4* tw) {
+  for (int e = threadIdx.x; e < kFT / 2; e += blockDim.x) {
+    const int j = e & 7, k = e >> 3;
+    float s0, c0, s1, c1;
+    sincospif((float)(2 * k * j) / 64.f, &s0, &c0);
+    sincospif((float)((2 * k + 1) * j) / 64.f, &s1, &c1);
+    tw[e] = make_float4(c0, -s0, c1, -s1);
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void twiddle(float2 (&v)[16], const float4* tw, int t) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float4 w = tw[8 * k + t];
+    if (k) v[2 * k] = cmul(v[2 * k], make_float2(w.x, w.y));
+    v[2 * k + 1] = cmul(v[2 * k + 1], make_float2(w.z, w.w));
+  }
+}
+__device__ __forceinline__ void twiddle_conj(float2 (&v)[16], const float4* tw, int t) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float4 w = tw[8 * k + t];
+    if (k) v[2 * k] = cmulc(v[2 * k], make_float2(w.x, w.y));
+    v[2 * k + 1] = cmulc(v[2 * k + 1], make_float2(w.z, w.w));
+  }
+}
+
+struct Lane {
+  int warp, grp, t;  // warp, group of eight lanes in it, lane in the group
+  __device__ Lane() : warp(threadIdx.x >> 5), grp((threadIdx.x >> 3) & 3), t(threadIdx.x & 7) {}
+  // row of group k of this warp in 32-row block blk: a half-warp's two rows are
+  // 4 apart (distinct bank pairs: 4 pitches are 8 mod 16 complex)
+  __device__ int row(int blk, int k) const {
+    return 32 * blk + (warp & 3) + 8 * ((warp >> 2) & 1) + 4 * (k & 1) + 16 * (k >> 1);
+  }
+  __device__ int row(int blk) const { return row(blk, grp); }
+  // column slot of this group: a half-warp's two columns (and partners) are adjacent
+  __device__ int slot() const { return 4 * warp + grp; }
 };
 
-__device__ __forceinline__ float2 twiddle(int k) {
-  float sn, cs;
-  sincospif((float)k / 64.f, &sn, &cs);
-  return make_float2(cs, -sn);
-}
-
-__device__ __forceinline__ void init_twiddles(TwTab& T) {
-  for (int e = threadIdx.x; e < 64 + 32 + 5 * 32; e += blockDim.x) {
-    if (e < 64) {
-      T.w[e] = twiddle(e);
-    } else if (e < 96) {
-      T.lane2[e - 64] = twiddle(2 * (e - 64));
-    } else {
-      const int k = (e - 96) >> 5, l = (e - 96) & 31, S = 1 << k;
-      const float2 w = twiddle((l & (S - 1)) * (64 >> k));
-      T.xs[k][l] = (l & S) ? make_float2(-w.x, -w.y) : w;
-    }
-  }
-  __syncthreads();
-}
-
-// J independent 128-point FFTs per warp, in registers. A lane holds four
-// values per transform; slot q = 2 s1 + s0 and lane l address element
-// e = 32 q + l of the natural input. Decimation in frequency: the spans 64
-// and 32 pair a lane's own slots (s1, then s0). Each shorter span 2^k pairs
-// the lanes l and l ^ 2^k: the two exchange the halves of their slot pairs
-// that the other needs -- lane bit k trades places with a slot bit whose
-// element bit is already done (s1, s0, s1, s0, s1 for k = 4 .. 0) -- so
-// every lane holds whole butterflies: per stage it sends two values of the
-// four and runs two butterflies, (m + o, (m - o) t) with its own value m,
-// the received o and t negated on the upper lane (the lower lane's a - b is
-// the upper lane's b - a). Output: lane l, slot q holds the spectrum at
-// 32 q + rev5(l). The J transforms share the twiddle loads and overlap each
-// other's latency (J = 2 in the row and column passes).
-template <int J, int K, int SB>  // lane bit K, slot bit SB
-__device__ __forceinline__ void dif_exchange_stage(float2 (&v)[J][4], const TwTab& T, int lane) {
-  const bool lower = ((lane >> K) & 1) == 0;
-  const float2 t = K == 0 ? make_float2(lower ? 1.f : -1.f, 0.f) : T.xs[K][lane];
+// 128-point transforms of one line of the buffer by a group of eight lanes, the
+// line's own storage carrying the exchange. Forward: v[i] = element t + 8 i in;
+// out v[q] = frequency 2 t + 16 q, v[8 + q] = 2 t + 1 + 16 q. Inverse
+// (unscaled): the reverse.
+//
+// Rows (element e at base + e, 16-byte aligned): the two frequencies of a lane
+// travel as one 16-byte word, word 8 k + (j ^ k) holding frequencies 2 k and
+// 2 k + 1 of lane j's 16-point DFT.
+__device__ __forceinline__ void fft_row(float2 (&v)[16], float2* base, const float4* tw, int t) {
+  dft16<false>(v);
+  twiddle(v, tw, t);
+  float4* b4 = reinterpret_cast<float4*>(base);
+  __syncwarp();  // the group has read its inputs from the line
 #pragma unroll
-  for (int pr = 0; pr < 2; ++pr) {
-    const int q0 = SB == 1 ? pr : 2 * pr, q1 = q0 | (1 << SB);
-    float2 mine[J], snd[J], o[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      mine[j] = lower ? v[j][q0] : v[j][q1];
-      snd[j] = lower ? v[j][q1] : v[j][q0];
-    }
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      o[j].x = __shfl_xor_sync(0xffffffffu, snd[j].x, 1 << K);
-      o[j].y = __shfl_xor_sync(0xffffffffu, snd[j].y, 1 << K);
-    }
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      v[j][q0] = cadd(mine[j], o[j]);
-      v[j][q1] = K == 0 ? make_float2(t.x * (mine[j].x - o[j].x), t.x * (mine[j].y - o[j].y))
-                        : cmul(csub(mine[j], o[j]), t);
-    }
-  }
-}
-
-template <int J>
-__device__ __forceinline__ void warp_fft_dif(float2 (&v)[J][4], const TwTab& T, int lane) {
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const float2 t = T.w[32 * q + lane];
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const float2 a = v[j][q], b = v[j][q + 2];
-      v[j][q] = cadd(a, b);
-      v[j][q + 2] = cmul(csub(a, b), t);
-    }
-  }
-  const float2 t1 = T.lane2[lane];
-#pragma unroll
-  for (int p = 0; p < 2; ++p)
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const float2 a = v[j][2 * p], b = v[j][2 * p + 1];
-      v[j][2 * p] = cadd(a, b);
-      v[j][2 * p + 1] = cmul(csub(a, b), t1);
-    }
-  dif_exchange_stage<J, 4, 1>(v, T, lane);
-  dif_exchange_stage<J, 3, 0>(v, T, lane);
-  dif_exchange_stage<J, 2, 1>(v, T, lane);
-  dif_exchange_stage<J, 1, 0>(v, T, lane);
-  dif_exchange_stage<J, 0, 1>(v, T, lane);
-}
-
-// The inverse stage of dif_exchange_stage (conjugate twiddle t*, unscaled):
-// the butterfly on the lane's own slot pair, (a + b t*, a - b t*), then the
-// same exchange of lane bit K with slot bit SB, which undoes itself. With
-// the signed twiddle s (= -t on the upper lane) and c = b s*, the lower lane
-// holds (a + c, a - c) and the upper (a - c, a + c): every lane keeps a + c,
-// sends a - c, and puts the received value in its other slot.
-template <int J, int K, int SB>
-__device__ __forceinline__ void dit_exchange_stage(float2 (&v)[J][4], const TwTab& T, int lane) {
-  const bool lower = ((lane >> K) & 1) == 0;
-  const float2 sc = K == 0 ? make_float2(lower ? 1.f : -1.f, 0.f) : conjf2(T.xs[K][lane]);
-#pragma unroll
-  for (int pr = 0; pr < 2; ++pr) {
-    const int q0 = SB == 1 ? pr : 2 * pr, q1 = q0 | (1 << SB);
-    float2 keep[J], o[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const float2 b = v[j][q1];
-      const float2 c = K == 0 ? make_float2(sc.x * b.x, sc.x * b.y) : cmul(b, sc);
-      const float2 a = v[j][q0];
-      keep[j] = cadd(a, c);
-      const float2 snd = csub(a, c);
-      o[j].x = __shfl_xor_sync(0xffffffffu, snd.x, 1 << K);
-      o[j].y = __shfl_xor_sync(0xffffffffu, snd.y, 1 << K);
-    }
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      v[j][q0] = lower ? keep[j] : o[j];
-      v[j][q1] = lower ? o[j] : keep[j];
-    }
-  }
-}
-
-// Inverse (conjugate twiddles), unscaled: input in the layout warp_fft_dif
-// leaves (lane l, slot q: frequency 32 q + rev5(l)), output natural
-// (lane l, slot q: element 32 q + l).
-template <int J>
-__device__ __forceinline__ void warp_ifft_dit(float2 (&v)[J][4], const TwTab& T, int lane) {
-  dit_exchange_stage<J, 0, 1>(v, T, lane);
-  dit_exchange_stage<J, 1, 0>(v, T, lane);
-  dit_exchange_stage<J, 2, 1>(v, T, lane);
-  dit_exchange_stage<J, 3, 0>(v, T, lane);
-  dit_exchange_stage<J, 4, 1>(v, T, lane);
-  const float2 t1 = conjf2(T.lane2[lane]);
-#pragma unroll
-  for (int p = 0; p < 2; ++p)
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const float2 a = v[j][2 * p], b = cmul(v[j][2 * p + 1], t1);
-      v[j][2 * p] = cadd(a, b);
-      v[j][2 * p + 1] = csub(a, b);
-    }
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const float2 t = conjf2(T.w[32 * q + lane]);
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const float2 a = v[j][q], b = cmul(v[j][q + 2], t);
-      v[j][q] = cadd(a, b);
-      v[j][q + 2] = csub(a, b);
-    }
-  }
-}
-
-// Position, in a row stored from the registers of warp_fft_dif (slot q of
-// lane l at 32 q + l), of frequency m: 32 (m div 32) + rev5(m mod 32).
-__device__ __forceinline__ int fpos(int m) { return (m & 96) | rev5(m & 31); }
-
-// Shared-memory slot of position i of such a row: bit 0 flipped by bits 4
-// and 5, so that a half-warp's 8-byte accesses in register order (32 q + l)
-// and in frequency order (fpos) both fall on 16 distinct bank pairs.
-__device__ __forceinline__ int rsw(int i) { return i ^ (((i >> 4) ^ (i >> 5)) & 1); }
-
-// packed row spectrum of a pair (stored as warp_fft_dif leaves it, at r) -> half spectra of the
-// even row (r[0..64]) and the odd row (r[kFP .. kFP+64]); one warp
-__device__ __forceinline__ void split_pair(float2* r, int lane) {
-  float2 e[3], o[3];
-  const int ms[3] = {lane, lane + 32, 64};
-  const int cnt = lane == 0 ? 3 : 2;
-  for (int q = 0; q < cnt; ++q) {
-    const int m = ms[q];
-    const float2 cm = r[rsw(fpos(m))], cn = conjf2(r[rsw(fpos((128 - m) & 127))]);
-    e[q] = make_float2(0.5f * (cm.x + cn.x), 0.5f * (cm.y + cn.y));
-    const float2 d = csub(cm, cn);  // (cm - conj(c_-m)) / (2i) = -i d / 2
-    o[q] = make_float2(0.5f * d.y, -0.5f * d.x);
-  }
+  for (int k = 0; k < 8; ++k)
+    b4[8 * k + (t ^ k)] = make_float4(v[2 * k].x, v[2 * k].y, v[2 * k + 1].x, v[2 * k + 1].y);
   __syncwarp();
-  for (int q = 0; q < cnt; ++q) {
-    r[ms[q]] = e[q];
-    r[kFP + ms[q]] = o[q];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const float4 w = b4[8 * t + (t ^ j)];
+    v[j] = make_float2(w.x, w.y);
+    v[8 + j] = make_float2(w.z, w.w);
   }
+  dft8<false>(v);
+  dft8<false>(v + 8);
+}
+__device__ __forceinline__ void ifft_row(float2 (&v)[16], float2* base, const float4* tw, int t) {
+  dft8<true>(v);
+  dft8<true>(v + 8);
+  float4* b4 = reinterpret_cast<float4*>(base);
+  __syncwarp();  // the group has read its inputs from the line
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    b4[8 * t + (t ^ j)] = make_float4(v[j].x, v[j].y, v[8 + j].x, v[8 + j].y);
   __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float4 w = b4[8 * k + (t ^ k)];
+    v[2 * k] = make_float2(w.x, w.y);
+    v[2 * k + 1] = make_float2(w.z, w.w);
+  }
+  twiddle_conj(v, tw, t);
+  dft16<true>(v);
 }
 
-// half spectra of a row pair -> packed full spectrum in the input layout of
-// warp_ifft_dit (frequency m at rsw(fpos(m))); one warp
-__device__ __forceinline__ void merge_pair(float2* r, int lane) {
-  float2 d[4];
+// Columns (element e at base + e kFP): frequency p of lane j's 16-point DFT at
+// element 8 p + (j ^ (p / 2)).
+__device__ __forceinline__ void fft_col(float2 (&v)[16], float2* base, const float4* tw, int t) {
+  dft16<false>(v);
+  twiddle(v, tw, t);
+  __syncwarp();  // the group has read its inputs from the line
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int m = lane + 32 * q;
-    float2 e, o;
-    if (m <= 64) {
-      e = r[m];
-      o = r[kFP + m];
-    } else {
-      e = conjf2(r[128 - m]);
-      o = conjf2(r[kFP + 128 - m]);
-    }
-    d[q] = make_float2(e.x - o.y, e.y + o.x);  // e + i o
+  for (int p = 0; p < 16; ++p) base[(8 * p + (t ^ (p >> 1))) * kFP] = v[p];
+  __syncwarp();
+  float2* mine = base + 16 * t * kFP;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    v[j] = mine[(t ^ j) * kFP];
+    v[8 + j] = mine[(8 + (t ^ j)) * kFP];
+  }
+  dft8<false>(v);
+  dft8<false>(v + 8);
+}
+__device__ __forceinline__ void ifft_col(float2 (&v)[16], float2* base, const float4* tw, int t) {
+  dft8<true>(v);
+  dft8<true>(v + 8);
+  __syncwarp();  // the group has read its inputs from the line
+  float2* mine = base + 16 * t * kFP;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    mine[(t ^ j) * kFP] = v[j];
+    mine[(8 + (t ^ j)) * kFP] = v[8 + j];
   }
   __syncwarp();
 #pragma unroll
-  for (int q = 0; q < 4; ++q) r[rsw(32 * q + rev5(lane))] = d[q];  // frequency lane + 32 q
+  for (int p = 0; p < 16; ++p) v[p] = base[(8 * p + (t ^ (p >> 1))) * kFP];
+  twiddle_conj(v, tw, t);
+  dft16<true>(v);
+}
+
+// frequencies of a row to and from its natural positions
+__device__ __forceinline__ void store_freqs(float2* row, const float2 (&v)[16], int t) {
+  float4* b4 = reinterpret_cast<float4*>(row);
+  __syncwarp();  // the group's exchange reads of this row are done
+#pragma unroll
+  for (int q = 0; q < 8; ++q) b4[t + 8 * q] = make_float4(v[q].x, v[q].y, v[8 + q].x, v[8 + q].y);
+}
+__device__ __forceinline__ void load_freqs(const float2* row, float2 (&v)[16], int t) {
+  const float4* b4 = reinterpret_cast<const float4*>(row);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const float4 w = b4[t + 8 * q];
+    v[q] = make_float2(w.x, w.y);
+    v[8 + q] = make_float2(w.z, w.w);
+  }
+}
+// elements t + 8 i of a column
+__device__ __forceinline__ void load_col(const float2* col, float2 (&v)[16], int t, bool conj) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    v[i] = col[(t + 8 * i) * kFP];
+    if (conj) v[i].y = -v[i].y;
+  }
+}
+__device__ __forceinline__ void store_col(float2* col, const float2 (&v)[16], int t, bool conj) {
+  __syncwarp();  // the group's exchange reads of this column are done
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    col[(t + 8 * i) * kFP] = conj ? make_float2(v[i].x, -v[i].y) : v[i];
+}
+
+// the same where not every group of the warp stores
+__device__ __forceinline__ void store_col_group(float2* col, const float2 (&v)[16], const Lane& L,
+                                                bool conj) {
+  __syncwarp(0xffu << (8 * L.grp));
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    col[(L.t + 8 * i) * kFP] = conj ? make_float2(v[i].x, -v[i].y) : v[i];
+}
+
+// This thread's 16 values of its column slot in a slot array: v at
+// (warp 16 + v) 32 + lane (a warp's loads are contiguous)
+__device__ __forceinline__ int slot_off() { return (threadIdx.x >> 5) * 512 + (threadIdx.x & 31); }
+__device__ __forceinline__ void store_slot(float2* a, const float2 (&v)[16]) {
+  a += slot_off();
+#pragma unroll
+  for (int i = 0; i < 16; ++i) a[32 * i] = v[i];
+}
+
+// The same slice through shared memory: a warp copies its contiguous 4 KB of a
+// slot array (or of S2) to its own staging buffer, one step before it is
+// needed, so that the L2 latency passes during the transform between. Each
+// warp waits for its own copies only.
+constexpr int kStage = 512;  // float2 per warp
+__device__ __forceinline__ void stage_slot(float2* st, const float2* a) {
+  const int lane = threadIdx.x & 31;
+  const float2* src = a + (threadIdx.x >> 5) * 512 + 2 * lane;
+  const unsigned dst = (unsigned)__cvta_generic_to_shared(st + 2 * lane);
+  __syncwarp();  // the warp's reads of the previous slice are done
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 512 * k), "l"(src + 64 * k)
+                 : "memory");
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void staged_ready() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncwarp();
 }
 
-// The column passes are split between the warps: warp w owns the column
-// slots w + 16 c (c < 4). Slot 0 carries two columns: the bins 0 and 64 of
-// a row's half spectrum are real (those of a real row), so columns 0 and 64
-// travel as one complex column, c0 + i c64, and one FFT serves both (the
-// two spectra are separated by Hermitian symmetry, C(k) = A(k) + i B(k)
-// with conj(C(-k)) = A(k) - i B(k)); every warp runs four column FFTs. A PSF
-// spectrum is stored column by column (column m: 128 rows, contiguous), so
-// a warp loads the values of its columns coalesced into registers:
-// kr[c][q] = spectrum(row 32 q + lane, column w + 16 c), c < 4, and on warp
-// 0 kr[4] = column 64.
-constexpr int kWarps = kFThreads / 32;
-constexpr int kColsPerWarp = (kFBins + kWarps - 1) / kWarps;  // 5
-using SpecRegs = float2[kColsPerWarp][4];
-
-// The spectra A (column 0) and B (column 64) from C = FFT(c0 + i c64) in
-// the layout of warp_fft_dif (lane l, slot q: frequency 32 q + rev5(l)).
-// The frequency -k of k = 32 q + s sits in slot 3 - q of the lane holding
-// 32 - s (s > 0), or in slot (4 - q) mod 4 of lane 0 (s = 0).
-__device__ __forceinline__ void split_dc_nyquist(const float2 (&v)[4], float2 (&a)[4],
-                                                 float2 (&b)[4], int lane) {
-  const int src = rev5((32 - rev5(lane)) & 31);
-  float2 p[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    p[q].x = __shfl_sync(0xffffffffu, v[3 - q].x, src);
-    p[q].y = __shfl_sync(0xffffffffu, v[3 - q].y, src);
-  }
-  if (lane == 0) {  // the shuffle brought v[3 - q]; the partner is v[(4 - q) mod 4]
-    p[0] = v[0];
-    p[1] = v[3];
-    p[2] = v[2];
-    p[3] = v[1];
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    a[q] = make_float2(0.5f * (v[q].x + p[q].x), 0.5f * (v[q].y - p[q].y));
-    const float2 d = make_float2(v[q].x - p[q].x, v[q].y + p[q].y);  // C(k) - conj(C(-k))
-    b[q] = make_float2(0.5f * d.y, -0.5f * d.x);
+// L2 prefetch by the whole CTA, one 128-byte line per lane: `rows` rows of
+// `bytes` bytes, `pitch` bytes apart (a tile's data of the next pair, which
+// DRAM would else deliver late). Bulk prefetches, one per row from one warp,
+// held that warp up for longer than they saved.
+__device__ __forceinline__ void prefetch_rows(const void* base, long long pitch, int rows,
+                                              int bytes) {
+  const int lines = (bytes + 254) >> 7;  // whatever the row's offset in its first line
+  for (int e = threadIdx.x; e < rows * lines; e += kFThreads) {
+    const int r = e / lines, l = e - r * lines;
+    const char* p = static_cast<const char*>(base) + r * pitch + min(128 * l, bytes - 1);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
   }
 }
 
-// c0 + i c64 for complex c0, c64
-__device__ __forceinline__ float2 pack_dc_nyquist(float2 c0, float2 c64) {
-  return make_float2(c0.x - c64.y, c0.y + c64.x);
+// the 128 x 128 region with origin (r0, c0) of a padded plane of `size`-byte elements
+__device__ __forceinline__ void prefetch_region(const void* plane, int size, const Geom& g, int r0,
+                                                int c0) {
+  const int ra = max(r0, 0), rb = min(r0 + kFT, g.H), ca = max(c0, 0), cb = min(c0 + kFT, g.W);
+  prefetch_rows(static_cast<const char*>(plane) + ((long long)(g.B + ra) * g.P + g.B + ca) * size,
+                (long long)size * g.P, rb - ra, size * (cb - ca));
 }
 
-// Visits (p, q) of a B x B output region, warp w taking the rows w, w + 16,
-// ... and its lanes the columns lane, lane + 32, ... (row addresses are
-// computed once per row; no division by B per element).
-template <class F>
-__device__ __forceinline__ void for_region(int B, F&& f) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int p = warp; p < B; p += kWarps)
-    for (int q = lane; q < B; q += 32) f(p, q);
-}
+// The second column of a slot: 128 - m (through the conjugate), or 64 for slot 0.
+__device__ __forceinline__ int second_col(int m) { return m ? kFT - m : 64; }
 
-__device__ __forceinline__ void load_spec_cols(SpecRegs& kr, const float2* kt) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int c = 0; c < kColsPerWarp; ++c) {
-    const int m = warp + kWarps * c;
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      kr[c][q] = m < kFBins ? kt[m * kFT + 32 * q + lane] : make_float2(0.f, 0.f);
-  }
-}
-
-// forward 2D transform, rows: 64 packed row FFTs and the split, two rows per
-// warp at a time (each warp owns row pairs warp + 16 i)
-__device__ void r2c_rows(float2* buf, const TwTab& T) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int k = warp; k < 64; k += 2 * kWarps) {
-    float2* r[2] = {buf + 2 * k * kFP, buf + 2 * (k + kWarps) * kFP};
-    float2 v[2][4];
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) v[j][q] = r[j][32 * q + lane];
-    warp_fft_dif<2>(v, T, lane);
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) r[j][rsw(32 * q + lane)] = v[j][q];
-    __syncwarp();
-    split_pair(r[0], lane);
-    split_pair(r[1], lane);
-  }
-  __syncthreads();
-}
-
-// J column FFTs (columns m[0..J)) of buf in place; with DN, m[0] = 0 is
-// the slot of columns 0 and 64 (forward: their real values in, their two
-// spectra out; inverse: their Hermitian spectra in, real values out)
-template <int J, bool INVERSE, bool DN>
-__device__ __forceinline__ void columns_inplace(float2* buf, const int (&m)[J], const TwTab& T,
-                                                int lane) {
-  float2 v[J][4];
-#pragma unroll
-  for (int j = 0; j < J; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float2* row = buf + (32 * q + lane) * kFP;
-      if (DN && j == 0)
-        v[j][q] = INVERSE ? pack_dc_nyquist(row[0], row[64]) : make_float2(row[0].x, row[64].x);
-      else
-        v[j][q] = row[m[j]];
-    }
-  if (INVERSE)
-    warp_ifft_dit<J>(v, T, lane);
-  else
-    warp_fft_dif<J>(v, T, lane);
-  if (DN && !INVERSE) {
-    float2 a[4], b[4];
-    split_dc_nyquist(v[0], a, b, lane);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      v[0][q] = a[q];
-      buf[(32 * q + lane) * kFP + 64] = b[q];
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < J; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float2* row = buf + (32 * q + lane) * kFP;
-      if (DN && INVERSE && j == 0) {
-        row[0] = make_float2(v[0][q].x, 0.f);
-        row[64] = make_float2(v[0][q].y, 0.f);
-      } else {
-        row[m[j]] = v[j][q];
-      }
-    }
-}
-
-// the 65 column FFTs as 64 slots: warp w owns the slots w + 16 c (c < 4),
-// two at a time; slot 0 (warp 0) holds columns 0 and 64
-template <bool INVERSE>
-__device__ __forceinline__ void all_columns(float2* buf, const TwTab& T) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// Row transforms of the 128 x 128 region whose rows load(r, t, v) gives
+// (v[i] = element t + 8 i of row r); ends at a CTA barrier
+template <class Load>
+__device__ __forceinline__ void rows_forward(float2* buf, const float4* tw, const Lane& L,
+                                             Load&& load) {
 #pragma unroll 1
-  for (int c = 0; c < 4; c += 2) {
-    const int m[2] = {warp + kWarps * c, warp + kWarps * (c + 1)};
-    if (warp == 0 && c == 0)
-      columns_inplace<2, INVERSE, true>(buf, m, T, lane);
-    else
-      columns_inplace<2, INVERSE, false>(buf, m, T, lane);
-  }
-}
-
-// forward real 2D transform in place (see the file comment)
-__device__ void r2c_2d(float2* buf, const TwTab& T) {
-  r2c_rows(buf, T);
-  all_columns<false>(buf, T);
-  __syncthreads();
-}
-
-// column slots c0, c0 + 1 of this warp (m = warp + 16 c): acc += FFT(buf)
-// conj(k^); with DN, slot 0 (columns 0 and 64)
-template <bool DN>
-__device__ __forceinline__ void columns_accumulate(const float2* buf, float2* acc,
-                                                   const SpecRegs& kr, int c0, const TwTab& T,
-                                                   int warp, int lane) {
-  float2 v[2][4];
-#pragma unroll
-  for (int j = 0; j < 2; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float2* row = buf + (32 * q + lane) * kFP;
-      v[j][q] = DN && j == 0 ? make_float2(row[0].x, row[64].x) : row[warp + kWarps * (c0 + j)];
-    }
-  warp_fft_dif<2>(v, T, lane);
-  if (DN) {
-    float2 a[4], b[4];
-    split_dc_nyquist(v[0], a, b, lane);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      v[0][q] = a[q];
-      float2* o = acc + (32 * q + lane) * kFP + 64;
-      *o = cadd(*o, cmulc(b[q], kr[4][q]));
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 2; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float2* o = acc + (32 * q + lane) * kFP + warp + kWarps * (c0 + j);
-      *o = cadd(*o, cmulc(v[j][q], kr[c0 + j][q]));
-    }
-}
-
-// forward transform of buf (destroyed) added, times conj(spectrum), into acc:
-// acc += FFT(buf) conj(k^), the column FFTs never written back
-// (no closing barrier: the caller's next barrier orders it)
-__device__ void r2c_2d_accumulate(float2* buf, float2* acc, const SpecRegs& kr, const TwTab& T) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  r2c_rows(buf, T);
-  if (warp == 0)
-    columns_accumulate<true>(buf, acc, kr, 0, T, warp, lane);
-  else
-    columns_accumulate<false>(buf, acc, kr, 0, T, warp, lane);
-  columns_accumulate<false>(buf, acc, kr, 2, T, warp, lane);
-}
-
-// merge, inverse row FFTs of the J row pairs k[0..J)
-template <int J>
-__device__ __forceinline__ void rows_inverse(float2* buf, const int (&k)[J], const TwTab& T,
-                                             int lane) {
-  float2 v[J][4];
-#pragma unroll
-  for (int j = 0; j < J; ++j) {
-    float2* r = buf + 2 * k[j] * kFP;
-    merge_pair(r, lane);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v[j][q] = r[rsw(32 * q + lane)];
-  }
-  warp_ifft_dit<J>(v, T, lane);
-#pragma unroll
-  for (int j = 0; j < J; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) buf[2 * k[j] * kFP + 32 * q + lane] = v[j][q];
-}
-
-// inverse transform, rows: merge and the packed row inverse FFTs of the row
-// pairs [k0, k1) (the rows a caller reads; the others are left undone), up
-// to three at a time per warp (43 pairs: one pass); sync = false leaves the
-// closing barrier to the caller
-__device__ void c2r_rows(float2* buf, const TwTab& T, int k0 = 0, int k1 = 64, bool sync = true) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int k = k0 + warp; k < k1; k += 3 * kWarps) {
-    if (k + 2 * kWarps < k1) {
-      const int kk[3] = {k, k + kWarps, k + 2 * kWarps};
-      rows_inverse<3>(buf, kk, T, lane);
-    } else if (k + kWarps < k1) {
-      const int kk[2] = {k, k + kWarps};
-      rows_inverse<2>(buf, kk, T, lane);
-    } else {
-      const int kk[1] = {k};
-      rows_inverse<1>(buf, kk, T, lane);
-    }
-  }
-  if (sync) __syncthreads();
-}
-
-// merge and inverse row FFTs of the J row pairs k[0..J), the results handed
-// to f(k, column, value) (value: real part row 2k, imaginary part row
-// 2k + 1; unscaled) instead of stored
-template <int J, class F>
-__device__ __forceinline__ void rows_inverse_apply(float2* buf, const int (&k)[J], const TwTab& T,
-                                                   int lane, F& f) {
-  float2 v[J][4];
-#pragma unroll
-  for (int j = 0; j < J; ++j) {
-    float2* r = buf + 2 * k[j] * kFP;
-    merge_pair(r, lane);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v[j][q] = r[rsw(32 * q + lane)];
-  }
-  warp_ifft_dit<J>(v, T, lane);
-#pragma unroll
-  for (int j = 0; j < J; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) f(k[j], 32 * q + lane, v[j][q]);
-}
-
-// c2r_rows with the results handed to f (see rows_inverse_apply); no
-// closing barrier
-template <class F>
-__device__ void c2r_rows_apply(float2* buf, const TwTab& T, int k0, int k1, F& f) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int k = k0 + warp; k < k1; k += 3 * kWarps) {
-    if (k + 2 * kWarps < k1) {
-      const int kk[3] = {k, k + kWarps, k + 2 * kWarps};
-      rows_inverse_apply<3>(buf, kk, T, lane, f);
-    } else if (k + kWarps < k1) {
-      const int kk[2] = {k, k + kWarps};
-      rows_inverse_apply<2>(buf, kk, T, lane, f);
-    } else {
-      const int kk[1] = {k};
-      rows_inverse_apply<1>(buf, kk, T, lane, f);
-    }
-  }
-}
-
-// inverse real 2D transform in place (unscaled); rows of the pairs [k0, k1)
-__device__ void c2r_2d(float2* buf, const TwTab& T, int k0 = 0, int k1 = 64) {
-  all_columns<true>(buf, T);
-  __syncthreads();
-  c2r_rows(buf, T, k0, k1);
-}
-
-// column slots c0, c0 + 1 of this warp: dst = IFFT(src . k^) along the
-// column; with DN, slot 0 (columns 0 and 64, real after the transform)
-template <bool DN>
-__device__ __forceinline__ void columns_product(const float2* src, float2* dst,
-                                                const SpecRegs& kr, int c0, const TwTab& T,
-                                                int warp, int lane) {
-  float2 v[2][4];
-#pragma unroll
-  for (int j = 0; j < 2; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float2* row = src + (32 * q + lane) * kFP;
-      v[j][q] = DN && j == 0
-                    ? pack_dc_nyquist(cmul(row[0], kr[0][q]), cmul(row[64], kr[4][q]))
-                    : cmul(row[warp + kWarps * (c0 + j)], kr[c0 + j][q]);
-    }
-  warp_ifft_dit<2>(v, T, lane);
-#pragma unroll
-  for (int j = 0; j < 2; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float2* row = dst + (32 * q + lane) * kFP;
-      if (DN && j == 0) {
-        row[0] = make_float2(v[0][q].x, 0.f);
-        row[64] = make_float2(v[0][q].y, 0.f);
-      } else {
-        row[warp + kWarps * (c0 + j)] = v[j][q];
-      }
-    }
-}
-
-// the column pass of dst = C2R(src . k^): dst's columns = IFFT(src . k^)
-// along the column; src is left intact; no closing barrier (the rows,
-// c2r_rows_apply, follow the caller's barrier)
-__device__ void columns_product_pass(const float2* src, float2* dst, const SpecRegs& kr,
-                                     const TwTab& T) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp == 0)
-    columns_product<true>(src, dst, kr, 0, T, warp, lane);
-  else
-    columns_product<false>(src, dst, kr, 0, T, warp, lane);
-  columns_product<false>(src, dst, kr, 2, T, warp, lane);
-}
-
-// values of the tile pixels (P, Q) and (P, Q + 1) after c2r_2d (unscaled),
-// Q even: one 16-byte load of the two packed row pairs' entries
-__device__ __forceinline__ float2 tile_pair_at(const float2* buf, int P, int Q) {
-  const float4 v = *reinterpret_cast<const float4*>(buf + (P >> 1) * 2 * kFP + Q);
-  return (P & 1) ? make_float2(v.y, v.w) : make_float2(v.x, v.z);
-}
-
-// Visits (p, q) of a B x B output region by column pairs, q = 0, 2, ..., warp
-// w taking the rows w, w + 16, ... and its lanes the pairs lane, lane + 32,
-// ... (B is even)
-template <class F>
-__device__ __forceinline__ void for_region_pairs(int B, F&& f) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int p = warp; p < B; p += kWarps)
-    for (int c = lane; c < B / 2; c += 32) f(p, 2 * c);
-}
-
-// value of tile pixel (P, Q) after c2r_2d (unscaled)
-__device__ __forceinline__ float tile_at(const float2* buf, int P, int Q) {
-  const float2 v = buf[(P >> 1) * 2 * kFP + Q];
-  return (P & 1) ? v.y : v.x;
-}
-
-// asynchronous 4-byte global -> shared copies (no register staging)
-__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(src) : "memory");
-}
-// asynchronous 8-byte global -> shared copy (both addresses 8-byte aligned)
-__device__ __forceinline__ void cp_async8(float* dst, const float* src) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// start copying the 128 x 128 region with origin (r0, c0) of a padded plane
-// into stg (row-major, zero outside the H x W image)
-__device__ void region_async(float* stg, const float* plane, const Geom& g, int r0, int c0) {
-  // warp w copies the rows w, w + 16, ...; a row's address is formed once
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int P = warp; P < kFT; P += kFThreads / 32) {
-    const int i = r0 + P;
-    const bool row_in = i >= 0 && i < g.H;
-    const float* src = plane + (long long)(g.B + i) * g.P + g.B + c0;
-    float* dst = stg + P * kFT;
-#pragma unroll
-    for (int c = 0; c < kFT / 32; ++c) {
-      const int Q = lane + 32 * c, j = c0 + Q;
-      if (row_in && j >= 0 && j < g.W)
-        cp_async4(dst + Q, src + Q);
-      else
-        dst[Q] = 0.f;
-    }
-  }
-  cp_async_commit();
-}
-
-// start copying the 128 x 128 region with origin (r0, c0) of a padded plane
-// straight into the packed row-pair layout of buf (rows 2k and 2k + 1 as the
-// real and imaginary parts of buf[2k kFP + j]; zero outside the image);
-// complete after cp_async_wait_all and a CTA barrier
-__device__ void region_async_packed(float2* buf, const float* plane, const Geom& g, int r0,
-                                    int c0) {
-  // warp w copies the row pairs w, w + 16, ...; lane 2 c + e takes row
-  // 2k + e, column c (+ 16 per step), so a warp writes 32 consecutive words
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* bf = reinterpret_cast<float*>(buf);
-  for (int k = warp; k < kFT / 2; k += kWarps) {
-    const int P = 2 * k + (lane & 1), i = r0 + P;
-    const bool row_in = i >= 0 && i < g.H;
-    const float* src = plane + (long long)(g.B + i) * g.P + g.B + c0;
-    float* dst = bf + 2 * (2 * k * kFP) + (lane & 1);
-#pragma unroll 8
-    for (int c = 0; c < kFT / 16; ++c) {
-      const int Q = (lane >> 1) + 16 * c, j = c0 + Q;
-      if (row_in && j >= 0 && j < g.W)
-        cp_async4(dst + 2 * Q, src + Q);
-      else
-        dst[2 * Q] = 0.f;
-    }
-  }
-  cp_async_commit();
-}
-
-// wait for the copies, then pack row pairs of stg into buf
-__device__ void pack_region(float2* buf, const float* stg) {
-  cp_async_wait_all();
-  __syncthreads();
-  for (int e = threadIdx.x; e < 64 * kFT; e += blockDim.x) {
-    const int k = e >> 7, j = e & (kFT - 1);
-    buf[2 * k * kFP + j] = make_float2(stg[2 * k * kFT + j], stg[(2 * k + 1) * kFT + j]);
+  for (int round = 0; round < 2; ++round) {
+    const int r = L.row((L.warp >> 3) + 2 * round);
+    float2 v[16];
+    load(r, v);
+    fft_row(v, buf + r * kFP, tw, L.t);
+    store_freqs(buf + r * kFP, v, L.t);
   }
   __syncthreads();
 }
 
-// one block per (exposure, phase): the Kc x Kc phase kernel (row pitch KP;
-// for r = 1 the PSF itself) at the top-left of a zero 128 x 128 tile
+// ---------------------------------------------------------------------------
+// spectra of the kernels
+// ---------------------------------------------------------------------------
+
+// One CTA per (pair, phase): S1 and S2 of k_a + i k_b; single = true: per
+// (exposure, phase) the slots and column 64 of k_t alone. The Kc x Kc phase
+// kernels (row pitch KP; for r = 1 the PSFs) at the top-left of a zero tile.
 __global__ void __launch_bounds__(kFThreads, 1)
-    fft_spectra_kernel(const float* __restrict__ ka, int Kc, int KP, float2* __restrict__ spec) {
-  extern __shared__ float2 fsm[];
-  __shared__ TwTab T;
-  float2* buf = fsm;
-  init_twiddles(T);
-  const float* ft = ka + (long long)blockIdx.x * Kc * KP;
-  for (int e = threadIdx.x; e < 64 * kFT; e += blockDim.x) {
-    const int k = e >> 7, j = e & (kFT - 1);
-    const int i = 2 * k;
-    const float a = (i < Kc && j < Kc) ? ft[i * KP + j] : 0.f;
-    const float b = (i + 1 < Kc && j < Kc) ? ft[(i + 1) * KP + j] : 0.f;
-    buf[2 * k * kFP + j] = make_float2(a, b);
-  }
-  __syncthreads();
-  r2c_2d(buf, T);
-  // column by column: out[m][row]
-  float2* out = spec + (long long)blockIdx.x * kFT * kFBins;
-  for (int e = threadIdx.x; e < kFT * kFBins; e += blockDim.x) {
-    const int m = e >> 7, rr = e & (kFT - 1);
-    out[e] = buf[rr * kFP + m];
-  }
-}
-
-// column slot m of phase_sum_columns (DN: slot 0, columns 0 and 64)
-template <bool DN>
-__device__ __forceinline__ void phase_sum_column(const float2* xs, const float2* kt, int R2,
-                                                 float2* dst, const TwTab& T, int m, int lane) {
-  const int per = kFT * kFBins;
-  float2 v[1][4];
+    fft_spectra_kernel(const float* __restrict__ ka, int n, int R2, int Kc, int KP, bool single,
+                       float2* __restrict__ out) {
+  extern __shared__ __align__(16) float2 fsm[];
+  __shared__ float4 tw[kFT / 2];
+  init_twiddles(tw);
+  const Lane L;
+  const int q = blockIdx.x / R2, phi = blockIdx.x - q * R2;
+  const int ta = single ? q : 2 * q, tb = ta + 1;
+  const float* fa = ka + ((long long)ta * R2 + phi) * Kc * KP;
+  const float* fb = !single && tb < n ? ka + ((long long)tb * R2 + phi) * Kc * KP : nullptr;
+  rows_forward(fsm, tw, L, [&](int r, float2 (&v)[16]) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) v[0][q] = make_float2(0.f, 0.f);
-  for (int ph = 0; ph < R2; ++ph) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int o = ph * per + m * kFT + 32 * q + lane;
-      if (DN) {
-        const int o64 = o + 64 * kFT;
-        v[0][q] = cadd(v[0][q], pack_dc_nyquist(cmul(xs[o], kt[o]), cmul(xs[o64], kt[o64])));
-      } else {
-        v[0][q] = cadd(v[0][q], cmul(xs[o], kt[o]));
-      }
-    }
-  }
-  warp_ifft_dit<1>(v, T, lane);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    float2* row = dst + (32 * q + lane) * kFP;
-    if (DN) {
-      row[0] = make_float2(v[0][q].x, 0.f);
-      row[64] = make_float2(v[0][q].y, 0.f);
-    } else {
-      row[m] = v[0][q];
-    }
-  }
-}
-
-// r > 1: the column pass of dst = C2R(sum_phi x^_phi . k^_phi) with both
-// spectra read from global memory (x^ from this tile's scratch,
-// L2-resident), column by column; no closing barrier (the rows,
-// c2r_rows_apply, follow the caller's barrier)
-__device__ void phase_sum_columns(const float2* xs, const float2* kt, int R2, float2* dst,
-                                  const TwTab& T) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int m = warp; m < 64; m += kWarps) {  // column slots; slot 0: columns 0 and 64
-    if (m == 0)
-      phase_sum_column<true>(xs, kt, R2, dst, T, m, lane);
-    else
-      phase_sum_column<false>(xs, kt, R2, dst, T, m, lane);
-  }
-}
-
-// the forward pass of one tile (tile index `tile` = ty gx + tx of its job)
-// for the exposures [t_begin, t_end); starts and ends at a CTA barrier, so
-// a persistent CTA can run many. STUDENT = false compiles the Gaussian
-// weights only (the split launch, which never runs the heavy-tailed model).
-template <bool STUDENT = true>
-__device__ void fft_forward_tile(const Shape& s, const FftLaunch& a, int ty, int tx, int tile,
-                                 float2* fsm, const TwTab& T, int t_begin, int t_end) {
-  float2* xh = fsm;
-  float2* wk = fsm + kFBuf;
-  float* stg = reinterpret_cast<float*>(fsm + 2 * kFBuf);  // 128 x 128 floats
-  const Geom& g = s.g;
-  const int hc = s.hc, B = kFT - 2 * hc, R2 = s.R2;
-  const int i0 = ty * B, j0 = tx * B;
-  const int per = kFT * kFBins;
-  // this tile's scratch block (sized for the adjoint's accumulators)
-  float2* xs = a.scratch + (long long)tile * (a.nu > 0.f ? 2 * R2 : R2) * per;
-  SpecRegs kr;
-  if (R2 == 1) {
-    load_spec_cols(kr, a.spec + (long long)t_begin * per);
-    region_async(stg, a.x, g, i0 - hc, j0 - hc);
-    pack_region(xh, stg);
-    r2c_2d(xh, T);
-  } else {
-    // the phases' spectra, column by column, into this tile's scratch
-    for (int ph = 0; ph < R2; ++ph) {
-      region_async(stg, a.x + (long long)ph * g.plane, g, i0 - hc, j0 - hc);
-      pack_region(xh, stg);
-      r2c_2d(xh, T);
-      for (int e = threadIdx.x; e < per; e += blockDim.x) {
-        const int m = e >> 7, rr = e & (kFT - 1);
-        xs[ph * per + e] = xh[rr * kFP + m];
-      }
-      __syncthreads();
-    }
-  }
-  for (int t = t_begin; t < t_end; ++t) {
-    // u of this exposure (B x B, row-major in stg) arrives during the
-    // inverse transform, by column pairs: the border (2 hc), the pitch (a
-    // multiple of 8) and the tile origins (multiples of B) are even, so a
-    // pair is 8-byte aligned; the last pair of an edge tile may read column
-    // W, inside the padded row (pitch > border + W) and never used
-    const long long tplane = (long long)t * g.plane;
-    {
-      const float* ut = a.u + tplane + (long long)(g.B + i0) * g.P + g.B + j0;
-      const int pmax = min(B, g.H - i0), qmax = min(B, g.W - j0);
-      for_region_pairs(B, [&](int p, int q) {
-        if (p < pmax && q < qmax) cp_async8(stg + p * B + q, ut + (long long)p * g.P + q);
-      });
-    }
-    cp_async_commit();
-    if (R2 == 1)
-      columns_product_pass(xh, wk, kr, T);
-    else
-      phase_sum_columns(xs, a.spec + (long long)t * R2 * per, R2, wk, T);
-    const int pmax = min(B, g.H - i0), qmax = min(B, g.W - j0);
-    const long long base = tplane + (long long)(g.B + i0) * g.P + g.B + j0;
-    if (STUDENT && a.nu > 0.f) {
-      // heavy-tailed weights u' = u (nu+1) / (nu + u (y - z)^2): both u' z
-      // (denominator) and u' y (numerator) go to planes. The rows are stored
-      // (pairs [hc, 64): z at rows [2 hc, 128)) and the weights computed
-      // after a barrier, by column pairs (the y loads of a fused form stall
-      // the row pass)
-      __syncthreads();
-      c2r_rows(wk, T, hc, 64, false);
-      // the next spectrum loads during the epilogue and the next column pass
-      if (R2 == 1 && t + 1 < t_end) load_spec_cols(kr, a.spec + (long long)(t + 1) * per);
-      cp_async_wait_all();
-      __syncthreads();
-      const float nu1 = a.nu + 1.f;
-      for_region_pairs(B, [&](int p, int q) {
-        if (p < pmax && q < qmax) {
-          const long long gi = base + (long long)p * g.P + q;
-          const bool two = q + 1 < qmax;
-          const float2 zz = tile_pair_at(wk, p + 2 * hc, q + 2 * hc);
-          const float2 uu = *reinterpret_cast<const float2*>(stg + p * B + q);
-          const float2 yy = two ? *reinterpret_cast<const float2*>(a.y + gi)
-                                : make_float2(a.y[gi], 0.f);
-          float wv[2], w2v[2];
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float z = (e ? zz.y : zz.x) * kFScale, uv = e ? uu.y : uu.x;
-            const float yv = e ? yy.y : yy.x, d = yv - z;
-            const float us = uv > 0.f ? uv * nu1 / fmaf(uv * d, d, a.nu) : 0.f;
-            wv[e] = us * z;
-            w2v[e] = us * yv;
-          }
-          if (two) {
-            *reinterpret_cast<float2*>(a.w + gi) = make_float2(wv[0], wv[1]);
-            *reinterpret_cast<float2*>(a.w2 + gi) = make_float2(w2v[0], w2v[1]);
-          } else {
-            a.w[gi] = wv[0];
-            a.w2[gi] = w2v[0];
-          }
-        }
-      });
-    } else {
-      // this warp's columns are done: the next spectrum loads during the rows
-      if (R2 == 1 && t + 1 < t_end) load_spec_cols(kr, a.spec + (long long)(t + 1) * per);
-      cp_async_wait_all();
-      __syncthreads();  // every column done, u landed
-      // the inverse rows of the pairs [hc, 64) (z at rows [2 hc, 128)) go
-      // straight from registers to the w plane: z(p, q) is row 2k + e - 2 hc,
-      // column c - 2 hc of the value (k, c) (e = 0 real part, 1 imaginary)
-      float* wt = a.w + base;
-      auto out = [&](int k, int c, float2 v) {
-        const int q = c - 2 * hc;
-        if (q < 0 || q >= qmax) return;
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int p = 2 * k + e - 2 * hc;
-          if (p < pmax) wt[(long long)p * g.P + q] = stg[p * B + q] * ((e ? v.y : v.x) * kFScale);
-        }
-      };
-      c2r_rows_apply(wk, T, hc, 64, out);
-    }
-    __syncthreads();  // wk and stg are free for the next exposure
-  }
-}
-
-__global__ void __launch_bounds__(kFThreads, 1)
-    fft_forward_kernel(const Shape s, const FftLaunch a) {
-  extern __shared__ float2 fsm[];
-  __shared__ TwTab T;
-  init_twiddles(T);
-  fft_forward_tile(s, a, blockIdx.y, blockIdx.x, blockIdx.y * gridDim.x + blockIdx.x, fsm, T, 0,
-                   s.n);
-}
-
-// column slot m of r2c_2d_accumulate_phases (DN: slot 0, columns 0 and 64)
-template <bool DN>
-__device__ __forceinline__ void accumulate_phases_column(const float2* buf, float2* acc,
-                                                         const float2* kt, int R2,
-                                                         const TwTab& T, int m, int lane) {
-  const int per = kFT * kFBins;
-  float2 v[1][4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const float2* row = buf + (32 * q + lane) * kFP;
-    v[0][q] = DN ? make_float2(row[0].x, row[64].x) : row[m];
-  }
-  warp_fft_dif<1>(v, T, lane);
-  if (DN) {
-    float2 a[4], b[4];
-    split_dc_nyquist(v[0], a, b, lane);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v[0][q] = a[q];
-    for (int ph = 0; ph < R2; ++ph) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int o = ph * per + 64 * kFT + 32 * q + lane;
-        acc[o] = cadd(acc[o], cmulc(b[q], kt[o]));
-      }
-    }
-  }
-  for (int ph = 0; ph < R2; ++ph) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int o = ph * per + m * kFT + 32 * q + lane;
-      acc[o] = cadd(acc[o], cmulc(v[0][q], kt[o]));
-    }
-  }
-}
-
-// r > 1: acc_phi += FFT(buf) conj(k^_phi) for every phase, accumulators in
-// this tile's scratch (column by column, each element one lane's)
-__device__ void r2c_2d_accumulate_phases(float2* buf, float2* acc, const float2* kt, int R2,
-                                         const TwTab& T) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  r2c_rows(buf, T);
-  for (int m = warp; m < 64; m += kWarps) {  // column slots; slot 0: columns 0 and 64
-    if (m == 0)
-      accumulate_phases_column<true>(buf, acc, kt, R2, T, m, lane);
-    else
-      accumulate_phases_column<false>(buf, acc, kt, R2, T, m, lane);
-  }
-  __syncthreads();
-}
-
-// Den of one phase (in sh after the inverse transform) -> the update; the
-// numerator is a.N, or (Student-t) the transformed tile num
-__device__ void update_phase(const float2* sh, const float2* num, const FftLaunch& a,
-                             const Geom& g, long long off, int i0, int j0, int B) {
-  const long long base = off + (long long)(g.B + i0) * g.P + g.B + j0;
-  const int pmax = min(B, g.H - i0), qmax = min(B, g.W - j0);
-  for_region(B, [&](int p, int q) {
-    if (p < pmax && q < qmax) {
-      const long long gi = base + (long long)p * g.P + q;
-      const float d = tile_at(sh, p, q) * kFScale;
-      const float xo = a.x[gi], nraw = a.N[gi];
-      const float nt = num ? tile_at(num, p, q) * kFScale : nraw;
-      float xv = xo;
-      // The transform leaves a rounding floor (~1e-7 of the tile's weighted
-      // model) where the exact denominator is 0; N, from the direct kernel,
-      // is exactly 0 when no valid pixel lies in the footprint, which is
-      // then the sign of a zero denominator (x unchanged, as for Den = 0);
-      // with Student-t weights too, since u' = 0 exactly where u = 0.
-      if (d > 0.f && nraw != 0.f) {
-        const float nv = fmaxf(nt, 0.f);
-        if (d < 1e-30f)  // denominator near zero: guarded ratio in FP64
-          xv = (float)((double)xo * (double)nv / (double)d);
-        else
-          xv = xo * nv / d;
-      }
-      a.xn[gi] = xv;
+    for (int i = 0; i < 16; ++i) {
+      const int c = L.t + 8 * i;
+      const bool in = r < Kc && c < Kc;
+      v[i] = make_float2(in ? fa[r * KP + c] : 0.f, in && fb ? fb[r * KP + c] : 0.f);
     }
   });
+  const int m = L.slot();
+  out += (long long)blockIdx.x * (single ? kCol : kPairSpec);
+  float2 v[16];
+  load_col(fsm + m, v, L.t, false);
+  fft_col(v, fsm + m, tw, L.t);
+  store_slot(out, v);
+  const int m2 = second_col(m);
+  load_col(fsm + m2, v, L.t, m != 0);
+  fft_col(v, fsm + m2, tw, L.t);
+  if (!single) {
+    store_slot(out + kSlots, v);
+  } else if (m == 0) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) out[kSlots + 8 * i + L.t] = v[i];
+  }
 }
 
-// Equal ranges: CTA b of P takes the units [b U / P, (b+1) U / P) of U.
-__device__ __forceinline__ long long split_start(long long U, int P, int b) {
-  return (long long)b * U / P;
+// ---------------------------------------------------------------------------
+// forward model
+// ---------------------------------------------------------------------------
+
+// x^ of one phase: the slot of this thread into X, column 64 into x64 (128
+// entries); starts and ends at a CTA barrier
+__device__ __forceinline__ void region_spectrum(const float* plane, const Geom& g, int r0, int c0,
+                                                float2* buf, const float4* tw, const Lane& L,
+                                                float2 (&X)[16], float2* x64) {
+  rows_forward(buf, tw, L, [&](int r, float2 (&v)[16]) {
+    const int i = r0 + r;
+    const bool row_in = i >= 0 && i < g.H;
+    const float* src = plane + (long long)(g.B + i) * g.P + g.B;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int j = c0 + L.t + 8 * q;
+      v[q] = make_float2(row_in && j >= 0 && j < g.W ? __ldcg(src + j) : 0.f, 0.f);
+    }
+  });
+  // column 64 first (slot 0's group, and with it its warp, for the warp
+  // barriers), then the slots: one copy of the transform's code
+  const int m = L.slot();
+#pragma unroll 1
+  for (int h = L.warp == 0; h >= 0; --h) {
+    float2* col = buf + (h ? second_col(m) : m);
+    load_col(col, X, L.t, false);
+    fft_col(X, col, tw, L.t);
+    if (h && m == 0) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) x64[8 * i + L.t] = X[i];
+    }
+  }
+  __syncthreads();
 }
 
-__device__ __forceinline__ int ld_acquire_gpu(const int* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
+// The forward pass of one tile for the pairs of exposures [q0, q1). R1: r = 1
+// (x^ in registers; otherwise the phases' x^ in xs). Starts and ends at a CTA
+// barrier, so a persistent CTA can run many; (nty, ntx), if known, is the tile
+// it runs next, whose x region is brought into L2 meanwhile.
+template <bool R1, bool STUDENT>
+__device__ void fft_forward_tile(const Shape& s, const FftLaunch& a, int ty, int tx, float2* xs,
+                                 float2* buf, float2* x64, const float4* tw, int q0, int q1,
+                                 int nty = -1, int ntx = 0) {
+  const Geom& g = s.g;
+  const Lane L;
+  const int hc = s.hc, B = kFT - 2 * hc, R2 = s.R2;
+  const int i0 = ty * B, j0 = tx * B;
+  const int m = L.slot(), m2 = second_col(m);
+  const int pmax = min(B, g.H - i0), qmax = min(B, g.W - j0);
+  float2* st = buf + kFBuf + L.warp * kStage;
+  auto prefetch_pair = [&](int q) {  // u (and y) of the tile
+    for (int t = 2 * q; t < min(2 * q + 2, s.n); ++t) {
+      const long long off = (long long)t * g.plane + (long long)(g.B + i0) * g.P + g.B + j0;
+      prefetch_rows(a.u + off, 4LL * g.P, pmax, 4 * qmax);
+      if (STUDENT) prefetch_rows(a.y + off, 4LL * g.P, pmax, 4 * qmax);
+    }
+  };
+  prefetch_pair(q0);
+  if (R1) stage_slot(st, a.spec + (long long)q0 * kPairSpec);
+  float2 X[16];
+  if (R1) {
+    region_spectrum(a.x, g, i0 - hc, j0 - hc, buf, tw, L, X, x64);
+  } else {
+    for (int ph = 0; ph < R2; ++ph) {
+      region_spectrum(a.x + (long long)ph * g.plane, g, i0 - hc, j0 - hc, buf, tw, L, X,
+                      xs + (long long)ph * kCol + kSlots);
+      store_slot(xs + (long long)ph * kCol, X);
+    }
+  }
+  for (int q = q0; q < q1; ++q) {
+    const float2* S = a.spec + (long long)q * R2 * kPairSpec;
+    if (q + 1 < q1)
+      prefetch_pair(q + 1);
+    else if (nty >= 0)
+      prefetch_region(a.x, 4, g, nty * B - hc, ntx * B - hc);
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {  // column m, then its partner
+      float2 v[16];
+      if (R1) {
+        const float2* sp = st + (threadIdx.x & 31);
+        staged_ready();
+        if (h == 1 && m == 0) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = cmul(x64[8 * i + L.t], sp[32 * i]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = cmul(X[i], sp[32 * i]);
+        }
+        // S2 arrives during this column's transform, the next pair's S1 during
+        // the second column's and the rows
+        if (h == 0)
+          stage_slot(st, S + kSlots);
+        else if (q + 1 < q1)
+          stage_slot(st, S + kPairSpec);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = make_float2(0.f, 0.f);
+        const bool c64 = h == 1 && m == 0;
+        const int xstep = c64 ? 8 : 32;
+#pragma unroll 2
+        for (int ph = 0; ph < R2; ++ph) {
+          const float2* sp = S + (long long)ph * kPairSpec + h * kSlots + slot_off();
+          const float2* xp = xs + (long long)ph * kCol + (c64 ? kSlots + L.t : slot_off());
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = cfma(v[i], xp[xstep * i], __ldg(sp + 32 * i));
+        }
+      }
+      float2* col = buf + (h == 0 ? m : m2);
+      ifft_col(v, col, tw, L.t);
+      store_col(col, v, L.t, h == 1 && m != 0);
+    }
+    __syncthreads();
+    // rows [2 hc, 128): z_a + i z_b at columns [2 hc, 128)
+    const int ta = 2 * q, tb = min(ta + 1, s.n - 1);  // (an odd last exposure: z_b unused)
+    const bool two = ta + 1 < s.n;
+    const int c_lo = 2 * hc - L.t, c_hi = 2 * hc + qmax - L.t;  // columns t + 8 i: 8 i in [c_lo, c_hi)
+#pragma unroll 1
+    for (int blk = 3 - (L.warp >> 3); blk >= 0 && 32 * blk + 31 >= 2 * hc; blk -= 2) {
+      const int r = L.row(blk), p = r - 2 * hc;
+      const bool row_ok = p >= 0 && p < pmax;
+      const long long rowoff = (long long)(g.B + i0 + p) * g.P + g.B + j0 - 2 * hc + L.t;
+      const float* ua = a.u + (long long)ta * g.plane + rowoff;
+      const float* ub = a.u + (long long)tb * g.plane + rowoff;
+      float2 u[16];  // in flight during the transform
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const bool in = row_ok && 8 * i >= c_lo && 8 * i < c_hi;
+        u[i] = make_float2(in ? __ldg(ua + 8 * i) : 0.f, in && two ? __ldg(ub + 8 * i) : 0.f);
+      }
+      float2 v[16];
+      load_freqs(buf + r * kFP, v, L.t);
+      ifft_row(v, buf + r * kFP, tw, L.t);
+      if (!row_ok) continue;
+      if (!STUDENT) {
+        float2* w = a.w + (long long)q * g.plane + rowoff;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if (8 * i >= c_lo && 8 * i < c_hi)
+            w[8 * i] = make_float2(u[i].x * (v[i].x * kFScale), u[i].y * (v[i].y * kFScale));
+      } else {
+        // heavy-tailed weights u' = u (nu+1) / (nu + u (y - z)^2): (u' z, u' y) per
+        // exposure
+        const float nu1 = a.nu + 1.f;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          if (e && !two) break;
+          const float* yp = a.y + (long long)(e ? tb : ta) * g.plane + rowoff;
+          float2* w = a.w + (long long)(ta + e) * g.plane + rowoff;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            if (8 * i >= c_lo && 8 * i < c_hi) {
+              const float z = (e ? v[i].y : v[i].x) * kFScale, uv = e ? u[i].y : u[i].x;
+              const float yv = __ldg(yp + 8 * i);
+              const float d = yv - z;
+              const float us = uv > 0.f ? uv * nu1 / fmaf(uv * d, d, a.nu) : 0.f;
+              w[8 * i] = make_float2(us * z, us * yv);
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();  // the buffer is free for the next pair
+  }
 }
-__device__ __forceinline__ void st_release_gpu(int* p, int v) {
-  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+
+// ---------------------------------------------------------------------------
+// adjoint and update
+// ---------------------------------------------------------------------------
+
+// one pixel of Eq. (2)
+__device__ __forceinline__ float update_pixel(float xo, float d, float nraw, float nt) {
+  // The transform leaves a rounding floor (~1e-7 of the tile's weighted
+  // model) where the exact denominator is 0; N, from the direct kernel,
+  // is exactly 0 when no valid pixel lies in the footprint, which is
+  // then the sign of a zero denominator (x unchanged, as for Den = 0);
+  // with Student-t weights too, since u' = 0 exactly where u = 0.
+  float xv = xo;
+  if (d > 0.f && nraw != 0.f) {
+    const float nv = fmaxf(nt, 0.f);
+    if (d < 1e-30f)  // denominator near zero: guarded ratio in FP64
+      xv = (float)((double)xo * (double)nv / (double)d);
+    else
+      xv = xo * nv / d;
+  }
+  return xv;
 }
+
+// From the columns in the buffer (every column of every row): inverse row
+// transforms of the rows [0, B) and the update of one phase. STUDENT: real part
+// Den, imaginary part N'. Starts and ends at a CTA barrier.
+template <bool STUDENT>
+__device__ __forceinline__ void rows_update(const Shape& s, const FftLaunch& a, int phi, int i0,
+                                            int j0, float2* buf, const float4* tw, const Lane& L) {
+  const Geom& g = s.g;
+  const int B = kFT - 2 * s.hc;
+  const int pmax = min(B, g.H - i0), qmax = min(B, g.W - j0);
+#pragma unroll 1
+  for (int blk = L.warp >> 3; blk < 4 && 32 * blk < pmax; blk += 2) {
+    const int r = L.row(blk);
+    float2 v[16];
+    load_freqs(buf + r * kFP, v, L.t);
+    ifft_row(v, buf + r * kFP, tw, L.t);
+    if (r >= pmax) continue;
+    const long long off =
+        (long long)phi * g.plane + (long long)(g.B + i0 + r) * g.P + g.B + j0 + L.t;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (L.t + 8 * i < qmax) {
+        const long long gi = off + 8 * i;
+        const float nraw = a.N[gi];
+        a.xn[gi] = update_pixel(__ldcg(a.x + gi), v[i].x, nraw, STUDENT ? v[i].y : nraw);
+      }
+  }
+  __syncthreads();
+}
+
+// Gaussian: the Hermitian accumulator of this thread's slot (acc) and, for
+// slot 0, column 64 (a64, 128 entries) -> the buffer's columns. H counts m >= 1
+// twice (see the file comment); columns 0 and 64 keep the real part.
+__device__ __forceinline__ void columns_gauss(const float2 (&acc)[16], const float2* a64, float2* buf,
+                                              const float4* tw, const Lane& L) {
+  const int m = L.slot(), m2 = second_col(m);
+  const float sc = m ? 0.5f * kFScale : kFScale;
+  // column 64 first (slot 0's group, and with it its warp, for the warp
+  // barriers), then the slots: one copy of the transform's code
+#pragma unroll 1
+  for (int h = L.warp == 0; h >= 0; --h) {
+    float2 v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      v[i] = acc[i];
+      if (h) v[i] = m ? make_float2(0.f, 0.f) : a64[8 * i + L.t];
+    }
+    float2* col = buf + (h ? m2 : m);
+    ifft_col(v, col, tw, L.t);
+    if (h && m) continue;  // (only slot 0's second column is wanted)
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = make_float2(sc * v[i].x, m ? sc * v[i].y : 0.f);
+    store_col_group(col, v, L, false);
+    if (m) store_col_group(buf + m2, v, L, true);
+  }
+  __syncthreads();
+}
+
+// Student-t: the slot's two columns, m from f and 128 - m (64 for slot 0) from
+// the conjugate of g -> the buffer's columns
+__device__ __forceinline__ void columns_student(float2 (&f)[16], const float2 (&gv)[16], float2* buf,
+                                                const float4* tw, const Lane& L) {
+  const int m = L.slot(), m2 = second_col(m);
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    float2* col = buf + (h ? m2 : m);
+    if (h) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) f[i] = gv[i];
+    }
+    ifft_col(f, col, tw, L.t);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) f[i] = make_float2(kFScale * f[i].x, kFScale * f[i].y);
+    store_col(col, f, L.t, h && m != 0);
+  }
+  __syncthreads();
+}
+
+// A warp's four rows (L.row(blk)) of the w region with origin (r0, c0) of
+// plane `w` (float2 on the padded planes; zero outside the image), by
+// asynchronous copies to dst, row pitch kFP: 32 lanes copy 256 contiguous
+// bytes, where loads in the transform's own order (eight lanes a row) touch
+// four rows an instruction.
+__device__ __forceinline__ void copy_w(float2* dst, const float2* w, const Geom& g, int r0, int c0,
+                                       int blk, const Lane& L) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int r = L.row(blk, k), i = r0 + r;
+    const bool row_in = i >= 0 && i < g.H;
+    const float2* src = w + (long long)(g.B + (row_in ? i : 0)) * g.P + g.B;
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst + L.row(0, k) * kFP + lane);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = c0 + lane + 32 * q;
+      const bool in = row_in && j >= 0 && j < g.W;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d + 256 * q),
+                   "l"(src + (in ? j : 0)), "r"(in ? 8 : 0)
+                   : "memory");
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void copies_ready() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncwarp();
+}
+
+// Row transforms of a w region. The warp's rows of the blocks 0 and 1 are
+// in flight to or in its part of the staging buffer (copy_w a column phase
+// ago), or, stage null, in flight to their place in buf; those of the blocks
+// 2 and 3 come straight to their place during the first transforms. Ends at a
+// CTA barrier.
+__device__ __forceinline__ void w_rows(float2* stage, const float2* w, const Geom& g, int r0,
+                                       int c0, float2* buf, const float4* tw, const Lane& L) {
+  const int blk = L.warp >> 3;
+  copies_ready();
+  copy_w(buf + (blk + 2) * 32 * kFP, w, g, r0, c0, blk + 2, L);
+#pragma unroll 1
+  for (int round = 0; round < 2; ++round) {
+    const int r = L.row(blk + 2 * round);
+    const float2* src = (round || !stage ? buf : stage) + r * kFP;
+    if (round) copies_ready();
+    float2 v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = src[L.t + 8 * i];
+    fft_row(v, buf + r * kFP, tw, L.t);
+    store_freqs(buf + r * kFP, v, L.t);
+  }
+  __syncthreads();
+}
+
 constexpr unsigned kPartPolls = 1u << 23;  // x ~0.3 us per poll: seconds, not a hang
 
-// A tile cut into parts (consecutive exposure ranges) on different CTAs
-// of a split launch: part q > 0 waits (bounded) for the tile's flag to
-// reach q, starts from the accumulator part q - 1 left in its CTA's slot,
-// and, unless it is the last part, leaves its own in this CTA's slot and
-// raises the flag to q + 1; the last part finishes the tile and resets the
-// flag. The exposures are summed in the order a whole-tile CTA sums them
-// (the same bits). A wait that gives up sets the timeout bit of the error
-// word and starts from zero.
-__device__ void adjoint_publish_part(const FftLaunch& a, int tile, const float2* sh, int q) {
-  float2* slot = a.partials + (long long)blockIdx.x * kFBuf;
-  for (int e = threadIdx.x; e < kFBuf; e += blockDim.x) slot[e] = sh[e];
+// A tile cut into parts (consecutive pairs) on different CTAs of a split
+// launch: part i > 0 waits (bounded) for the tile's flag to reach i, starts
+// from the accumulator part i - 1 left in its CTA's slot, and, unless it is
+// the last part, leaves its own in this CTA's slot and raises the flag to
+// i + 1; the last part finishes the tile and resets the flag. The pairs are
+// summed in the order a whole-tile CTA sums them (the same bits). A wait that
+// gives up sets the timeout bit of the error word and starts from zero.
+__device__ void publish_part(const FftLaunch& a, int tile, const float2 (&acc)[16],
+                             const float2* a64, int part) {
+  float2* slot = a.partials + (long long)blockIdx.x * kCol;
+  store_slot(slot, acc);
+  for (int e = threadIdx.x; e < kFT; e += blockDim.x) slot[kSlots + e] = a64[e];
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) st_release_gpu(a.counters + tile, q + 1);
+  if (threadIdx.x == 0) st_release(a.counters + tile, part + 1);
 }
 
-__device__ void adjoint_resume_part(const FftLaunch& a, int tile, float2* sh, int q, int prev_cta,
-                                    bool last) {
+__device__ void resume_part(const FftLaunch& a, int tile, float2 (&acc)[16], float2* a64, int part,
+                            int prev_cta, bool last) {
   __shared__ int ok;
   if (threadIdx.x == 0) {
     unsigned i = 0;
-    while (i < kPartPolls && ld_acquire_gpu(a.counters + tile) < q) {
+    while (i < kPartPolls && ld_acquire(a.counters + tile) < part) {
       __nanosleep(200);
       ++i;
     }
@@ -1045,99 +808,345 @@ __device__ void adjoint_resume_part(const FftLaunch& a, int tile, float2* sh, in
       a.counters[tile] = 0;  // ready for the next launch
   }
   __syncthreads();
-  const float2* slot = a.partials + (long long)prev_cta * kFBuf;
-  for (int e = threadIdx.x; e < kFBuf; e += blockDim.x)
-    sh[e] = ok ? __ldcg(slot + e) : make_float2(0.f, 0.f);
-}
-
-// the adjoint pass and the update of one tile; starts and ends at a CTA
-// barrier. r = 1 Gaussian: one accumulator in shared memory. Otherwise the
-// accumulators live in the tile's scratch: R2 for Den, and for Student-t R2
-// more for N' (the w2 planes, transformed the same way). A split launch
-// (r = 1 Gaussian) runs part q of a cut tile: the sources [k_begin, k_end),
-// resumed from CTA prev_cta's part q - 1 (prev_cta < 0: from zero), then
-// the update if it is the last part, else published for part q + 1.
-__device__ void fft_adjoint_tile(const Shape& s, const FftLaunch& a, int ty, int tx, int tile,
-                                 float2* fsm, const TwTab& T, int k_begin = 0, int k_end = -1,
-                                 int q = 0, int prev_cta = -1, bool last = true) {
-  float2* sh = fsm;
-  float2* wk = fsm + kFBuf;
-  // the w regions arrive straight in the packed layout, alternating between
-  // two work buffers: one is transformed while the next region lands in the other
-  float2* wbuf[2] = {fsm + kFBuf, fsm + 2 * kFBuf};
-  const Geom& g = s.g;
-  const int hc = s.hc, B = kFT - 2 * hc, R2 = s.R2;
-  const int i0 = ty * B, j0 = tx * B;
-  const int per = kFT * kFBins;
-  const bool student = a.nu > 0.f;
-  const bool in_smem = R2 == 1 && !student;
-  const int nacc = student ? 2 * R2 : R2;
-  float2* acc = a.scratch + (long long)tile * nacc * per;
-  // sources in order: w_0 (, w2_0), w_1 (, w2_1), ...
-  const int nsrc = student ? 2 * s.n : s.n;
-  if (k_end < 0) k_end = nsrc;
-  auto src_plane = [&](int k) -> const float* {
-    return student ? ((k & 1) ? a.w2 : a.w) + (long long)(k >> 1) * g.plane
-                   : a.w + (long long)k * g.plane;
-  };
-  SpecRegs kr;
-  if (in_smem) {
-    if (prev_cta >= 0)
-      adjoint_resume_part(a, tile, sh, q, prev_cta, last);
-    else
-      for (int e = threadIdx.x; e < kFBuf; e += blockDim.x) sh[e] = make_float2(0.f, 0.f);
-    load_spec_cols(kr, a.spec + (long long)k_begin * per);
-  } else {
-    for (int e = threadIdx.x; e < nacc * per; e += blockDim.x) acc[e] = make_float2(0.f, 0.f);
-  }
-  region_async_packed(wbuf[k_begin & 1], src_plane(k_begin), g, i0 - hc, j0 - hc);
-  for (int k = k_begin; k < k_end; ++k) {
-    float2* cur = wbuf[k & 1];
-    cp_async_wait_all();
-    __syncthreads();  // region k landed; every reader of the other buffer is done
-    // the next source's region arrives during this transform
-    if (k + 1 < k_end)
-      region_async_packed(wbuf[(k + 1) & 1], src_plane(k + 1), g, i0 - hc, j0 - hc);
-    if (in_smem) {
-      r2c_2d_accumulate(cur, sh, kr, T);  // the next loop-top barrier orders it
-      if (k + 1 < k_end) load_spec_cols(kr, a.spec + (long long)(k + 1) * per);
-    } else {
-      const int t = student ? k >> 1 : k, base = student ? (k & 1) * R2 : 0;
-      r2c_2d_accumulate_phases(cur, acc + (long long)base * per, a.spec + (long long)t * R2 * per,
-                               R2, T);
-    }
-  }
-  if (in_smem) {
-    __syncthreads();  // the last accumulation is complete
-    if (!last) {
-      adjoint_publish_part(a, tile, sh, q);
-    } else {
-      c2r_2d(sh, T, 0, (B + 1) / 2);  // Den is read at rows [0, B)
-      update_phase(sh, nullptr, a, g, 0, i0, j0, B);
-    }
-  } else {
-    for (int ph = 0; ph < R2; ++ph) {
-      for (int e = threadIdx.x; e < per; e += blockDim.x) {
-        const int m = e >> 7, rr = e & (kFT - 1);
-        sh[rr * kFP + m] = acc[ph * per + e];
-        if (student) wk[rr * kFP + m] = acc[(R2 + ph) * per + e];
-      }
-      __syncthreads();
-      c2r_2d(sh, T, 0, (B + 1) / 2);
-      if (student) c2r_2d(wk, T, 0, (B + 1) / 2);
-      update_phase(sh, student ? wk : nullptr, a, g, (long long)ph * g.plane, i0, j0, B);
-      __syncthreads();
-    }
-  }
+  const float2* slot = a.partials + (long long)prev_cta * kCol;
+  const float2* mine = slot + slot_off();
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = ok ? __ldcg(mine + 32 * i) : make_float2(0.f, 0.f);
+  for (int e = threadIdx.x; e < kFT; e += blockDim.x)
+    a64[e] = ok ? __ldcg(slot + kSlots + e) : make_float2(0.f, 0.f);
   __syncthreads();
 }
 
+// groups > 1: counts this CTA's group of the tile in; the CTA that brings the
+// last one returns true, with the others' accumulators visible to it, and the
+// counter back at zero.
+__device__ bool last_group(const FftLaunch& a, int tile) {
+  __shared__ int last_s;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const bool last = atomicAdd(a.counters + tile, 1) == a.groups - 1;
+    if (last) a.counters[tile] = 0;
+    last_s = last;
+  }
+  __syncthreads();
+  if (last_s) __threadfence();
+  return last_s != 0;
+}
+
+// The adjoint pass and the update of one tile, r = 1: the sources of the pairs
+// [q0, q1) (Student-t: their exposures, w + i w2 each, into the accumulators of
+// both columns of a slot). grp >= 0: group grp of the tile's groups (its
+// accumulators go to partials; the last to arrive adds them and finishes).
+// Otherwise (Gaussian) part `part` of a split launch (prev_cta < 0: from zero),
+// which finishes the tile if it is the last. (nty, ntx): as in
+// fft_forward_tile. Starts and ends at a CTA barrier.
+template <bool STUDENT>
+__device__ void fft_adjoint_tile(const Shape& s, const FftLaunch& a, int ty, int tx, int tile,
+                                 float2* buf, float2* a64, const float4* tw, int q0, int q1,
+                                 int grp, int part = 0, int prev_cta = -1, bool last = true,
+                                 int nty = -1, int ntx = 0) {
+  constexpr int kPer = STUDENT ? 2 * kSlots : kCol;  // float2 of a partial accumulator
+  const Geom& g = s.g;
+  const Lane L;
+  const int hc = s.hc, B = kFT - 2 * hc;
+  const int i0 = ty * B, j0 = tx * B;
+  const int m = L.slot(), m2 = second_col(m);
+  const int blk = L.warp >> 3;
+  float2 acc[16], acc2[STUDENT ? 16 : 1];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    acc[i] = make_float2(0.f, 0.f);
+    if (STUDENT) acc2[STUDENT ? i : 0] = make_float2(0.f, 0.f);
+  }
+  if (!STUDENT) {
+    if (prev_cta >= 0) {
+      resume_part(a, tile, acc, a64, part, prev_cta, last);
+    } else {
+      for (int e = threadIdx.x; e < kFT; e += blockDim.x) a64[e] = make_float2(0.f, 0.f);
+      __syncthreads();
+    }
+  }
+  const int k0 = STUDENT ? 2 * q0 : q0, k1 = STUDENT ? min(2 * q1, s.n) : q1;
+  float2* stage = buf + kFBuf;
+  float2* st = stage + L.warp * kStage;  // Student-t: this warp's slice of the spectrum
+  if (!STUDENT)
+    copy_w(stage + blk * 32 * kFP, a.w + (long long)k0 * g.plane, g, i0 - hc, j0 - hc, blk, L);
+  for (int k = k0; k < k1; ++k) {
+    const float2* w = a.w + (long long)k * g.plane;
+    if (k + 1 < k1) {
+      prefetch_region(w + g.plane, 8, g, i0 - hc, j0 - hc);
+    } else {
+      if (last) {  // what the update reads
+        const long long off = (long long)(g.B + i0) * g.P + g.B + j0;
+        const int rows = min(B, g.H - i0), bytes = 4 * min(B, g.W - j0);
+        prefetch_rows(a.x + off, 4LL * g.P, rows, bytes);
+        prefetch_rows(a.N + off, 4LL * g.P, rows, bytes);
+      }
+      if (nty >= 0) prefetch_region(a.w, 8, g, nty * B - hc, ntx * B - hc);
+    }
+    if (STUDENT) {
+      // the staging buffer holds the spectrum, so both blocks of rows come to
+      // their place in buf now; column 64 of the spectrum goes to a64
+      const float2* S1 = a.spec1 + (long long)k * kCol;
+      copy_w(buf + blk * 32 * kFP, w, g, i0 - hc, j0 - hc, blk, L);
+      stage_slot(st, S1);
+      if (L.warp == 0)
+        for (int e = threadIdx.x; e < kFT; e += 32) a64[e] = __ldg(S1 + kSlots + e);
+      w_rows(nullptr, w, g, i0 - hc, j0 - hc, buf, tw, L);
+    } else {
+      w_rows(stage, w, g, i0 - hc, j0 - hc, buf, tw, L);
+      if (k + 1 < k1)
+        copy_w(stage + blk * 32 * kFP, w + g.plane, g, i0 - hc, j0 - hc, blk, L);
+    }
+    const float2* S = a.spec + (long long)k * kPairSpec + slot_off();
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      float2 kv[STUDENT ? 1 : 16];  // in flight during the transform
+      if (!STUDENT) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) kv[STUDENT ? 0 : i] = __ldg(S + h * kSlots + 32 * i);
+      }
+      float2 v[16];
+      float2* col = buf + (h == 0 ? m : m2);
+      load_col(col, v, L.t, h == 1 && m != 0);
+      fft_col(v, col, tw, L.t);
+      if (STUDENT) {
+        const bool c64 = h == 1 && m == 0;
+        const float2* sp = c64 ? a64 + L.t : st + (threadIdx.x & 31);
+        const int step = c64 ? 8 : 32;
+        if (h == 0) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) acc[i] = cfmac(acc[i], v[i], sp[step * i]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            acc2[STUDENT ? i : 0] = cfmac(acc2[STUDENT ? i : 0], v[i], sp[step * i]);
+        }
+      } else if (h == 1 && m == 0) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          float2* o = a64 + 8 * i + L.t;
+          *o = cfmac(*o, v[i], kv[STUDENT ? 0 : i]);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[i] = cfmac(acc[i], v[i], kv[STUDENT ? 0 : i]);
+      }
+    }
+    __syncthreads();  // the buffer is free for the next source
+  }
+  if (grp >= 0 && a.groups > 1) {
+    float2* mine = a.partials + ((long long)tile * a.groups + grp) * kPer;
+    store_slot(mine, acc);
+    if (STUDENT) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) mine[kSlots + slot_off() + 32 * i] = acc2[STUDENT ? i : 0];
+    } else {
+      for (int e = threadIdx.x; e < kFT; e += blockDim.x) mine[kSlots + e] = a64[e];
+    }
+    if (!last_group(a, tile)) return;
+    const float2* base = a.partials + (long long)tile * a.groups * kPer;
+    for (int k = 0; k < a.groups; ++k) {
+      const float2* p = base + (long long)k * kPer;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const float2 v = __ldcg(p + slot_off() + 32 * i);
+        acc[i] = k ? cadd(acc[i], v) : v;
+        if (STUDENT) {
+          const float2 v2 = __ldcg(p + kSlots + slot_off() + 32 * i);
+          acc2[STUDENT ? i : 0] = k ? cadd(acc2[STUDENT ? i : 0], v2) : v2;
+        }
+      }
+      if (!STUDENT)
+        for (int e = threadIdx.x; e < kFT; e += blockDim.x) {
+          const float2 v = __ldcg(p + kSlots + e);
+          a64[e] = k ? cadd(a64[e], v) : v;
+        }
+    }
+    __syncthreads();
+  }
+  if constexpr (STUDENT) {
+    columns_student(acc, acc2, buf, tw, L);
+  } else {
+    if (!last) {
+      publish_part(a, tile, acc, a64, part);
+      __syncthreads();
+      return;
+    }
+    columns_gauss(acc, a64, buf, tw, L);
+  }
+  rows_update<STUDENT>(s, a, 0, i0, j0, buf, tw, L);
+}
+
+// The same for r > 1, with the accumulators in this item's scratch (`mine`).
+// Layout per phase: Gaussian kCol (slots, column 64), Student-t 2 kSlots (the columns m,
+// then the partners).
+template <bool STUDENT>
+__device__ void fft_adjoint_tile_scratch(const Shape& s, const FftLaunch& a, int ty, int tx,
+                                         int tile, float2* mine, float2* buf, float2* a64,
+                                         const float4* tw, int q0, int q1) {
+  const Geom& g = s.g;
+  const Lane L;
+  const int hc = s.hc, B = kFT - 2 * hc, R2 = s.R2;
+  const int i0 = ty * B, j0 = tx * B;
+  const int m = L.slot(), m2 = second_col(m);
+  const int per = STUDENT ? 2 * kSlots : kCol;
+  const int k0 = STUDENT ? 2 * q0 : q0, k1 = STUDENT ? min(2 * q1, s.n) : q1;
+  float2* stage = buf + kFBuf;
+  copy_w(stage + (L.warp >> 3) * 32 * kFP, a.w + (long long)k0 * g.plane, g, i0 - hc, j0 - hc,
+         L.warp >> 3, L);
+  for (int k = k0; k < k1; ++k) {
+    const float2* w = a.w + (long long)k * g.plane;
+    if (k + 1 < k1) prefetch_region(w + g.plane, 8, g, i0 - hc, j0 - hc);
+    w_rows(stage, w, g, i0 - hc, j0 - hc, buf, tw, L);
+    if (k + 1 < k1)
+      copy_w(stage + (L.warp >> 3) * 32 * kFP, w + g.plane, g, i0 - hc, j0 - hc, L.warp >> 3, L);
+    float2 f[16], c[16];  // the transforms of column m and of its partner
+    load_col(buf + m, f, L.t, false);
+    fft_col(f, buf + m, tw, L.t);
+    load_col(buf + m2, c, L.t, m != 0);
+    fft_col(c, buf + m2, tw, L.t);
+    for (int ph = 0; ph < R2; ++ph) {
+      float2* o = mine + (long long)ph * per + slot_off();
+      if (STUDENT) {
+        const float2* S1 = a.spec1 + ((long long)k * R2 + ph) * kCol;
+        const float2* sp = S1 + slot_off();
+        const float2* sc = m ? sp : S1 + kSlots + L.t;
+        const int cstep = m ? 32 : 8;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float2 z = make_float2(0.f, 0.f);
+          const float2 of = k > k0 ? o[32 * i] : z, oc = k > k0 ? o[kSlots + 32 * i] : z;
+          o[32 * i] = cfmac(of, f[i], sp[32 * i]);
+          o[kSlots + 32 * i] = cfmac(oc, c[i], sc[cstep * i]);
+        }
+      } else {
+        const float2* sp = a.spec + ((long long)k * R2 + ph) * kPairSpec + slot_off();
+        float2* o64 = mine + (long long)ph * per + kSlots + L.t;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float2 z = make_float2(0.f, 0.f);
+          float2 of = k > k0 ? o[32 * i] : z;
+          of = cfmac(of, f[i], sp[32 * i]);
+          if (m) {
+            of = cfmac(of, c[i], sp[kSlots + 32 * i]);
+          } else {
+            const float2 oc = k > k0 ? o64[8 * i] : z;
+            o64[8 * i] = cfmac(oc, c[i], sp[kSlots + 32 * i]);
+          }
+          o[32 * i] = of;
+        }
+      }
+    }
+    __syncthreads();  // the buffer is free for the next source
+  }
+  const long long gstep = (long long)R2 * per;  // scratch of one group
+  int groups = 1;
+  if (a.groups > 1) {
+    if (!last_group(a, tile)) return;
+    groups = a.groups;
+    mine = a.scratch + (long long)tile * groups * gstep;
+  }
+  for (int ph = 0; ph < R2; ++ph) {
+    const float2* p = mine + (long long)ph * per;
+    float2 f[16], c[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) f[i] = c[i] = make_float2(0.f, 0.f);
+    for (int k = 0; k < groups; ++k) {
+      const float2* pk = p + k * gstep;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const float2 v = __ldcg(pk + slot_off() + 32 * i);
+        f[i] = k ? cadd(f[i], v) : v;
+        if (STUDENT) {
+          const float2 w = __ldcg(pk + kSlots + slot_off() + 32 * i);
+          c[i] = k ? cadd(c[i], w) : w;
+        }
+      }
+      if (!STUDENT)
+        for (int e = threadIdx.x; e < kFT; e += blockDim.x) {
+          const float2 v = __ldcg(pk + kSlots + e);
+          a64[e] = k ? cadd(a64[e], v) : v;
+        }
+    }
+    __syncthreads();
+    if (STUDENT)
+      columns_student(f, c, buf, tw, L);
+    else
+      columns_gauss(f, a64, buf, tw, L);
+    rows_update<STUDENT>(s, a, ph, i0, j0, buf, tw, L);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// kernels
+// ---------------------------------------------------------------------------
+
+// pairs [*q0, *q1) of group grp of G over the NP pairs
+__device__ __forceinline__ void group_range(int n, int G, int grp, int* q0, int* q1) {
+  const int NP = (n + 1) / 2;
+  *q0 = (int)((long long)NP * grp / G);
+  *q1 = (int)((long long)NP * (grp + 1) / G);
+}
+
+// float2 of scratch per (tile, group): x^ of the phases (r > 1), then the
+// accumulators
+__host__ __device__ inline long long scratch_floats2(int R2, bool student) {
+  const long long acc = (long long)R2 * (student ? 2 * kSlots : kCol);
+  const long long x = R2 > 1 ? (long long)R2 * kCol : 0;
+  return acc > x ? acc : x;
+}
+
+// item = tile * groups + group
+template <bool R1, bool STUDENT>
+__device__ __forceinline__ void forward_item(const Shape& s, const FftLaunch& a, int gxt, int item,
+                                             float2* fsm, float2* x64, const float4* tw) {
+  const int tile = item / a.groups, grp = item - tile * a.groups;
+  int q0, q1;
+  group_range(s.n, a.groups, grp, &q0, &q1);
+  fft_forward_tile<R1, STUDENT>(s, a, tile / gxt, tile % gxt,
+                                R1 ? nullptr : a.scratch + item * scratch_floats2(s.R2, STUDENT),
+                                fsm, x64, tw, q0, q1);
+}
+
+template <bool R1, bool STUDENT>
+__device__ __forceinline__ void adjoint_item(const Shape& s, const FftLaunch& a, int gxt, int item,
+                                             float2* fsm, float2* a64, const float4* tw) {
+  const int tile = item / a.groups, grp = item - tile * a.groups;
+  int q0, q1;
+  group_range(s.n, a.groups, grp, &q0, &q1);
+  if (R1)
+    fft_adjoint_tile<STUDENT>(s, a, tile / gxt, tile % gxt, tile, fsm, a64, tw, q0, q1, grp);
+  else
+    fft_adjoint_tile_scratch<STUDENT>(
+        s, a, tile / gxt, tile % gxt, tile,
+        a.scratch + item * (long long)s.R2 * (STUDENT ? 2 * kSlots : kCol), fsm, a64, tw, q0, q1);
+}
+
+template <bool R1, bool STUDENT>
 __global__ void __launch_bounds__(kFThreads, 1)
-    fft_adjoint_kernel(const Shape s, const FftLaunch a) {
-  extern __shared__ float2 fsm[];
-  __shared__ TwTab T;
-  init_twiddles(T);
-  fft_adjoint_tile(s, a, blockIdx.y, blockIdx.x, blockIdx.y * gridDim.x + blockIdx.x, fsm, T);
+    fft_forward_kernel(const Shape s, const FftLaunch a, int gxt) {
+  extern __shared__ __align__(16) float2 fsm[];
+  __shared__ float4 tw[kFT / 2];
+  __shared__ float2 x64[kFT];
+  init_twiddles(tw);
+  forward_item<R1, STUDENT>(s, a, gxt, blockIdx.x, fsm, x64, tw);
+}
+
+template <bool R1, bool STUDENT>
+__global__ void __launch_bounds__(kFThreads, 1)
+    fft_adjoint_kernel(const Shape s, const FftLaunch a, int gxt) {
+  extern __shared__ __align__(16) float2 fsm[];
+  __shared__ float4 tw[kFT / 2];
+  __shared__ float2 a64[kFT];
+  init_twiddles(tw);
+  adjoint_item<R1, STUDENT>(s, a, gxt, blockIdx.x, fsm, a64, tw);
+}
+
+// Equal ranges: CTA b of P takes the units [b U / P, (b+1) U / P) of U.
+__device__ __forceinline__ long long split_start(long long U, int P, int b) {
+  return (long long)b * U / P;
 }
 
 // Split forms (r = 1 Gaussian, at least as many tiles as CTAs): P =
@@ -1145,40 +1154,46 @@ __global__ void __launch_bounds__(kFThreads, 1)
 // CTA per tile would (CTA b takes the tiles b + P i, neighbours side by
 // side, so their overlapping regions share the L2); the R = tiles - Wf P
 // tiles of the last, partial wave are spread so that no SM idles through it.
-// Forward: the R n (tile, exposure) units of the last wave in equal ranges
-// over all CTAs (tile-major; a CTA recomputes x^ for each tile it touches).
+// Forward: the (tile, pair) units of the last wave in equal ranges over all
+// CTAs (tile-major; a CTA recomputes x^ for each tile it touches).
 __global__ void __launch_bounds__(kFThreads, 1)
     fft_forward_split_kernel(const Shape s, const FftLaunch a, int gxt, int tiles) {
-  extern __shared__ float2 fsm[];
-  __shared__ TwTab T;
-  init_twiddles(T);
-  const int P = a.split_ctas, n = s.n, b = blockIdx.x;
+  extern __shared__ __align__(16) float2 fsm[];
+  __shared__ float4 tw[kFT / 2];
+  __shared__ float2 x64[kFT];
+  init_twiddles(tw);
+  const int P = a.split_ctas, n = (s.n + 1) / 2, b = blockIdx.x;
   const int Wf = tiles / P, R = tiles - Wf * P;
-  for (int i = 0; i < Wf; ++i) {
-    const int tile = b + P * i;
-    fft_forward_tile<false>(s, a, tile / gxt, tile % gxt, tile, fsm, T, 0, n);
-  }
   const long long U = (long long)R * n, base = (long long)Wf * P * n;
   const long long u_end = split_start(U, P, b + 1);
-  for (long long u = split_start(U, P, b); u < u_end;) {
-    const int tile = (int)((base + u) / n), t0 = (int)((base + u) % n);
-    const int t1 = (int)min((long long)n, t0 + (u_end - u));
-    fft_forward_tile<false>(s, a, tile / gxt, tile % gxt, tile, fsm, T, t0, t1);
-    u += t1 - t0;
+  long long u = split_start(U, P, b);
+  for (int i = 0; i < Wf || u < u_end; ++i) {
+    int tile, q0 = 0, q1 = n;
+    if (i < Wf) {
+      tile = b + P * i;
+    } else {
+      tile = (int)((base + u) / n), q0 = (int)((base + u) % n);
+      q1 = (int)min((long long)n, q0 + (u_end - u));
+      u += q1 - q0;
+    }
+    const int next = i + 1 < Wf ? tile + P : -1;
+    fft_forward_tile<true, false>(s, a, tile / gxt, tile % gxt, nullptr, fsm, x64, tw, q0, q1,
+                                  next >= 0 ? next / gxt : -1, next >= 0 ? next % gxt : 0);
   }
 }
 
-// Adjoint: last-wave tile j is cut into k = min(n, P / R) parts of
-// consecutive exposures, part q on CTA q R + j, which runs it after
+// Adjoint: last-wave tile j is cut into k = min(pairs, P / R) parts of
+// consecutive pairs, part q on CTA q R + j, which runs it after
 // q Wf / (k - 1) of its whole tiles (part 0 first, part k - 1 last), so
 // each part finds its predecessor done waves earlier and the last wave
 // costs 1 / k of a tile.
 __global__ void __launch_bounds__(kFThreads, 1)
     fft_adjoint_split_kernel(const Shape s, const FftLaunch a, int gxt, int tiles) {
-  extern __shared__ float2 fsm[];
-  __shared__ TwTab T;
-  init_twiddles(T);
-  const int P = a.split_ctas, n = s.n, b = blockIdx.x;
+  extern __shared__ __align__(16) float2 fsm[];
+  __shared__ float4 tw[kFT / 2];
+  __shared__ float2 a64[kFT];
+  init_twiddles(tw);
+  const int P = a.split_ctas, n = (s.n + 1) / 2, b = blockIdx.x;
   const int Wf = tiles / P, R = tiles - Wf * P;
   const int k = R > 0 ? max(1, min(n, P / R)) : 0;
   const int has = b < k * R, q = has ? b / R : 0, j = has ? b % R : 0;
@@ -1192,12 +1207,14 @@ __global__ void __launch_bounds__(kFThreads, 1)
     } else {
       tile = b + P * (it - (has && it > pos));
     }
-    fft_adjoint_tile(s, a, tile / gxt, tile % gxt, tile, fsm, T, k0, k1, qq, prev, last);
+    const int next = it + 1 < Wf && it != pos ? tile + P : -1;
+    fft_adjoint_tile<false>(s, a, tile / gxt, tile % gxt, tile, fsm, a64, tw, k0, k1, -1, qq, prev, last,
+                     next >= 0 ? next / gxt : -1, next >= 0 ? next % gxt : 0);
   }
 }
 
-// Persistent forms for a batch of FFT jobs: every CTA claims (job, tile)
-// items from a device counter until the list is exhausted; jobs whose
+// Persistent forms for a batch of FFT jobs: every CTA claims (job, item)
+// entries from a device counter until the list is exhausted; jobs whose
 // iterations are done are skipped. One launch for the forward passes of all
 // jobs, then one for the adjoints (the adjoint reads its neighbours' w).
 __device__ __forceinline__ int claim_item(int* counter, int* slot) {
@@ -1210,10 +1227,11 @@ __device__ __forceinline__ int claim_item(int* counter, int* slot) {
 __global__ void __launch_bounds__(kFThreads, 1)
     fft_batch_forward_kernel(const FftBatchJob* __restrict__ jobs, const int2* __restrict__ items,
                              const int* __restrict__ n_items, int* __restrict__ counter) {
-  extern __shared__ float2 fsm[];
-  __shared__ TwTab T;
+  extern __shared__ __align__(16) float2 fsm[];
+  __shared__ float4 tw[kFT / 2];
+  __shared__ float2 x64[kFT];
   __shared__ int slot;
-  init_twiddles(T);
+  init_twiddles(tw);
   const int total = *n_items;
   for (;;) {
     const int item = claim_item(counter, &slot);
@@ -1221,17 +1239,21 @@ __global__ void __launch_bounds__(kFThreads, 1)
     const int2 w = items[item];
     const FftBatchJob& J = jobs[w.x];
     if (J.remaining <= 0) continue;
-    fft_forward_tile(J.s, J.a[J.cur], w.y / J.gxt, w.y % J.gxt, w.y, fsm, T, 0, J.s.n);
+    if (J.s.R2 == 1)
+      forward_item<true, false>(J.s, J.a[J.cur], J.gxt, w.y, fsm, x64, tw);
+    else
+      forward_item<false, false>(J.s, J.a[J.cur], J.gxt, w.y, fsm, x64, tw);
   }
 }
 
 __global__ void __launch_bounds__(kFThreads, 1)
     fft_batch_adjoint_kernel(const FftBatchJob* __restrict__ jobs, const int2* __restrict__ items,
                              const int* __restrict__ n_items, int* __restrict__ counter) {
-  extern __shared__ float2 fsm[];
-  __shared__ TwTab T;
+  extern __shared__ __align__(16) float2 fsm[];
+  __shared__ float4 tw[kFT / 2];
+  __shared__ float2 a64[kFT];
   __shared__ int slot;
-  init_twiddles(T);
+  init_twiddles(tw);
   const int total = *n_items;
   for (;;) {
     const int item = claim_item(counter, &slot);
@@ -1239,7 +1261,10 @@ __global__ void __launch_bounds__(kFThreads, 1)
     const int2 w = items[item];
     const FftBatchJob& J = jobs[w.x];
     if (J.remaining <= 0) continue;
-    fft_adjoint_tile(J.s, J.a[J.cur], w.y / J.gxt, w.y % J.gxt, w.y, fsm, T);
+    if (J.s.R2 == 1)
+      adjoint_item<true, false>(J.s, J.a[J.cur], J.gxt, w.y, fsm, a64, tw);
+    else
+      adjoint_item<false, false>(J.s, J.a[J.cur], J.gxt, w.y, fsm, a64, tw);
   }
 }
 
@@ -1251,69 +1276,91 @@ __global__ void fft_batch_advance_kernel(FftBatchJob* __restrict__ jobs, int njo
   }
 }
 
-}  // namespace
-
-static size_t fft_tiles(const Shape& s) {
-  const int B = kFT - 2 * s.hc;
-  return (size_t)((s.g.W + B - 1) / B) * ((s.g.H + B - 1) / B);
-}
-
-// layout of the FFT buffer: PSF spectra (n R2), w planes (n), for Student-t
-// the w2 planes (n), then the per-tile scratch (r > 1: tiles R2 spectra;
-// Student-t: tiles 2 R2)
-size_t fft_w2_offset(const Shape& s) {
-  const size_t spec = ((size_t)s.n * s.R2 * kFT * kFBins * sizeof(float2) + 255) & ~(size_t)255;
-  const size_t wpl = ((size_t)s.n * s.g.plane * sizeof(float) + 255) & ~(size_t)255;
-  return spec + wpl;
-}
-
-size_t fft_scratch_offset(const Shape& s, bool student) {
-  const size_t wpl = ((size_t)s.n * s.g.plane * sizeof(float) + 255) & ~(size_t)255;
-  return fft_w2_offset(s) + (student ? wpl : 0);
-}
-
-size_t fft_split_offset(const Shape& s, bool student) {
-  const int nacc = student ? 2 * s.R2 : (s.R2 > 1 ? s.R2 : 0);
-  const size_t scratch = fft_tiles(s) * nacc * kFT * kFBins * sizeof(float2);
-  return (fft_scratch_offset(s, student) + scratch + 255) & ~(size_t)255;
-}
-
-static bool fft_splits_adjoint(const Shape& s, bool student) { return s.R2 == 1 && !student; }
-
-size_t fft_counters_offset(const Shape& s, bool student, int split_ctas) {
-  const size_t parts = fft_splits_adjoint(s, student) && split_ctas > 0
-                           ? (size_t)split_ctas * kFBuf * sizeof(float2)
-                           : 0;
-  return fft_split_offset(s, student) + parts;
-}
-
-size_t fft_buffer_bytes(const Shape& s, bool student, int split_ctas) {
-  const size_t counters =
-      fft_splits_adjoint(s, student) && split_ctas > 0 ? fft_tiles(s) * sizeof(int) : 0;
-  return fft_counters_offset(s, student, split_ctas) + counters;
-}
-
-// two transform buffers and a 128 x 128 float staging area
-// three transform buffers (the adjoint: accumulator and two work buffers;
-// the forward: x^, work buffer and a 128 x 128 float staging area)
-size_t fft_smem_bytes() { return 3 * (size_t)kFBuf * sizeof(float2); }
-
-int fft_tile_side(const Shape& s) { return kFT - 2 * s.hc; }
-
-cudaError_t launch_fft_spectra(const Shape& s, const float* ka, float2* spec, cudaStream_t st) {
-  const size_t smem = (size_t)kFBuf * sizeof(float2);
-  cudaError_t e = allow_max_dynamic_smem((const void*)fft_spectra_kernel);
+template <bool R1, bool STUDENT>
+cudaError_t launch_pair(const Shape& s, const FftLaunch& a, int gxt, int tiles, cudaStream_t st) {
+  const size_t smem = fft_smem_bytes();
+  cudaError_t e = allow_max_dynamic_smem((const void*)fft_forward_kernel<R1, STUDENT>);
+  if (e == cudaSuccess) e = allow_max_dynamic_smem((const void*)fft_adjoint_kernel<R1, STUDENT>);
   if (e != cudaSuccess) return e;
-  fft_spectra_kernel<<<s.n * s.R2, kFThreads, smem, st>>>(ka, s.Kc, s.KP, spec);
+  fft_forward_kernel<R1, STUDENT><<<tiles * a.groups, kFThreads, smem, st>>>(s, a, gxt);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  fft_adjoint_kernel<R1, STUDENT><<<tiles * a.groups, kFThreads, smem, st>>>(s, a, gxt);
   return cudaGetLastError();
 }
 
+size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
+
+}  // namespace
+
+int fft_tile_side(const Shape& s) { return kFT - 2 * s.hc; }
+
 int fft_tiles_x(const Shape& s) {
-  const int B = kFT - 2 * s.hc;
+  const int B = fft_tile_side(s);
   return (s.g.W + B - 1) / B;
 }
 
-int fft_tiles_total(const Shape& s) { return (int)fft_tiles(s); }
+int fft_tiles_total(const Shape& s) {
+  const int B = fft_tile_side(s);
+  return fft_tiles_x(s) * ((s.g.H + B - 1) / B);
+}
+
+// Exposure groups per tile: the count that takes the fewest transforms one
+// after the other, ceil(tiles G / SMs) rounds of ceil(pairs / G) pairs plus
+// about one transform of overhead (x^, or the inverse and the update). It
+// depends on the shape alone: a job's bits are the same alone and in a batch.
+int fft_groups(const Shape& s) {
+  const long long tiles = fft_tiles_total(s);
+  const int NP = (s.n + 1) / 2;
+  int best = 1;
+  long long best_cost = 0;
+  for (int G = 1; G <= NP && (G == 1 || tiles * G <= 2 * kSMs); ++G) {
+    const long long cost = (tiles * G + kSMs - 1) / kSMs * ((NP + G - 1) / G + 1);
+    if (G == 1 || cost < best_cost) {
+      best = G;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
+// pair spectra, single spectra (Student-t), w planes, scratch, partials, counters
+FftLayout fft_layout(const Shape& s, bool student, int split_ctas) {
+  FftLayout L{};
+  const size_t NP = (s.n + 1) / 2, tiles = fft_tiles_total(s), G = fft_groups(s);
+  const size_t wplanes = student ? s.n : NP;  // float2 planes
+  size_t off = 0;
+  auto take = [&](size_t bytes) { const size_t o = off; off += up256(bytes); return o; };
+  L.spec = take(NP * s.R2 * kPairSpec * sizeof(float2));
+  L.spec1 = take(student ? (size_t)s.n * s.R2 * kCol * sizeof(float2) : 0);
+  L.w = take(wplanes * s.g.plane * sizeof(float2));
+  const bool r1 = s.R2 == 1;
+  L.scratch = take(r1 ? 0 : tiles * G * scratch_floats2(s.R2, student) * sizeof(float2));
+  // slots of the split launch (one per CTA) or of the groups
+  const bool split = r1 && !student && split_ctas > 0 && tiles >= (size_t)split_ctas;
+  L.partials = take((split ? (size_t)split_ctas : r1 && G > 1 ? tiles * G : 0) *
+                    (student ? 2 * kSlots : kCol) * sizeof(float2));
+  L.counters = take(split || G > 1 ? tiles * sizeof(int) : 0);
+  L.total = off;
+  return L;
+}
+
+// the transform buffer and the staging buffer (the forward pass: 4 KB of
+// spectrum per warp; the adjoint: 64 rows of the next w region)
+size_t fft_smem_bytes() {
+  return (size_t)(kFBuf + std::max(kFThreads / 32 * kStage, 64 * kFP)) * sizeof(float2);
+}
+
+cudaError_t launch_fft_spectra(const Shape& s, const float* ka, float2* spec, float2* spec1,
+                               cudaStream_t st) {
+  const size_t smem = fft_smem_bytes();
+  cudaError_t e = allow_max_dynamic_smem((const void*)fft_spectra_kernel);
+  if (e != cudaSuccess) return e;
+  fft_spectra_kernel<<<(s.n + 1) / 2 * s.R2, kFThreads, smem, st>>>(ka, s.n, s.R2, s.Kc, s.KP,
+                                                                    false, spec);
+  if ((e = cudaGetLastError()) != cudaSuccess || !spec1) return e;
+  fft_spectra_kernel<<<s.n * s.R2, kFThreads, smem, st>>>(ka, s.n, s.R2, s.Kc, s.KP, true, spec1);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_fft_batch(const FftBatchJob* jobs, int njobs, const int2* items,
                              const int* n_items, int* counters, int ctas, cudaStream_t st) {
@@ -1334,31 +1381,20 @@ cudaError_t launch_fft_batch(const FftBatchJob* jobs, int njobs, const int2* ite
 }
 
 cudaError_t launch_fft_iter(const Shape& s, const FftLaunch& a, cudaStream_t st) {
+  const int gxt = fft_tiles_x(s), tiles = fft_tiles_total(s);
+  if (a.nu > 0.f)
+    return s.R2 == 1 ? launch_pair<true, true>(s, a, gxt, tiles, st)
+                     : launch_pair<false, true>(s, a, gxt, tiles, st);
+  if (s.R2 > 1) return launch_pair<false, false>(s, a, gxt, tiles, st);
+  if (a.split_ctas <= 0 || tiles < a.split_ctas)
+    return launch_pair<true, false>(s, a, gxt, tiles, st);
   const size_t smem = fft_smem_bytes();
-  cudaError_t e = allow_max_dynamic_smem((const void*)fft_forward_kernel);
-  if (e == cudaSuccess) e = allow_max_dynamic_smem((const void*)fft_adjoint_kernel);
-  if (e == cudaSuccess) e = allow_max_dynamic_smem((const void*)fft_forward_split_kernel);
+  cudaError_t e = allow_max_dynamic_smem((const void*)fft_forward_split_kernel);
   if (e == cudaSuccess) e = allow_max_dynamic_smem((const void*)fft_adjoint_split_kernel);
   if (e != cudaSuccess) return e;
-  const int B = fft_tile_side(s);
-  const dim3 grid((s.g.W + B - 1) / B, (s.g.H + B - 1) / B);
-  // the split forms: r = 1 (the forward pass of r > 1 keeps x^ in the
-  // tile's scratch), Gaussian (the partial slots), at least as many tiles
-  // as CTAs
-  const bool split = s.R2 == 1 && a.nu <= 0.f && a.split_ctas > 0 && a.partials &&
-                     a.counters && a.err && (long long)fft_tiles(s) >= a.split_ctas;
-  if (split)
-    fft_forward_split_kernel<<<a.split_ctas, kFThreads, smem, st>>>(s, a, (int)grid.x,
-                                                                     (int)fft_tiles(s));
-  else
-    fft_forward_kernel<<<grid, kFThreads, smem, st>>>(s, a);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (split)
-    fft_adjoint_split_kernel<<<a.split_ctas, kFThreads, smem, st>>>(s, a, (int)grid.x,
-                                                                     (int)fft_tiles(s));
-  else
-    fft_adjoint_kernel<<<grid, kFThreads, smem, st>>>(s, a);
+  fft_forward_split_kernel<<<a.split_ctas, kFThreads, smem, st>>>(s, a, gxt, tiles);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  fft_adjoint_split_kernel<<<a.split_ctas, kFThreads, smem, st>>>(s, a, gxt, tiles);
   return cudaGetLastError();
 }
 

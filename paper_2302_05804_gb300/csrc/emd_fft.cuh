@@ -7,43 +7,46 @@
 
 namespace emd {
 
-// FFT path: overlap-save on 128 x 128 tiles
+// FFT path: overlap-save on 128 x 128 tiles, two exposures per complex transform
 struct FftLaunch {
-  const float* x;       // current iterate (padded plane)
+  const float* x;       // current iterate (padded planes)
   float* xn;            // next iterate
   const float* N;       // numerator
   const float* u;       // n weight planes
-  float* w;             // n planes of u_t z_t (written by the forward pass)
-  const float2* spec;   // n R2 half spectra of the phase kernels, 65 columns x 128 rows each
-  float2* scratch;      // per tile (r > 1 or Student-t): R2 half spectra of the phases
-                        // of x, then the adjoint's accumulators (R2, or 2 R2 for
-                        // Student-t: Den then N'); unused for r = 1 Gaussian
+  float2* w;            // weighted model images on the padded planes, as float2:
+                        // Gaussian: plane q holds (w_2q, w_2q+1); Student-t: plane t
+                        // holds (u'_t z_t, u'_t y_t)
+  const float2* spec;   // pair spectra (fft_pair_spec float2 per pair and phase)
+  const float2* spec1;  // Student-t: spectra of the single kernels
+  float2* scratch;      // r > 1, per (tile, group): the phases' x^, then the adjoint's
+                        // accumulators
   const float* y;       // Student-t: n data planes (masked pixels 0)
-  float* w2;            // Student-t: n planes of u'_t y_t
   float nu;             // Student-t degrees of freedom; 0 = Gaussian
-  // split launch (r = 1, at least split_ctas tiles): split_ctas persistent
-  // CTAs take equal ranges of the (tile, exposure) units; an adjoint tile
-  // cut between two CTAs passes its head's accumulator through the head
-  // CTA's slot (partials, one per CTA) and the tile's flag (counters).
-  // split_ctas = 0: one CTA per tile.
+  int groups;           // exposure groups per tile (fft_groups)
+  // groups > 1: accumulators of the groups of a tile, one slot per (tile, group), and
+  // arrival counters per tile. Split launch (r = 1 Gaussian, at least
+  // split_ctas tiles): one slot per CTA and a flag per tile (emd_fft.cu).
   float2* partials;
   int* counters;
-  int split_ctas;
+  int split_ctas;       // SMs of the device
   int* err;  // device error word (a bounded wait that gives up sets kErrTimeout)
 };
-// bytes of the FFT buffer; split_ctas > 0 adds the split launch's partial
-// accumulators and counters (r = 1 Gaussian)
-size_t fft_buffer_bytes(const Shape& s, bool student, int split_ctas = 0);
-size_t fft_split_offset(const Shape& s, bool student);     // bytes before the partials
-size_t fft_counters_offset(const Shape& s, bool student, int split_ctas);
+
+// The FFT buffer: byte offsets of its parts and its size. student: heavy-tailed
+// noise; split_ctas: persistent CTAs of the split launch (0: none)
+struct FftLayout {
+  size_t spec, spec1, w, scratch, partials, counters, total;
+};
+FftLayout fft_layout(const Shape& s, bool student, int split_ctas);
+int fft_groups(const Shape& s);  // exposure groups per tile of this shape
 size_t fft_smem_bytes();
 int fft_tile_side(const Shape& s);
-size_t fft_w2_offset(const Shape& s);                      // bytes before the w2 planes
-size_t fft_scratch_offset(const Shape& s, bool student);  // bytes before the scratch
-cudaError_t launch_fft_spectra(const Shape& s, const float* ka, float2* spec, cudaStream_t st);
+// spec (and, when not null, spec1) from the adjoint kernels ka
+cudaError_t launch_fft_spectra(const Shape& s, const float* ka, float2* spec, float2* spec1,
+                               cudaStream_t st);
 cudaError_t launch_fft_iter(const Shape& s, const FftLaunch& a, cudaStream_t st);
 
-// batch of FFT jobs: persistent forward and adjoint kernels over (job, tile)
+// batch of FFT jobs: persistent forward and adjoint kernels over (job, tile and group)
 struct FftBatchJob {
   Shape s;
   FftLaunch a[2];  // with x = buffer c, xn = buffer c^1, for c = cur

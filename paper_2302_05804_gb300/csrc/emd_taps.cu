@@ -32,7 +32,6 @@ namespace emd {
 namespace {
 
 constexpr int kSMs = 152;
-constexpr uint32_t kBarrierPolls = 1u << 23;  // x ~0.5 us per poll: seconds, not a hang
 
 // ---------------------------------------------------------------------------
 // correlation with the taps in the constant bank
@@ -425,32 +424,6 @@ struct SplitArgs {
   int numerator;    // w = u y instead of u z; the sum goes to a.Nw as it is
   int gx, T;
 };
-
-// Grid barrier number `round` (from 1) of a cooperative launch; every thread
-// of the CTA calls it. Bounded: a wait that gives up raises the abort flag,
-// which ends all later waits; returns false then.
-__device__ bool grid_barrier(int* ctrl, int round, int* ok_s) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    atomicAdd(&ctrl[0], 1);
-    const int target = round * (int)gridDim.x;
-    uint32_t i = 0;
-    bool ok = false;
-    for (; i < kBarrierPolls; ++i) {
-      if (ld_acquire(&ctrl[0]) >= target) {
-        ok = true;
-        break;
-      }
-      if (ld_relaxed(&ctrl[2])) break;
-      if (i > 64) __nanosleep(100);
-    }
-    if (!ok) atomicExch(&ctrl[2], 1);
-    *ok_s = ok;
-  }
-  __syncthreads();
-  return *ok_s != 0;
-}
 
 template <int V, bool STUDENT>
 __global__ void __launch_bounds__(SplitTile<V>::TH / 2 * (SplitTile<V>::TW / SplitTile<V>::RX))
