@@ -66,6 +66,29 @@ __device__ __forceinline__ void corr_taps(float (&acc)[RX], const float4 k,
 // inside 55: all execute over 90 % FMAs, and what differs is the dispatch
 // stall (0.3-0.5 per issue), which more warps cover and a larger block, with
 // fewer loads, does not.
+// U source rows (U = 2 or 4) of a block of four output rows, the first at row
+// s: xb[0] holds its window, q[j] the quad of kernel row s - 1 - j; skew: 4 if
+// s mod 4 = 3 (the rows' skew steps at the next row), else 0. The next row's
+// window is loaded before a row's FMAs. On return xb[0] holds row s + U.
+template <int U, int RX>
+__device__ __forceinline__ void corr4_rows(float (&acc)[4][RX], float4 (&q)[3],
+                                           float (&xb)[2][RX + 4], const float*& row,
+                                           const float*& kq, int pitch, int KP, int skew) {
+  float4 nw[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    nw[u] = *reinterpret_cast<const float4*>(kq);
+    kq += KP;
+    row += u == 0 ? pitch + skew : pitch;
+    corr_window<RX>(xb[(u + 1) & 1], row);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) corr_taps<RX>(acc[p], p <= u ? nw[u - p] : q[p - u - 1], xb[u & 1]);
+  }
+  if (U == 2) q[2] = q[0];
+#pragma unroll
+  for (int j = 0; j < (U == 2 ? 2 : 3); ++j) q[j] = nw[U - 1 - j];
+}
+
 template <int RY, int RX>
 __device__ __forceinline__ void corr_tile(float (&acc)[RY][RX], const SPlane& src, int oy,
                                           int ox, const float* __restrict__ ks, int KP,
@@ -101,25 +124,77 @@ __device__ __forceinline__ void corr_tile(float (&acc)[RY][RX], const SPlane& sr
       }
       corr_taps<RX>(acc[1], k1, xv);  // source row Kc: output row 1 only
     }
-  } else {
+    return;
+  }
+  if constexpr (RY == 4) {
+    // rows 0 .. 2 and Kc .. Kc + 2 as unrolled triangles, no checks between
+    if (Kc >= 3) {
 #pragma unroll 1
-    for (int b = 0; b < KP; b += 4) {
-      float4 kv[RY];  // quad of kernel row a in slot a mod RY
-      const float* row = col + b;
-      const float* kq = ks + b;
+      for (int b = 0; b < KP; b += 4) {
+        const float* row = col + b;
+        const float* kq = ks + b;
+        float xb[2][RX + 4];
+        float4 q[3];
+        corr_window<RX>(xb[0], row);
+        q[2] = *reinterpret_cast<const float4*>(kq);
+        q[1] = *reinterpret_cast<const float4*>(kq + KP);
+        q[0] = *reinterpret_cast<const float4*>(kq + 2 * KP);
+        kq += 3 * KP;
+        row += pitch;
+        corr_window<RX>(xb[1], row);
+        corr_taps<RX>(acc[0], q[2], xb[0]);
+        row += pitch;
+        corr_window<RX>(xb[0], row);
+        corr_taps<RX>(acc[0], q[1], xb[1]);
+        corr_taps<RX>(acc[1], q[2], xb[1]);
+        row += pitch;
+        corr_window<RX>(xb[1], row);
+        corr_taps<RX>(acc[0], q[0], xb[0]);
+        corr_taps<RX>(acc[1], q[1], xb[0]);
+        corr_taps<RX>(acc[2], q[2], xb[0]);
+#pragma unroll
+        for (int c = 0; c < RX + 4; ++c) xb[0][c] = xb[1][c];
+        // Kc mod 4 = 1: two rows at a time, one loop: a remainder after the
+        // four-row loop would push the code out of the instruction cache
+        if ((Kc & 3) == 3) {
 #pragma unroll 1
-      for (int s0 = 0; s0 < Kc + RY - 1; s0 += RY, row += RY * pitch + 4, kq += RY * KP) {
-#pragma unroll
-        for (int u = 0; u < RY; ++u) {
-          const int s = s0 + u;
-          if (s >= Kc + RY - 1) break;
-          float xv[RX + 4];
-          corr_window<RX>(xv, row + u * pitch);
-          if (s < Kc) kv[u] = *reinterpret_cast<const float4*>(kq + u * KP);
-#pragma unroll
-          for (int p = 0; p < RY; ++p)
-            if (s - p >= 0 && s - p < Kc) corr_taps<RX>(acc[p], kv[(u + RY - p) % RY], xv);
+          for (int s = 3; s < Kc; s += 4) corr4_rows<4, RX>(acc, q, xb, row, kq, pitch, KP, 4);
+        } else {
+#pragma unroll 1
+          for (int s = 3, skew = 4; s < Kc; s += 2, skew ^= 4)
+            corr4_rows<2, RX>(acc, q, xb, row, kq, pitch, KP, skew);
         }
+        row += (Kc & 3) == 3 ? pitch + 4 : pitch;
+        corr_window<RX>(xb[1], row);
+        corr_taps<RX>(acc[1], q[0], xb[0]);
+        corr_taps<RX>(acc[2], q[1], xb[0]);
+        corr_taps<RX>(acc[3], q[2], xb[0]);
+        row += pitch;
+        corr_window<RX>(xb[0], row);
+        corr_taps<RX>(acc[2], q[0], xb[1]);
+        corr_taps<RX>(acc[3], q[1], xb[1]);
+        corr_taps<RX>(acc[3], q[0], xb[0]);
+      }
+      return;
+    }
+  }
+#pragma unroll 1
+  for (int b = 0; b < KP; b += 4) {
+    float4 kv[RY];  // quad of kernel row a in slot a mod RY
+    const float* row = col + b;
+    const float* kq = ks + b;
+#pragma unroll 1
+    for (int s0 = 0; s0 < Kc + RY - 1; s0 += RY, row += RY * pitch + 4, kq += RY * KP) {
+#pragma unroll
+      for (int u = 0; u < RY; ++u) {
+        const int s = s0 + u;
+        if (s >= Kc + RY - 1) break;
+        float xv[RX + 4];
+        corr_window<RX>(xv, row + u * pitch);
+        if (s < Kc) kv[u] = *reinterpret_cast<const float4*>(kq + u * KP);
+#pragma unroll
+        for (int p = 0; p < RY; ++p)
+          if (s - p >= 0 && s - p < Kc) corr_taps<RX>(acc[p], kv[(u + RY - p) % RY], xv);
       }
     }
   }

@@ -41,19 +41,19 @@ __device__ __forceinline__ float4 bank_quad(const TapBank& bank, int off) {
   return reinterpret_cast<const float4*>(bank.k)[off >> 2];
 }
 
-// U source rows (U = 2 or 4), the first at row s with s mod 4 = 3: xv holds
-// its window, q[j] the quad of kernel row s - 1 - j. On return xv holds row
-// s + U.
+// U source rows (U = 2 or 4), the first at row s: xv holds its window, q[j] the
+// quad of kernel row s - 1 - j; skew: 4 if s mod 4 = 3 (the rows' skew steps at
+// the next row), else 0. On return xv holds row s + U.
 template <int U>
 __device__ __forceinline__ void bank_rows(float (&acc)[4][16], float4 (&q)[3], float (&xv)[20],
                                           const float*& row, int& ko, int pitch, int KP,
-                                          const TapBank& bank) {
+                                          const TapBank& bank, int skew) {
   float4 nw[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     nw[u] = bank_quad(bank, ko);
     ko += KP;
-    row += u == 0 ? pitch + 4 : pitch;  // the skew steps where s mod 4 = 0
+    row += u == 0 ? pitch + skew : pitch;
 #pragma unroll
     for (int p = 0; p < 4; ++p) corr_taps<16>(acc[p], p <= u ? nw[u - p] : q[p - u - 1], xv);
     corr_window<16>(xv, row);
@@ -95,10 +95,17 @@ __device__ __forceinline__ void corr_bank(float (&acc)[4][16], const SPlane& src
     q[0] = k2;
     q[1] = k1;
     q[2] = k0;
-    int s = 3;
+    // Kc mod 4 = 1: two rows at a time, one loop: a remainder after the
+    // four-row loop pushed the code out of the instruction cache (K = 25 at 40
+    // TFLOP/s)
+    if ((Kc & 3) == 3) {
 #pragma unroll 1
-    for (; s + 4 <= Kc; s += 4) bank_rows<4>(acc, q, xv, row, ko, pitch, KP, bank);
-    if (s < Kc) bank_rows<2>(acc, q, xv, row, ko, pitch, KP, bank);  // Kc mod 4 = 1
+      for (int s = 3; s < Kc; s += 4) bank_rows<4>(acc, q, xv, row, ko, pitch, KP, bank, 4);
+    } else {
+#pragma unroll 1
+      for (int s = 3, skew = 4; s < Kc; s += 2, skew ^= 4)
+        bank_rows<2>(acc, q, xv, row, ko, pitch, KP, bank, skew);
+    }
     corr_taps<16>(acc[1], q[0], xv);
     corr_taps<16>(acc[2], q[1], xv);
     corr_taps<16>(acc[3], q[2], xv);
@@ -292,10 +299,9 @@ struct TapsArgs {
   FusedArgs a;      // t0, t1: all exposures of the iteration
   float* w;         // chunk planes (heavy-tailed: then chunk planes of w2)
   float* part;      // parts: chunk x R2 planes (heavy-tailed: twice)
-  int* counters;    // parts: one per (phase, tile)
   int c0, ne;       // exposures [c0, c0 + ne) of this launch
   int epi;          // exposures per forward item
-  int parts;        // adjoint partials per exposure, summed by the last CTA of a tile
+  int parts;        // adjoint partials per exposure, summed by taps_sum_kernel
   int numerator;    // the sum over the exposures goes to a.Nw as it is
   int gx, T;        // tiles per row, tiles
 };
@@ -337,7 +343,6 @@ __global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), 
     taps_adjoint_kernel(const Shape s, const TapsArgs A, const __grid_constant__ TapBank bank) {
   constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NY = TH / 4, NT = NY * (TW / 16);
   extern __shared__ __align__(128) float smem[];
-  __shared__ int flag_s;
   const Geom& g = s.g;
   const SPlane sp{smem, TW + s.KP};
   const int my = threadIdx.x % NY, mx = threadIdx.x / NY;
@@ -396,8 +401,17 @@ __global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), 
       }
     }
   }
-  if (A.parts && last_to_arrive(A.counters + phi * A.T + k, A.ne, &flag_s))
-    sum_parts<4, 16, STUDENT>(s, A.a, A.part, A.ne, phi, i, j, first, last, A.numerator);
+}
+
+// parts: adds the chunk's partials in exposure order, one row of 4 x 128 pixels
+// per CTA (blockIdx.y: row, z: phase). A launch of its own: counting the items
+// of a tile in instead costs every item a fence and an atomic round trip.
+template <bool STUDENT>
+__global__ void __launch_bounds__(128) taps_sum_kernel(const Shape s, const TapsArgs A) {
+  const int j = 4 * (blockIdx.x * 128 + threadIdx.x);
+  if (j < s.g.W)
+    sum_parts<1, 4, STUDENT>(s, A.a, A.part, A.ne, blockIdx.z, blockIdx.y, j, A.c0 == A.a.t0,
+                             A.c0 + A.ne == A.a.t1, A.numerator);
 }
 
 // ---------------------------------------------------------------------------
@@ -630,7 +644,6 @@ cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunc
   TapsArgs A;
   A.a = h.a;
   A.w = h.work;
-  A.counters = h.counters + 64;
   A.parts = p.parts;
   A.numerator = numerator;
   A.gx = cdiv(s.W, TW);
@@ -654,6 +667,10 @@ cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunc
     taps_adjoint_kernel<V, STUDENT>
         <<<dim3(A.T, s.R2, p.parts ? A.ne : 1), NT, smem, st>>>(s, A, bank);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (p.parts) {
+      taps_sum_kernel<STUDENT><<<dim3(cdiv(s.W, 512), s.H, s.R2), 128, 0, st>>>(s, A);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
   }
   return cudaSuccess;
 }
