@@ -413,6 +413,93 @@ __device__ __forceinline__ void rows_forward(float2* buf, const float4* tw, cons
 }
 
 // ---------------------------------------------------------------------------
+// tensor memory as thread-private storage (r = 2)
+// ---------------------------------------------------------------------------
+
+// A slot's spectrum is 16 complex values a thread, so four phases' are 128
+// words of each of the 512 threads: the SM's 256 KB of tensor memory, which
+// the FFT form does not use otherwise. x^ (forward) and the Gaussian
+// accumulators (adjoint) of r = 2 live there instead of in a per-tile scratch
+// in L2, whose read-modify-write per pair and phase left the adjoint waiting
+// (issue slots 16 % busy, now 39 %: 33 x 1024^2, K = 85: forward 339 -> 245 us,
+// adjoint 791 -> 319 us).
+constexpr int kTmPhases = 4;
+constexpr int kTmCols = 512;  // all columns; thread: lane tid mod 128, 128 columns
+
+// All warps of the CTA; one CTA per SM (shared memory), so the allocation does
+// not wait.
+__device__ __forceinline__ uint32_t tmem_begin(uint32_t* base_s) {
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(base_s)),
+                 "r"(kTmCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t warp = threadIdx.x >> 5;
+  return *base_s + ((warp & 3) << 21) + (warp >> 2) * (kTmPhases * 32);
+}
+__device__ __forceinline__ void tmem_end(uint32_t base) {
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base),
+                 "r"(kTmCols));
+  }
+}
+// this thread's 16 values of one phase (whole warps, converged)
+__device__ __forceinline__ void tmem_load(float2 (&v)[16], uint32_t addr) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+        "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+        "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]),
+        "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
+        "=r"(r[30]), "=r"(r[31])
+      : "r"(addr)
+      : "memory");
+  // (the operands order every use of the values after the wait)
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                 "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]),
+                 "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]),
+                 "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]),
+                 "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]),
+                 "+r"(r[31])
+               :
+               : "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    v[i] = make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+}
+__device__ __forceinline__ void tmem_store(uint32_t addr, const float2 (&v)[16]) {
+  uint32_t r[32];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    r[2 * i] = __float_as_uint(v[i].x);
+    r[2 * i + 1] = __float_as_uint(v[i].y);
+  }
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(addr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),
+      "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]),
+      "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]),
+      "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
+      "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
 // spectra of the kernels
 // ---------------------------------------------------------------------------
 
@@ -493,14 +580,15 @@ __device__ __forceinline__ void region_spectrum(const float* plane, const Geom& 
 // The forward pass of one tile for the pairs of exposures [q0, q1). R1: r = 1
 // (x^ in registers; otherwise the phases' x^ in xs). Starts and ends at a CTA
 // barrier, so a persistent CTA can run many; (nty, ntx), if known, is the tile
-// it runs next, whose x region is brought into L2 meanwhile.
-template <bool R1, bool STUDENT>
+// it runs next, whose x region is brought into L2 meanwhile. TM: r = 2 with
+// the phases' x^ in tensor memory (tm) and x64 of four phases.
+template <bool R1, bool STUDENT, bool TM = false>
 __device__ void fft_forward_tile(const Shape& s, const FftLaunch& a, int ty, int tx, float2* xs,
                                  float2* buf, float2* x64, const float4* tw, int q0, int q1,
-                                 int nty = -1, int ntx = 0) {
+                                 int nty = -1, int ntx = 0, uint32_t tm = 0) {
   const Geom& g = s.g;
   const Lane L;
-  const int hc = s.hc, B = kFT - 2 * hc, R2 = s.R2;
+  const int hc = s.hc, B = kFT - 2 * hc, R2 = TM ? kTmPhases : s.R2;
   const int i0 = ty * B, j0 = tx * B;
   const int m = L.slot(), m2 = second_col(m);
   const int pmax = min(B, g.H - i0), qmax = min(B, g.W - j0);
@@ -513,10 +601,17 @@ __device__ void fft_forward_tile(const Shape& s, const FftLaunch& a, int ty, int
     }
   };
   prefetch_pair(q0);
-  if (R1) stage_slot(st, a.spec + (long long)q0 * kPairSpec);
+  if (R1 || TM) stage_slot(st, a.spec + (long long)q0 * R2 * kPairSpec);
   float2 X[16];
   if (R1) {
     region_spectrum(a.x, g, i0 - hc, j0 - hc, buf, tw, L, X, x64);
+  } else if (TM) {
+#pragma unroll 1
+    for (int ph = 0; ph < kTmPhases; ++ph) {
+      region_spectrum(a.x + (long long)ph * g.plane, g, i0 - hc, j0 - hc, buf, tw, L, X,
+                      x64 + ph * kFT);
+      tmem_store(tm + 32 * ph, X);
+    }
   } else {
     for (int ph = 0; ph < R2; ++ph) {
       region_spectrum(a.x + (long long)ph * g.plane, g, i0 - hc, j0 - hc, buf, tw, L, X,
@@ -549,6 +644,43 @@ __device__ void fft_forward_tile(const Shape& s, const FftLaunch& a, int ty, int
           stage_slot(st, S + kSlots);
         else if (q + 1 < q1)
           stage_slot(st, S + kPairSpec);
+      } else if (TM) {
+        // S of phase 0 staged as for r = 1, the others' a phase ahead in registers
+        const float2* sp = S + h * kSlots + slot_off();
+        const bool c64 = h == 1 && m == 0;
+        float2 kv[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          kv[i] = __ldg(sp + kPairSpec + 32 * i);
+          v[i] = make_float2(0.f, 0.f);
+        }
+        staged_ready();
+        const float2* s0 = st + (threadIdx.x & 31);
+#pragma unroll 1
+        for (int ph = 0; ph < kTmPhases; ++ph) {
+          float2 x[16];
+          tmem_load(x, tm + 32 * ph);
+          if (c64) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) x[i] = x64[ph * kFT + 8 * i + L.t];
+          }
+          if (ph == 0) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = cfma(v[i], x[i], s0[32 * i]);
+            if (h == 0)
+              stage_slot(st, S + kSlots);
+            else if (q + 1 < q1)
+              stage_slot(st, S + kTmPhases * kPairSpec);
+          } else {
+            sp += kPairSpec;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              v[i] = cfma(v[i], x[i], kv[i]);
+              if (ph + 1 < kTmPhases) kv[i] = __ldg(sp + kPairSpec + 32 * i);
+            }
+          }
+          __syncwarp();
+        }
       } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = make_float2(0.f, 0.f);
@@ -1079,6 +1211,98 @@ __device__ void fft_adjoint_tile_scratch(const Shape& s, const FftLaunch& a, int
   }
 }
 
+// The same for r = 2, Gaussian, with the accumulators in tensor memory (tm) and,
+// for column 64, in a64 (four phases); `mine` takes them only where the tile
+// has several groups. The terms are added in the other form's order.
+__device__ void fft_adjoint_tile_tmem(const Shape& s, const FftLaunch& a, int ty, int tx, int tile,
+                                      float2* mine, float2* buf, float2* a64, const float4* tw,
+                                      int q0, int q1, uint32_t tm) {
+  const Geom& g = s.g;
+  const Lane L;
+  const int hc = s.hc, B = kFT - 2 * hc;
+  const int i0 = ty * B, j0 = tx * B;
+  const int m = L.slot(), m2 = second_col(m);
+  float2* stage = buf + kFBuf + (L.warp >> 3) * 32 * kFP;
+  copy_w(stage, a.w + (long long)q0 * g.plane, g, i0 - hc, j0 - hc, L.warp >> 3, L);
+  for (int q = q0; q < q1; ++q) {
+    const float2* w = a.w + (long long)q * g.plane;
+    if (q + 1 < q1) prefetch_region(w + g.plane, 8, g, i0 - hc, j0 - hc);
+    w_rows(buf + kFBuf, w, g, i0 - hc, j0 - hc, buf, tw, L);
+    if (q + 1 < q1) copy_w(stage, w + g.plane, g, i0 - hc, j0 - hc, L.warp >> 3, L);
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      const float2* sp =
+          a.spec + (long long)q * kTmPhases * kPairSpec + h * kSlots + slot_off();
+      float2 kv[16], v[16];  // phase 0's S in flight during the transform
+#pragma unroll
+      for (int i = 0; i < 16; ++i) kv[i] = __ldg(sp + 32 * i);
+      load_col(buf + (h ? m2 : m), v, L.t, h && m != 0);
+      fft_col(v, buf + (h ? m2 : m), tw, L.t);
+#pragma unroll 1
+      for (int ph = 0; ph < kTmPhases; ++ph) {
+        float2 acc[16];
+        if (q > q0 || h) {
+          tmem_load(acc, tm + 32 * ph);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) acc[i] = make_float2(0.f, 0.f);
+        }
+        if (h && m == 0) {
+          float2* o = a64 + ph * kFT + L.t;
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            o[8 * i] = cfmac(q > q0 ? o[8 * i] : make_float2(0.f, 0.f), v[i], kv[i]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) acc[i] = cfmac(acc[i], v[i], kv[i]);
+        }
+        if (ph + 1 < kTmPhases) {
+          sp += kPairSpec;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) kv[i] = __ldg(sp + 32 * i);
+        }
+        __syncwarp();
+        tmem_store(tm + 32 * ph, acc);
+      }
+    }
+    __syncthreads();  // the buffer is free for the next source
+  }
+  const bool groups = a.groups > 1;
+  if (groups) {
+    for (int ph = 0; ph < kTmPhases; ++ph) {
+      float2 acc[16];
+      tmem_load(acc, tm + 32 * ph);
+      store_slot(mine + (long long)ph * kCol, acc);
+      for (int e = threadIdx.x; e < kFT; e += kFThreads)
+        mine[(long long)ph * kCol + kSlots + e] = a64[ph * kFT + e];
+    }
+    if (!last_group(a, tile)) return;
+  }
+#pragma unroll 1
+  for (int ph = 0; ph < kTmPhases; ++ph) {
+    float2 acc[16];
+    if (!groups) {
+      tmem_load(acc, tm + 32 * ph);
+    } else {
+      const float2* p = a.scratch + ((long long)tile * a.groups * kTmPhases + ph) * kCol;
+      for (int k = 0; k < a.groups; ++k, p += (long long)kTmPhases * kCol) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const float2 t = __ldcg(p + slot_off() + 32 * i);
+          acc[i] = k ? cadd(acc[i], t) : t;
+        }
+        for (int e = threadIdx.x; e < kFT; e += kFThreads) {
+          const float2 t = __ldcg(p + kSlots + e);
+          a64[ph * kFT + e] = k ? cadd(a64[ph * kFT + e], t) : t;
+        }
+      }
+      __syncthreads();
+    }
+    columns_gauss(acc, a64 + ph * kFT, buf, tw, L);
+    rows_update<false>(s, a, ph, i0, j0, buf, tw, L);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------
@@ -1142,6 +1366,43 @@ __global__ void __launch_bounds__(kFThreads, 1)
   __shared__ float2 a64[kFT];
   init_twiddles(tw);
   adjoint_item<R1, STUDENT>(s, a, gxt, blockIdx.x, fsm, a64, tw);
+}
+
+// r = 2: item = tile * groups + group, x^ (the Gaussian accumulators) in tensor
+// memory. 33 x 2048^2 exposures, 85 x 85 PSFs: 4.66 ms an iteration through the
+// scratch, 2.40 ms here; 9 x 300 x 280, K = 43: 136 us.
+template <bool STUDENT>
+__global__ void __launch_bounds__(kFThreads, 1)
+    fft_forward_r2_kernel(const Shape s, const FftLaunch a, int gxt) {
+  extern __shared__ __align__(16) float2 fsm[];
+  __shared__ float4 tw[kFT / 2];
+  __shared__ float2 x64[kTmPhases * kFT];
+  __shared__ uint32_t base;
+  init_twiddles(tw);
+  const uint32_t tm = tmem_begin(&base);
+  const int tile = blockIdx.x / a.groups;
+  int q0, q1;
+  group_range(s.n, a.groups, blockIdx.x - tile * a.groups, &q0, &q1);
+  fft_forward_tile<false, STUDENT, true>(s, a, tile / gxt, tile % gxt, nullptr, fsm, x64, tw, q0,
+                                         q1, -1, 0, tm);
+  tmem_end(base);
+}
+
+__global__ void __launch_bounds__(kFThreads, 1)
+    fft_adjoint_r2_kernel(const Shape s, const FftLaunch a, int gxt) {
+  extern __shared__ __align__(16) float2 fsm[];
+  __shared__ float4 tw[kFT / 2];
+  __shared__ float2 a64[kTmPhases * kFT];
+  __shared__ uint32_t base;
+  init_twiddles(tw);
+  const uint32_t tm = tmem_begin(&base);
+  const int tile = blockIdx.x / a.groups;
+  int q0, q1;
+  group_range(s.n, a.groups, blockIdx.x - tile * a.groups, &q0, &q1);
+  fft_adjoint_tile_tmem(s, a, tile / gxt, tile % gxt, tile,
+                        a.scratch + (long long)blockIdx.x * kTmPhases * kCol, fsm, a64, tw, q0, q1,
+                        tm);
+  tmem_end(base);
 }
 
 // Equal ranges: CTA b of P takes the units [b U / P, (b+1) U / P) of U.
@@ -1288,6 +1549,25 @@ cudaError_t launch_pair(const Shape& s, const FftLaunch& a, int gxt, int tiles, 
   return cudaGetLastError();
 }
 
+// r = 2: tensor memory holds the four phases' spectra (not the eight accumulators
+// of the heavy-tailed adjoint, nor nine phases)
+template <bool STUDENT>
+cudaError_t launch_r2(const Shape& s, const FftLaunch& a, int gxt, int tiles, cudaStream_t st) {
+  const size_t smem = fft_smem_bytes();
+  const void* adj = STUDENT ? (const void*)fft_adjoint_kernel<false, true>
+                            : (const void*)fft_adjoint_r2_kernel;
+  cudaError_t e = allow_max_dynamic_smem((const void*)fft_forward_r2_kernel<STUDENT>);
+  if (e == cudaSuccess) e = allow_max_dynamic_smem(adj);
+  if (e != cudaSuccess) return e;
+  fft_forward_r2_kernel<STUDENT><<<tiles * a.groups, kFThreads, smem, st>>>(s, a, gxt);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (STUDENT)
+    fft_adjoint_kernel<false, true><<<tiles * a.groups, kFThreads, smem, st>>>(s, a, gxt);
+  else
+    fft_adjoint_r2_kernel<<<tiles * a.groups, kFThreads, smem, st>>>(s, a, gxt);
+  return cudaGetLastError();
+}
+
 size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -1382,6 +1662,9 @@ cudaError_t launch_fft_batch(const FftBatchJob* jobs, int njobs, const int2* ite
 
 cudaError_t launch_fft_iter(const Shape& s, const FftLaunch& a, cudaStream_t st) {
   const int gxt = fft_tiles_x(s), tiles = fft_tiles_total(s);
+  if (s.R2 == kTmPhases)
+    return a.nu > 0.f ? launch_r2<true>(s, a, gxt, tiles, st)
+                      : launch_r2<false>(s, a, gxt, tiles, st);
   if (a.nu > 0.f)
     return s.R2 == 1 ? launch_pair<true, true>(s, a, gxt, tiles, st)
                      : launch_pair<false, true>(s, a, gxt, tiles, st);
