@@ -41,14 +41,18 @@ TILE_SHAPES = {"64": 1, "48": 2, "32": 3}
 TILE_NAMES = {1: "64 x 128 tiles, 4 x 16 outputs per thread",
               2: "48 x 128 tiles, 3 x 16 outputs per thread",
               3: "32 x 128 tiles, 2 x 16 outputs per thread"}
-# kernels one emd_iterate(ctx, 1) call launches: the halo-exchange (or
-# CTA-pair) kernel (FP32); the x split and the tensor-core forward and adjoint
+# kernels one emd_iterate(ctx, 1) call launches: direct_form() for FP32; the
+# CTA-pair kernel (FP32_PAIR); the x split and the tensor-core forward and adjoint
 # kernels (BF16 modes); the x maximum, the power-of-two scales, the split and
 # the two tensor-core kernels (FP16 modes); the FFT forward and adjoint kernels
-LAUNCHES_PER_STEP = {"fp32": 1, "fp32_pair": 1, "bf16": 3, "split_bf16": 3, "fp16": 5,
+LAUNCHES_PER_STEP = {"fp32_pair": 1, "bf16": 3, "split_bf16": 3, "fp16": 5,
                      "split_fp16": 5, "fft": 2}
 # sources whose change invalidates a committed DRAM-traffic record, per kernel
 KERNEL_SOURCES = {
+    "taps": ["paper_2302_05804_gb300/csrc/emd_taps.cu",
+             "paper_2302_05804_gb300/csrc/emd_taps.cuh",
+             "paper_2302_05804_gb300/csrc/emd_corr.cuh",
+             "paper_2302_05804_gb300/csrc/emd_internal.cuh"],
     "halo": ["paper_2302_05804_gb300/csrc/emd_halo.cu",
              "paper_2302_05804_gb300/csrc/emd_halo.cuh",
              "paper_2302_05804_gb300/csrc/emd_corr.cuh",
@@ -125,10 +129,31 @@ def tc_executed_flops(H, W, n, K, r, nprod):
     return tiles * n * r * r * Kc * nprod * 2 * (128 * 128 * Kd) * 2
 
 
+def direct_form(H, W, n, K, r, nu, tile_shape):
+    """(kernel names, launches per iteration) of the FP32 direct iteration: the
+    library's rule (direct_plan in csrc/emd_taps.cu); a fixed tile shape runs
+    the halo-exchange kernel."""
+    hc = ((K - 1) // 2 + r - 1) // r
+    Kc = 2 * hc + 1
+    KP = (Kc + 3) // 4 * 4
+    T = -(-W // 128) * -(-H // 64)
+    cap = 7600 // (Kc * KP) // (r * r) if Kc >= 5 else 0
+    taps = min(cap, n, max(4, 8192 // T))
+    if not tile_shape and taps > 0 and T * taps >= 500:
+        parts = T * r * r < 4 * 152
+        per = 1 + (r * r if parts else 0)
+        chunk = min(taps, max(taps, 2) * per // (2 * per)) if nu > 0 else taps
+        names = "taps_forward_kernel + taps_adjoint_kernel" + (" + taps_sum_kernel" if parts else "")
+        return names, -(-n // chunk) * (3 if parts else 2)
+    if not tile_shape and T * n < 4000 and T < 500:
+        return "split_kernel", 1
+    return "halo_kernel", 1
+
+
 def fft_flops(H, W, n, K, r, nu):
     """flops one FFT-form iteration runs: 128^2 real transforms (2.5 N log2 N
-    each, N = 128^2) on overlap-save tiles of 128 - 2 hc outputs, and the
-    spectrum products. Forward: R2 + n transforms per tile; adjoint: n + R2,
+    each, N = 128^2; two share one complex transform) on overlap-save tiles of
+    128 - 2 hc outputs, and the spectrum products. Forward: R2 + n transforms per tile; adjoint: n + R2,
     or 2 n + 2 R2 with the heavy-tailed numerator planes."""
     hc = ((K - 1) // 2 + r - 1) // r
     B = 128 - 2 * hc
@@ -190,7 +215,8 @@ def variant_roofline(name, p, launch_s, peak32, peak32_src, sms):
     ach = flops / launch_s / 1e12
     return {"bound": "alu", "achieved": ach, "peak": peak32, "unit": "TFLOP/s",
             "frac": ach / peak32, "peak_source": peak32_src,
-            "kernel": "fused_kernel" if name == "fp32_pair" else "halo_kernel"}
+            "kernel": "fused_kernel" if name == "fp32_pair" else
+                      direct_form(p.H, p.W, p.n, p.K, p.r, nu, None)[0]}
 
 
 def kernel_source_hash(kernel):
@@ -531,7 +557,7 @@ def run_ours(args):
             torch.cuda.synchronize()
     tile = d.tile_shape() if prec == 0 else None
 
-    # timed region: K steps, one fused-kernel launch each, events per step
+    # timed region: K steps of one iteration each, events per step
     ev = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps + 1)]
     sampler = ClockSampler(local)
     sampler.start()
@@ -572,16 +598,18 @@ def run_ours(args):
                     "fft_tflop_per_iteration": fl / 1e12}
     elif prec in (0, 6):
         peak = peak32
-        kern = "halo" if prec == 0 else "fused"
+        form = direct_form(p.H, p.W, p.n, p.K, p.r, args.nu, args.tile_shape)[0]
+        kern = "fused" if prec == 6 else "halo" if form == "halo_kernel" else "taps"
         # the committed DRAM records are of the Gaussian instances
         traffic = committed_traffic(kern, args.workload) if args.nu == 0 else None
         roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak, "traffic": traffic,
-                    "kernel": {"halo": "halo_kernel (FP32 FMA, persistent, w ring in L2)",
+                    "kernel": {"taps": form + " (FP32 FMA)",
+                               "halo": "halo_kernel (FP32 FMA, persistent, w ring in L2)",
                                "fused": "fused_kernel (FP32 FMA, CTA pairs)"}[kern] +
                               (" heavy-tailed instance" if args.nu > 0 else ""),
                     "peak_source": peak32_src}
-        if prec == 0:
+        if kern == "halo":
             how = ("fixed by --tile-shape" if args.tile_shape else
                    "autotuned" if tile[1] else "autotuner undecided")
             roofline["tile"] = f"{TILE_NAMES[tile[0]]} ({how})"
@@ -682,7 +710,9 @@ def run_ours(args):
             "data": "synthetic",
             "config": config_of(args), "roofline": roofline, "cpu_baseline": cpu,
             "e2e": e2e,
-            "gpu_launches": args.steps * LAUNCHES_PER_STEP[args.precision] *
+            "gpu_launches": args.steps *
+                            (direct_form(p.H, p.W, p.n, p.K, p.r, args.nu, args.tile_shape)[1]
+                             if args.precision == "fp32" else LAUNCHES_PER_STEP[args.precision]) *
                             (2 if args.nu > 0 and args.precision == "fp32_pair" else 1),
             "clocks": clocks,
             "serving": serving, "serving_direct_fp32": serving_direct, "psf_fit": psf_fit,

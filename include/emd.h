@@ -124,7 +124,8 @@ int emd_set_x(emd_ctx *ctx, const float *x0);
 
 /* Run k >= 0 iterations of Eq. (2) on the current iterate (stream-ordered,
  * asynchronous). A bounded device-side wait that gives up (the FP32
- * halo-exchange kernel's dependency waits; the FFT form's split launch,
+ * halo-exchange kernel's dependency waits; the grid barriers of the FP32
+ * form for small images, a cooperative launch; the FFT form's split launch,
  * where part of a tile waits for the part before it) sets the context's
  * error word: the next emd_get_x or emd_loglik returns EMD_ETIMEOUT, and the
  * iterate is then not valid (set it again with emd_set_x); the context's
@@ -161,20 +162,26 @@ int emd_loglik_chi2(emd_ctx *ctx, double *out, double *chi2);
  * EMD_PREC_FFT_FP32 computes the forward model and the adjoint of each
  * iteration by FP32 FFTs (overlap-save: output tiles of 128 - 2 hc pixels,
  * hc = floor(((K-1)/2 + r - 1) / r), transformed as 128 x 128 real tiles
- * of the polyphase planes); it needs n extra exposure planes of device
- * memory for the weighted model images u_t z_t and, for r > 1, a per-tile
- * scratch of r^2 spectra (66.5 KB each), allocated on first selection.
- * EMD_PREC_FP32 (Gaussian noise) runs one persistent kernel per iteration
- * that computes each pixel's forward model once and passes the weighted
- * model images u_t z_t between 64 x 128 tiles through a ring of tile
+ * of the polyphase planes); it needs n extra exposure planes (n + 1
+ * for odd n) of device memory for the weighted model images u_t z_t and, for
+ * r > 1, a per-tile scratch of r^2 spectra (66.5 KB each), allocated on first
+ * selection.
+ * EMD_PREC_FP32 runs, per chunk of exposures, a forward launch (weighted model
+ * images u_t z_t into work planes of the context, which emd_ctx_bytes counts:
+ * at most four for large images) and an adjoint launch, whose kernels' taps
+ * travel in the launch parameters; images of a few tiles run (tile, exposure)
+ * items with grid barriers, many iterations per cooperative launch (about 2 ms
+ * of them). PSFs too large for the launch parameters (r^2 kernels above 30 KB)
+ * and contexts with a fixed tile shape (emd_set_tile_shape) run one persistent
+ * kernel per iteration that passes u_t z_t between tiles through a ring of tile
  * buffers in device memory (about 1030 tiles of 32 KB at 4096^2, fewer for
  * smaller images; emd_ctx_bytes_precision counts them), allocated at the
- * first such iteration. EMD_PREC_FP32_PAIR gives the same iterates bit for
- * bit from the kernel that keeps u_t z_t in the shared memory of a CTA
- * pair per tile and recomputes the forward model on a 2 hc halo around it
- * (no extra memory, 1.48x the multiply-adds at K = 43). emd_loglik
- * computes the forward model once per pixel in every mode except
- * EMD_PREC_FP32_PAIR. */
+ * first such iteration; batches and emd_iterate_streaming run it too.
+ * EMD_PREC_FP32_PAIR gives the same iterates bit for bit from the kernel that
+ * keeps u_t z_t in the shared memory of a CTA pair per tile and recomputes the
+ * forward model on a 2 hc halo around it (no extra memory, 1.48x the
+ * multiply-adds at K = 43). emd_loglik computes the forward model once per
+ * pixel in every mode except EMD_PREC_FP32_PAIR. */
 int emd_set_precision(emd_ctx *ctx, int mode);
 
 /*
@@ -208,13 +215,16 @@ enum emd_noise {
 };
 int emd_set_noise(emd_ctx *ctx, int model, double nu);
 
-/* Tile shape of the FP32 halo-exchange iteration (EMD_PREC_FP32). Its 128
+/* Tile shape of the FP32 halo-exchange iteration (EMD_PREC_FP32; setting one
+ * selects that kernel). Its 128
  * threads compute a tile of rows x 128 pixels, each thread a (rows/16) x 16
  * block of outputs:
  *   EMD_TILE_64         64 rows, two CTAs per SM
  *   EMD_TILE_48         48 rows, three CTAs per SM (at most 168 registers)
  *   EMD_TILE_32         32 rows, four CTAs per SM where the shared memory allows
- * EMD_TILE_AUTO (the default) lets the autotuner choose: the first
+ * EMD_TILE_AUTO (the default) takes the launch forms described at
+ * emd_set_precision where they apply (nothing to choose: emd_get_tile_shape then
+ * says EMD_TILE_64, decided); else the autotuner chooses: the first
  * iterations of a problem shape (H, W, n, K, r, noise model) not seen before
  * in this process run each candidate twice, timed with CUDA events on the
  * context's stream and read without blocking at later calls, and the

@@ -1,7 +1,7 @@
 // emd_direct.cu -- FP32 direct-convolution kernels of the EM update (Sec. 2,
 // Eq. (2)), one GPU, sm_103a.
 //
-// The hot kernel (fused_kernel) computes, for one 128 x 128 tile of the
+// fused_kernel (EMD_PREC_FP32_PAIR) computes, for one 128 x 128 tile of the
 // latent grid and all exposures t in ascending order,
 //     w_t = u_t . (F_t x)        on the tile plus a halo of hc pixels
 //     Den += F_t^T w_t            on the tile

@@ -1,5 +1,8 @@
 // emd_halo.cu -- the FP32 direct EM iteration of Sec. 2, Eq. (2) (Eq. (3)
-// for r > 1) as one persistent kernel over two kinds of work items:
+// for r > 1) as one persistent kernel over two kinds of work items (full
+// iterations of a context run in emd_taps.cu unless their kernels are too large
+// for its launches or the tile shape is fixed; streaming passes and batches
+// run here):
 //
 //   forward item (t, tile)   w_t = u_t . (F_t x) on the 64 x 128 tile,
 //                            stored in one slot of a ring of tile buffers

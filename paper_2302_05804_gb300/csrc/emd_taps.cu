@@ -9,15 +9,20 @@
 // the vector registers, and the loop runs at 68-72 TFLOP/s of the derived
 // 80.5 (K = 43, 64 x 128 tiles), against 55 with the taps in shared memory,
 // whose limit is the dispatch stall of FMAs with three register operands.
-// 30 KB of parameters hold 4 kernels of 43 x 43; Den is read and written
-// once per exposure as in halo_kernel.
+// 30 KB of parameters hold 4 kernels of 43 x 43. Large images add each
+// exposure to Den as it is done; smaller ones keep a chunk's sums in work
+// planes and a third launch adds them in exposure order, so that exposures run
+// side by side. 4096^2 x 33, K = 43: 78.8 ms an iteration in halo_kernel,
+// 62.8 here (0.81 of the derived FP32 peak); bound by the FMA pipe, 44 taps a
+// row for 43, and each launch's last wave.
 //
 // Split form (images of a few tiles). halo_kernel adds the exposures of a
 // tile one after the other, so a 128 x 128 image keeps 2 of 152 SMs busy. Here
 // (tile, exposure) items are independent: every exposure's adjoint sum goes
 // to a work plane of its own and the last CTA to finish a tile adds the planes
 // in exposure order. One cooperative launch runs many iterations, two
-// grid barriers each; tiles shrink with the image.
+// grid barriers each; tiles shrink with the image. Bound by barriers and latency
+// (128 x 128 x 4, K = 15: 104 -> 32 us an iteration).
 //
 // Both give halo_kernel's iterates bit for bit: every output's taps are
 // summed in the same order (emd_corr.cuh), each exposure's adjoint sum starts

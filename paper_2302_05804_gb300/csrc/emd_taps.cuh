@@ -34,7 +34,7 @@ int tap_bank_kernels(const Shape& s);
 struct DirectLaunch {
   FusedArgs a;      // x, xn, u, y, kf, ka, N, Nw, Den, err, nu
   float* work;      // plan.planes planes, zero outside the image
-  int* counters;    // split / parts: zero between launches (direct_counter_ints of them)
+  int* counters;    // split: zero between launches (direct_counter_ints of them)
 };
 int direct_counter_ints(const Shape& s);
 
