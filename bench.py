@@ -166,7 +166,8 @@ def fft_flops(H, W, n, K, r, nu):
 def fft_kernels(H, W, n, K, r, nu, sms):
     """Names of the two kernels an FFT-form iteration launches: the split
     forms (persistent, one CTA per SM) for r = 1 Gaussian with at least as
-    many tiles as SMs, else one CTA per tile."""
+    many tiles as SMs, else one CTA per tile and exposure group (for r = 2
+    their _r2 forms, with the spectra in tensor memory)."""
     hc = ((K - 1) // 2 + r - 1) // r
     B = 128 - 2 * hc
     tiles = -(-H // B) * -(-W // B)
