@@ -777,6 +777,7 @@ int emd_set_frames(emd_ctx* c, const float* y, const float* v, const float* f,
     CK(emd::launch_split_iters(s, c->plan[0], d, c->x[0], c->x[1], 1, true, c->st));
   else
     CK(emd::launch_fused(s, d.a, 1, c->part, c->st));
+  CK(emd::launch_numerator_marks(s, c->u, c->ka, c->N, c->st));
   // default strictly positive start
   double x0 = 1.0;
   if (c->su > 0.0) {

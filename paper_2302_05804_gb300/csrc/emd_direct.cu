@@ -642,6 +642,75 @@ cudaError_t launch_reduce_final(const double* part, int nblocks, int ncols, doub
 }
 
 // ---------------------------------------------------------------------------
+// numerator: telling a cancelled sum from an empty footprint
+// ---------------------------------------------------------------------------
+
+// A latent pixel whose footprint holds no valid pixel keeps its x. The direct
+// forms see that as Den = 0 exactly; the FFT form, whose Den carries a rounding
+// floor, sees it as N = +0. But N can also cancel to 0 where valid pixels do reach
+// it (terms of both signs, or data that are 0), and then x' = 0. This kernel
+// stores -0 in those pixels: equal to 0 in every comparison and sum, told apart by
+// its bits. The pixels with N = 0 are few, or lie in areas without valid pixels:
+// a tile (16 x 64 pixels, one phase) without any returns after reading N, one that
+// no valid pixel reaches after one look at its window, and in the others a warp
+// searches each pixel's footprint, exposure by exposure, up to the first hit.
+constexpr int kMarkH = 16, kMarkW = 64;
+
+__global__ void __launch_bounds__(256)
+    numerator_marks_kernel(const Shape s, const float* __restrict__ u,
+                           const float* __restrict__ ka, float* __restrict__ N) {
+  __shared__ int list[kMarkH * kMarkW];
+  __shared__ int count;
+  const Geom& g = s.g;
+  const int gx = (g.W + kMarkW - 1) / kMarkW, phi = blockIdx.y;
+  const int i0 = blockIdx.x / gx * kMarkH, j0 = blockIdx.x % gx * kMarkW;
+  float* Np = N + (long long)phi * g.plane + (long long)(g.B + i0) * g.P + g.B + j0;
+  if (threadIdx.x == 0) count = 0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < kMarkH * kMarkW; e += blockDim.x) {
+    const int p = e / kMarkW, q = e % kMarkW;
+    if (i0 + p < g.H && j0 + q < g.W && __float_as_uint(Np[(long long)p * g.P + q]) == 0u)
+      list[atomicAdd(&count, 1)] = e;
+  }
+  __syncthreads();
+  const int total = count;
+  if (total == 0) return;
+  // the window starts hc rows and columns before the tile (border 2 hc); past
+  // the image the padded planes hold u = 0
+  const float* win = u + (long long)(i0 + s.hc) * g.P + j0 + s.hc;
+  const int rows = kMarkH + 2 * s.hc, cols = kMarkW + 2 * s.hc;
+  int any = 0;
+  for (int t = 0; t < s.n && !any; ++t) {
+    bool hit = false;
+    for (int e = threadIdx.x; e < rows * cols; e += blockDim.x)
+      hit |= win[t * g.plane + (long long)(e / cols) * g.P + e % cols] > 0.f;
+    any = __syncthreads_or(hit);
+  }
+  if (!any) return;
+  const int lane = threadIdx.x & 31, taps = s.Kc * s.KP;
+  for (int k = threadIdx.x >> 5; k < total; k += blockDim.x >> 5) {
+    const int p = list[k] / kMarkW, q = list[k] % kMarkW;
+    bool found = false;
+    for (int t = 0; t < s.n && !found; ++t) {
+      const float* kt = ka + ((long long)t * s.R2 + phi) * taps;
+      const float* ut = win + t * g.plane + (long long)p * g.P + q;
+      bool hit = false;
+      for (int m = lane; m < taps; m += 32)
+        if (kt[m] != 0.f) hit |= ut[(long long)(m / s.KP) * g.P + m % s.KP] > 0.f;
+      found = __any_sync(0xffffffffu, hit);
+    }
+    if (found && lane == 0) Np[(long long)p * g.P + q] = -0.f;
+  }
+}
+
+cudaError_t launch_numerator_marks(const Shape& s, const float* u, const float* ka, float* N,
+                                   cudaStream_t st) {
+  const int tiles = (s.W + kMarkW - 1) / kMarkW * ((s.H + kMarkH - 1) / kMarkH);
+  numerator_marks_kernel<<<dim3(tiles, s.R2), 256, 0, st>>>(s, u, ka, N);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
 // polyphase PSF kernels: for phase (py, px) and offsets d in [-hc, hc]
 //   c[dy][dx] = sum_{s,t < r} f[r dy + s + h - py][r dx + t + h - px]
 // ka[a][b] = c[a - hc][b - hc] (adjoint, a correlation), kf = ka flipped

@@ -780,12 +780,12 @@ __device__ void fft_forward_tile(const Shape& s, const FftLaunch& a, int ty, int
 // one pixel of Eq. (2)
 __device__ __forceinline__ float update_pixel(float xo, float d, float nraw, float nt) {
   // The transform leaves a rounding floor (~1e-7 of the tile's weighted
-  // model) where the exact denominator is 0; N, from the direct kernel,
-  // is exactly 0 when no valid pixel lies in the footprint, which is
-  // then the sign of a zero denominator (x unchanged, as for Den = 0);
-  // with Student-t weights too, since u' = 0 exactly where u = 0.
+  // model) where the exact denominator is 0. The numerator is +0 exactly there,
+  // where no valid pixel lies in the footprint, and nowhere else (a sum that
+  // cancels is -0, numerator_marks_kernel): x then stays, as for Den = 0; with
+  // Student-t weights too, since u' = 0 exactly where u = 0.
   float xv = xo;
-  if (d > 0.f && nraw != 0.f) {
+  if (d > 0.f && __float_as_uint(nraw) != 0u) {
     const float nv = fmaxf(nt, 0.f);
     if (d < 1e-30f)  // denominator near zero: guarded ratio in FP64
       xv = (float)((double)xo * (double)nv / (double)d);

@@ -119,6 +119,10 @@ cudaError_t launch_build_kernels(const Shape& s, const float* f_raw, float* kf,
 cudaError_t launch_fused(const Shape& s, const FusedArgs& a, int mode, double* part,
                          cudaStream_t st);
 int fused_blocks(const Shape& s);
+// N: a sum that cancelled to 0 becomes -0; +0 stays where no valid pixel lies in the
+// footprint
+cudaError_t launch_numerator_marks(const Shape& s, const float* u, const float* ka, float* N,
+                                   cudaStream_t st);
 // one CTA waiting (bounded by `limit` polls) on an mbarrier nothing arrives on
 cudaError_t launch_wait_selftest(uint32_t limit, int* err, cudaStream_t st);
 cudaError_t launch_fill_latent(const Shape& s, float* x, float c,
