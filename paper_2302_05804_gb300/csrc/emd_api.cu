@@ -248,10 +248,10 @@ int iterate_direct(emd_ctx* c, int k) {
     const emd::DirectLaunch d = direct_launch(c);
     int done = 1;
     if (p.form == emd::kFormTaps) {
-      CK(emd::launch_taps_iter(c->s, p, d, c->hkf.data(), c->hka.data(), false, c->st));
+      CK(emd::launch_taps_iter(c->s, p, d, c->hkf.data(), c->hka.data(), c->st));
     } else {
       done = std::min(k, emd::split_iters_per_launch(c->s));
-      CK(emd::launch_split_iters(c->s, p, d, c->x[c->cur], c->x[c->cur ^ 1], done, false, c->st));
+      CK(emd::launch_split_iters(c->s, p, d, c->x[c->cur], c->x[c->cur ^ 1], done, c->st));
     }
     c->cur ^= done & 1;
     k -= done;
@@ -745,11 +745,14 @@ int emd_set_frames(emd_ctx* c, const float* y, const float* v, const float* f,
   if (tmp) CK(cudaFreeAsync(tmp, c->st));
   CK(emd::launch_reduce_final(c->part, emd::kRedBlocks, 4, c->sums, c->st));
   CK(emd::launch_build_kernels(s, c->fraw, c->kf, c->ka, c->st));
+  const size_t nk = (size_t)s.n * s.R2 * s.Kc * s.KP;
   if (c->plan[0].form == emd::kFormTaps) {
-    const size_t nk = (size_t)s.n * s.R2 * s.Kc * s.KP;
     c->hkf.resize(nk);
-    c->hka.resize(nk);
     CK(cudaMemcpyAsync(c->hkf.data(), c->kf, nk * sizeof(float), cudaMemcpyDeviceToHost, c->st));
+  }
+  const bool taps_numerator = emd::numerator_exposures(s) > 0;
+  if (taps_numerator) {
+    c->hka.resize(nk);
     CK(cudaMemcpyAsync(c->hka.data(), c->ka, nk * sizeof(float), cudaMemcpyDeviceToHost, c->st));
   }
   double h[4];
@@ -766,17 +769,16 @@ int emd_set_frames(emd_ctx* c, const float* y, const float* v, const float* f,
   c->suy = h[1];
   c->su = h[2];
   c->nvalid = h[3];
-  // numerator N = sum_t F_t^T (u_t y_t)
-  // (the Gaussian numerator whatever the noise model; the same sums in the
-  // same order from every form)
-  emd::DirectLaunch d = direct_launch(c);
-  d.a.Nw = c->N;
-  if (c->plan[0].form == emd::kFormTaps)
-    CK(emd::launch_taps_iter(s, c->plan[0], d, c->hkf.data(), c->hka.data(), true, c->st));
-  else if (c->plan[0].form == emd::kFormSplit)
-    CK(emd::launch_split_iters(s, c->plan[0], d, c->x[0], c->x[1], 1, true, c->st));
-  else
-    CK(emd::launch_fused(s, d.a, 1, c->part, c->st));
+  // numerator N = sum_t F_t^T (u_t y_t), the Gaussian one whatever the noise model;
+  // the same sums in the same order from both kernels. Scratch: the x planes, which
+  // are filled below, and Den.
+  emd::FusedArgs a = fused_args(c);
+  if (taps_numerator) {
+    float* const part[emd::kNumParts] = {c->x[0], c->x[1], c->Den};
+    CK(emd::launch_numerator(s, c->u, c->y, c->hka.data(), c->N, part, c->st));
+  } else {
+    CK(emd::launch_fused(s, a, 1, c->part, c->st));
+  }
   CK(emd::launch_numerator_marks(s, c->u, c->ka, c->N, c->st));
   // default strictly positive start
   double x0 = 1.0;

@@ -53,6 +53,30 @@ __device__ __forceinline__ void corr_taps(float (&acc)[RX], const float4 k,
   for (int c = 0; c < RX; ++c) acc[c] = fmaf(k.w, xv[c + 3], acc[c]);
 }
 
+template <int RY, int RX>
+__device__ __forceinline__ void corr_zero(float (&a)[RY][RX]) {
+#pragma unroll
+  for (int p = 0; p < RY; ++p)
+#pragma unroll
+    for (int c = 0; c < RX; ++c) a[p][c] = 0.f;
+}
+template <int RY, int RX>
+__device__ __forceinline__ void corr_add(float (&sum)[RY][RX], const float (&a)[RY][RX]) {
+#pragma unroll
+  for (int p = 0; p < RY; ++p)
+#pragma unroll
+    for (int c = 0; c < RX; ++c) sum[p][c] += a[p][c];
+}
+// where a correlation's FMAs go: the block sums where there are any, else the sums
+template <int RY, int RX>
+__device__ __forceinline__ float (&corr_target(float (&)[RY][RX], float (&block)[RY][RX]))[RY][RX] {
+  return block;
+}
+template <int RY, int RX>
+__device__ __forceinline__ float (&corr_target(float (&sum)[RY][RX], float (&)[1][1]))[RY][RX] {
+  return sum;
+}
+
 // The loop that bounds every direct-form kernel, on blocks of RY x RX outputs
 // (oy a multiple of RY; Kc odd). Tap quads outside, source rows inside: a
 // quad that a source row brings for output row 0 stays in a register for
@@ -89,15 +113,24 @@ __device__ __forceinline__ void corr4_rows(float (&acc)[4][RX], float4 (&q)[3],
   for (int j = 0; j < (U == 2 ? 2 : 3); ++j) q[j] = nw[U - 1 - j];
 }
 
-template <int RY, int RX>
-__device__ __forceinline__ void corr_tile(float (&acc)[RY][RX], const SPlane& src, int oy,
+//
+// BLOCKS (the numerator): the taps of each quad of columns are summed from zero
+// and the blocks then added. One FP32 chain of Kc^2 terms would leave an error
+// that no later iteration takes out again, since N is computed once per frame set;
+// blocks of 4 Kc leave about half of it (43 x 43, 2e-7 -> 9e-8).
+template <int RY, int RX, bool BLOCKS = false>
+__device__ __forceinline__ void corr_tile(float (&sum)[RY][RX], const SPlane& src, int oy,
                                           int ox, const float* __restrict__ ks, int KP,
                                           int Kc) {
+  static_assert(!BLOCKS || RY == 2, "blocks are summed in the two-row form only");
   const float* col = srow<RY>(src, oy) + ox;
   const int pitch = src.pitch;
+  float block[BLOCKS ? RY : 1][BLOCKS ? RX : 1];
+  float(&acc)[RY][RX] = corr_target<RY, RX>(sum, block);
   if constexpr (RY == 2) {
 #pragma unroll 1
     for (int b = 0; b < KP; b += 4) {
+      if (BLOCKS) corr_zero<RY, RX>(acc);
       const float* row = col + b;  // row s at row + s * pitch + 4 * (s / 2)
       const float* kq = ks + b;
       float xv[RX + 4];
@@ -123,6 +156,7 @@ __device__ __forceinline__ void corr_tile(float (&acc)[RY][RX], const SPlane& sr
         corr_window<RX>(xv, row);
       }
       corr_taps<RX>(acc[1], k1, xv);  // source row Kc: output row 1 only
+      if (BLOCKS) corr_add<RY, RX>(sum, acc);
     }
     return;
   }
@@ -207,13 +241,13 @@ __device__ __forceinline__ void corr_tile(float (&acc)[RY][RX], const SPlane& sr
 // grid that they straddle (the second word is the neighbour's first, an L1
 // hit): four scalar stores per word would conflict four ways. LOADS words
 // in flight per thread. CG: loads bypass L1 (the plane is written by other
-// SMs during the launch).
-template <int RY, int NT, int LOADS, bool CG>
-__device__ __forceinline__ void stage_window(const SPlane& sp, const float* base, int P, int c0,
-                                             int rows, int cols) {
+// SMs during the launch). stage_words: the words come from load(offset from the
+// row start `base` would be).
+template <int RY, int NT, int LOADS, class Load>
+__device__ __forceinline__ void stage_words(const SPlane& sp, Load&& load, int P, int c0, int rows,
+                                            int cols) {
   const int sh = c0 & 3, nq = cols >> 2;
   const int total = rows * nq;
-  base += c0 & ~3;
   for (int e0 = threadIdx.x; e0 < total; e0 += NT * LOADS) {
     float4 v[LOADS], w[LOADS];
 #pragma unroll
@@ -221,9 +255,9 @@ __device__ __forceinline__ void stage_window(const SPlane& sp, const float* base
       const int e = e0 + q * NT;
       if (e < total) {
         const int R = e / nq, m = e - R * nq;
-        const float4* p = reinterpret_cast<const float4*>(base + (long long)R * P) + m;
-        v[q] = CG ? __ldcg(p) : __ldg(p);
-        if (sh) w[q] = CG ? __ldcg(p + 1) : __ldg(p + 1);
+        const long long off = (long long)R * P + (c0 & ~3) + 4 * m;
+        v[q] = load(off);
+        if (sh) w[q] = load(off + 4);
       }
     }
 #pragma unroll
@@ -239,6 +273,18 @@ __device__ __forceinline__ void stage_window(const SPlane& sp, const float* base
       }
     }
   }
+}
+
+template <int RY, int NT, int LOADS, bool CG>
+__device__ __forceinline__ void stage_window(const SPlane& sp, const float* base, int P, int c0,
+                                             int rows, int cols) {
+  stage_words<RY, NT, LOADS>(
+      sp,
+      [base](long long off) {
+        const float4* p = reinterpret_cast<const float4*>(base + off);
+        return CG ? __ldcg(p) : __ldg(p);
+      },
+      P, c0, rows, cols);
 }
 
 // flags between CTAs

@@ -185,8 +185,9 @@ __device__ __forceinline__ void cluster_wait() {
 // caller owns the mbarrier, its phase, the timeout flag and the chi-square
 // accumulator so a persistent kernel can run many tiles per CTA pair.
 // STUDENT: heavy-tailed weights (a.nu > 0); compiled separately so that the
-// Gaussian kernel carries none of that code.
-template <bool STUDENT>
+// Gaussian kernel carries none of that code. NUM: mode 1, whose taps are summed
+// in blocks (corr_tile).
+template <bool STUDENT, bool NUM = false>
 __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, const int mode,
                                            const int i0, const int j0, const int q, float* smem,
                                            uint64_t* mbar, uint32_t& phase, bool& timed_out,
@@ -220,10 +221,10 @@ __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, c
   const int ccols = 16 * s.MXf;
 
   const int t0 = a.t0, t1 = a.t1;  // exposures of this launch, ascending
-  const bool xchg = (mode == 0 || mode == 3);  // forward, weights, halo swap, adjoint
+  const bool xchg = !NUM && (mode == 0 || mode == 3);  // forward, weights, halo swap, adjoint
   for (int t = t0; t < t1; ++t) {
     const long long tplane = (long long)t * g.plane;
-    if (mode != 1) {
+    if (!NUM) {
       // ---------------- forward: z = sum_phi kf_phi (x) x_phi -----------------
       float acc[4][16];
 #pragma unroll
@@ -348,7 +349,7 @@ __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, c
       for (int p = 0; p < 2; ++p)
 #pragma unroll
         for (int c = 0; c < 16; ++c) acc2[p][c] = 0.f;
-      if (!timed_out) corr_tile<2, 16>(acc2, ws, 2 * amy, 16 * amx, ksa, KP, Kc);
+      if (!timed_out) corr_tile<2, 16, NUM>(acc2, ws, 2 * amy, 16 * amx, ksa, KP, Kc);
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
         const int i = i0 + kHalf * q + 2 * amy + p;
@@ -363,7 +364,7 @@ __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, c
           if (t + 1 < t1) {
             a.Den[grow + c] = acc2[p][c];
           } else if (i < g.H && j < g.W) {
-            if (mode == 1 || mode == 3) {
+            if (NUM || mode == 3) {
               a.Nw[grow + c] = acc2[p][c];
             } else {
               const float d = acc2[p][c];
@@ -386,7 +387,7 @@ __device__ __forceinline__ void fused_tile(const Shape& s, const FusedArgs& a, c
   if (xchg) cluster_wait();  // [B_{n-1}]
 }
 
-template <bool STUDENT>
+template <bool STUDENT, bool NUM>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     fused_kernel(const Shape s, const FusedArgs a, const int mode, double* __restrict__ part) {
   extern __shared__ __align__(128) float smem[];
@@ -402,8 +403,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   uint32_t phase = 0;
   bool timed_out = false;
   double chi = 0.0;
-  fused_tile<STUDENT>(s, a, mode, blockIdx.y * kTile, (blockIdx.x >> 1) * kTile, q, smem, &mbar_s,
-                      phase, timed_out, chi);
+  fused_tile<STUDENT, NUM>(s, a, mode, blockIdx.y * kTile, (blockIdx.x >> 1) * kTile, q, smem,
+                           &mbar_s, phase, timed_out, chi);
   if (mode == 2) {
     const double tot = block_sum_f64(chi, red);
     if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = tot;
@@ -415,20 +416,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   }
 }
 
-template <bool STUDENT>
+template <bool STUDENT, bool NUM>
 cudaError_t launch_fused_t(const Shape& s, const FusedArgs& a, int mode, double* part,
                            cudaStream_t st) {
-  cudaError_t e = allow_max_dynamic_smem((const void*)fused_kernel<STUDENT>);
+  cudaError_t e = allow_max_dynamic_smem((const void*)fused_kernel<STUDENT, NUM>);
   if (e != cudaSuccess) return e;
   dim3 grid(2 * s.gx, s.gy), block(kThreads);
-  fused_kernel<STUDENT><<<grid, block, s.smem_fused, st>>>(s, a, mode, part);
+  fused_kernel<STUDENT, NUM><<<grid, block, s.smem_fused, st>>>(s, a, mode, part);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fused(const Shape& s, const FusedArgs& a, int mode, double* part,
                          cudaStream_t st) {
-  return a.nu > 0.f ? launch_fused_t<true>(s, a, mode, part, st)
-                    : launch_fused_t<false>(s, a, mode, part, st);
+  if (mode == 1) return launch_fused_t<false, true>(s, a, mode, part, st);
+  return a.nu > 0.f ? launch_fused_t<true, false>(s, a, mode, part, st)
+                    : launch_fused_t<false, false>(s, a, mode, part, st);
 }
 
 int fused_blocks(const Shape& s) { return 2 * s.gx * s.gy; }

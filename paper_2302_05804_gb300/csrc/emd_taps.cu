@@ -69,14 +69,18 @@ __device__ __forceinline__ void bank_rows(float (&acc)[4][16], float4 (&q)[3], f
 }
 
 // corr_tile<4, 16> with the kernel at bank.k[koff ..] (Kc odd and >= 5, rows
-// of KP floats): the same sums in the same order. Rows 0 .. 2 and Kc .. Kc + 2
+// of KP floats): the same sums in the same order, in blocks (corr_tile) too. Rows 0 .. 2 and Kc .. Kc + 2
 // are unrolled triangles, so the loop over the rows between carries no checks.
-__device__ __forceinline__ void corr_bank(float (&acc)[4][16], const SPlane& src, int oy, int ox,
+template <bool BLOCKS = false>
+__device__ __forceinline__ void corr_bank(float (&sum)[4][16], const SPlane& src, int oy, int ox,
                                           const TapBank& bank, int koff, int KP, int Kc) {
   const float* col = srow<4>(src, oy) + ox;
   const int pitch = src.pitch;
+  float block[BLOCKS ? 4 : 1][BLOCKS ? 16 : 1];
+  float(&acc)[4][16] = corr_target<4, 16>(sum, block);
 #pragma unroll 1
   for (int b = 0; b < KP; b += 4) {
+    if (BLOCKS) corr_zero<4, 16>(acc);
     const float* row = col + b;
     int ko = koff + b;
     float xv[20];
@@ -121,6 +125,7 @@ __device__ __forceinline__ void corr_bank(float (&acc)[4][16], const SPlane& src
     row += pitch;
     corr_window<16>(xv, row);
     corr_taps<16>(acc[3], q[0], xv);
+    if (BLOCKS) corr_add<4, 16>(sum, acc);
   }
 }
 
@@ -174,16 +179,6 @@ __device__ __forceinline__ void store_w(const Geom& g, const float (&acc)[RY][RX
   }
 }
 
-// w = u y on a tile's pixels inside the image
-__device__ __forceinline__ void store_uy(const Geom& g, int i0, int j0, int TH, int TW, int NT,
-                                         const float* u, const float* y, float* w) {
-  for (int e = threadIdx.x; e < TH * TW; e += NT) {
-    const int i = i0 + e / TW, j = j0 + e % TW;
-    const long long off = (long long)(g.B + i) * g.P + g.B + j;
-    if (i < g.H && j < g.W) w[off] = u[off] * y[off];
-  }
-}
-
 // one pixel of Eq. (2) (the expressions of halo_kernel)
 __device__ __forceinline__ float em_update(float xo, float d, float n) {
   float xv = xo;
@@ -207,8 +202,7 @@ __device__ __forceinline__ float em_update(float xo, float d, float n) {
 // K = 15: 32.2 -> 29.2 us an iteration).
 template <int RY, int RX, bool STUDENT>
 __device__ __forceinline__ void sum_parts(const Shape& s, const FusedArgs& a, const float* part,
-                                          int ne, int phi, int i0, int j0, bool first, bool last,
-                                          bool numerator) {
+                                          int ne, int phi, int i0, int j0, bool first, bool last) {
   constexpr int NP = STUDENT ? 2 : 1, NR = RX >= 16 ? 1 : RY;  // rows of a block
   const Geom& g = s.g;
   const long long pb = (long long)phi * g.plane, step = (long long)s.R2 * g.plane;
@@ -218,14 +212,13 @@ __device__ __forceinline__ void sum_parts(const Shape& s, const FusedArgs& a, co
     if (i0 + p0 >= g.H || j0 >= g.W) break;
     const long long off = pb + (long long)(g.B + i0 + p0) * g.P + g.B + j0;
     float d[NP][NR][RX], xo[NR][RX], nn[NR][RX];
-    const bool update = last && !numerator;
 #pragma unroll
     for (int p = 0; p < NR; ++p)
 #pragma unroll
       for (int c = 0; c < RX; ++c) {
         const long long o = off + (long long)p * g.P + c;
-        xo[p][c] = update ? __ldcg(a.x + o) : 0.f;
-        nn[p][c] = update && !STUDENT ? a.N[o] : 0.f;
+        xo[p][c] = last ? __ldcg(a.x + o) : 0.f;
+        nn[p][c] = last && !STUDENT ? a.N[o] : 0.f;
 #pragma unroll
         for (int q = 0; q < NP; ++q)
           d[q][p][c] = first ? 0.f : __ldcg((q == 0 ? a.Den : a.Nw) + o);
@@ -252,13 +245,13 @@ __device__ __forceinline__ void sum_parts(const Shape& s, const FusedArgs& a, co
       for (int c = 0; c < RX; ++c) {
         if (j0 + c >= g.W) break;
         const long long o = off + (long long)p * g.P + c;
-        if (update) {
+        if (last) {
           const float n = STUDENT ? d[NP - 1][p][c] : nn[p][c];
           a.xn[o] = em_update(xo[p][c], d[0][p][c], n);
         } else {
 #pragma unroll
           for (int q = 0; q < NP; ++q)
-            ((q == 0 && !(last && numerator)) ? a.Den : a.Nw)[o] = d[q][p][c];
+            (q == 0 ? a.Den : a.Nw)[o] = d[q][p][c];
         }
       }
     }
@@ -317,8 +310,8 @@ __device__ __forceinline__ bool last_to_arrive(int* counter, int ne, int* flag_s
 // chunk fills the SMs several times over, 64 x 64 (64 threads) otherwise, whose
 // items divide the SMs more evenly.
 template <int V> struct TapsTile;
-template <> struct TapsTile<0> { static constexpr int TH = 64, TW = 128, MINB = 3; };
-template <> struct TapsTile<1> { static constexpr int TH = 64, TW = 64, MINB = 5; };
+template <> struct TapsTile<0> { static constexpr int TH = 64, TW = 128, MINB = 3, NUMB = 2; };
+template <> struct TapsTile<1> { static constexpr int TH = 64, TW = 64, MINB = 5, NUMB = 4; };
 
 struct TapsArgs {
   FusedArgs a;      // t0, t1: all exposures of the iteration
@@ -327,7 +320,6 @@ struct TapsArgs {
   int c0, ne;       // exposures [c0, c0 + ne) of this launch
   int epi;          // exposures per forward item
   int parts;        // adjoint partials per exposure, summed by taps_sum_kernel
-  int numerator;    // the sum over the exposures goes to a.Nw as it is
   int gx, T;        // tiles per row, tiles
 };
 
@@ -408,10 +400,9 @@ __global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), 
             acc[p][2 * c + 1] = v.y + acc[p][2 * c + 1];
           }
         }
-        if (end && A.numerator) run2 = reinterpret_cast<float2*>(A.a.Nw + pb + off);
         // not the last exposure; or the heavy-tailed Den, kept for pass 1
         // (read back below by the thread that wrote it)
-        if (!end || A.numerator || (STUDENT && pass == 0)) {
+        if (!end || (STUDENT && pass == 0)) {
 #pragma unroll
           for (int c = 0; c < 8; ++c) run2[c] = make_float2(acc[p][2 * c], acc[p][2 * c + 1]);
           continue;
@@ -436,7 +427,7 @@ __global__ void __launch_bounds__(128) taps_sum_kernel(const Shape s, const Taps
   const int j = 4 * (blockIdx.x * 128 + threadIdx.x);
   if (j < s.g.W)
     sum_parts<1, 4, STUDENT>(s, A.a, A.part, A.ne, blockIdx.z, blockIdx.y, j, A.c0 == A.a.t0,
-                             A.c0 + A.ne == A.a.t1, A.numerator);
+                             A.c0 + A.ne == A.a.t1);
 }
 
 // ---------------------------------------------------------------------------
@@ -460,7 +451,6 @@ struct SplitArgs {
   int* ctrl;        // [0] barrier arrivals, [1] CTAs finished, [2] abort flag
   int* counters;    // one per (phase, tile)
   int chunk, iters;
-  int numerator;    // w = u y instead of u z; the sum goes to a.Nw as it is
   int gx, T;
 };
 
@@ -498,11 +488,6 @@ __global__ void __launch_bounds__(SplitTile<V>::TH / 2 * (SplitTile<V>::TW / Spl
         const int i0 = (k / A.gx) * TH, j0 = (k % A.gx) * TW;
         float acc[2][RX];
         zero_block(acc);
-        if (A.numerator) {
-          store_uy(g, i0, j0, TH, TW, NT, a.u + (long long)t * g.plane,
-                   a.y + (long long)t * g.plane, A.w + (long long)e * g.plane);
-          continue;
-        }
         for (int phi = 0; phi < s.R2; ++phi) {
           stage(a.x + (long long)phi * g.plane,
                 a.kf + ((long long)t * s.R2 + phi) * s.Kc * s.KP, i0, j0, true);
@@ -530,8 +515,7 @@ __global__ void __launch_bounds__(SplitTile<V>::TH / 2 * (SplitTile<V>::TW / Spl
                       A.part + (long long)((pass * ne + e) * s.R2 + phi) * g.plane);
         }
         if (last_to_arrive(A.counters + rest, ne, &flag_s))
-          sum_parts<2, RX, STUDENT>(s, a, A.part, ne, phi, i0 + 2 * my, j0 + RX * mx, first, last,
-                                    A.numerator);
+          sum_parts<2, RX, STUDENT>(s, a, A.part, ne, phi, i0 + 2 * my, j0 + RX * mx, first, last);
       }
       if (ok) ok = grid_barrier(A.ctrl, ++round, &flag_s);
     }
@@ -567,6 +551,111 @@ size_t split_smem_bytes(const Shape& s, int TH, int TW) {
 }
 
 int cdiv(int a, int b) { return (a + b - 1) / b; }
+
+// ---------------------------------------------------------------------------
+// the numerator N = sum_t F_t^T (u_t y_t)
+// ---------------------------------------------------------------------------
+
+// One adjoint pass in the taps form, its windows staged as products u y straight
+// from the planes (no work planes). It runs once per frame set, and its rounding
+// stays in every iterate: the taps are summed in blocks (corr_tile). Images whose
+// tiles do not fill the SMs run up to kNumParts + 1 exposures side by side: the
+// first adds to N in place, the others' sums go to planes that are scratch at that
+// time, and a second launch adds those in exposure order (33 x 1024^2, K = 43, set-up
+// and log-likelihood included: 6.73 ms with three such planes, 6.89 with one).
+struct NumeratorArgs {
+  const float *u, *y;     // n planes
+  float* N;               // R2 planes
+  float* part[kNumParts]; // R2 planes each
+  int c0, ne;             // exposures [c0, c0 + ne) of this launch
+  int parts;              // one exposure per blockIdx.z: 0 into N, z into part[z - 1]
+  int gx;                 // tiles per row
+};
+
+template <int V>
+__global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), TapsTile<V>::NUMB)
+    taps_numerator_kernel(const Shape s, const NumeratorArgs A,
+                          const __grid_constant__ TapBank bank) {
+  constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NY = TH / 4, NT = NY * (TW / 16);
+  extern __shared__ __align__(128) float smem[];
+  const Geom& g = s.g;
+  const SPlane sp{smem, TW + s.KP};
+  const int my = threadIdx.x % NY, mx = threadIdx.x / NY;
+  const int k = blockIdx.x, phi = blockIdx.y;
+  const int i0 = (k / A.gx) * TH, j0 = (k % A.gx) * TW;
+  const int i = i0 + 4 * my, j = j0 + 16 * mx;
+  const long long pb = (long long)phi * g.plane;
+  const int e0 = A.parts ? blockIdx.z : 0, e1 = A.parts ? e0 + 1 : A.ne;
+  for (int e = e0; e < e1; ++e) {
+    const long long row0 = (long long)(A.c0 + e) * g.plane + (long long)(i0 + s.hc) * g.P;
+    const float *u = A.u + row0, *y = A.y + row0;
+    __syncthreads();  // readers of the previous window are done
+    stage_words<4, NT, 4>(
+        sp,
+        [u, y](long long off) {
+          const float4 a = __ldg(reinterpret_cast<const float4*>(u + off));
+          const float4 b = __ldg(reinterpret_cast<const float4*>(y + off));
+          return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
+        },
+        g.P, j0 + s.hc, TH + 2 * s.hc, TW + s.KP);
+    __syncthreads();
+    float acc[4][16];
+    zero_block(acc);
+    corr_bank<true>(acc, sp, 4 * my, 16 * mx, bank, (e * s.R2 + phi) * s.Kc * s.KP, s.KP, s.Kc);
+    const bool in_place = !A.parts || e == 0;
+    if (in_place && A.c0 + e > 0) {
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+          if (i + p < g.H && j + c < g.W)
+            acc[p][c] += A.N[pb + (long long)(g.B + i + p) * g.P + g.B + j + c];
+    }
+    store_block(g, acc, i, j, (in_place ? A.N : A.part[e - 1]) + pb);
+  }
+}
+
+// N += the launch's parts in exposure order, rows of pixels by pairs
+__global__ void __launch_bounds__(128)
+    numerator_sum_kernel(const Shape s, const NumeratorArgs A) {
+  const int j = 2 * (blockIdx.x * 128 + threadIdx.x);
+  if (j >= s.g.W) return;
+  const long long off =
+      blockIdx.z * s.g.plane + (long long)(s.g.B + blockIdx.y) * s.g.P + s.g.B + j;
+  float2 v = *reinterpret_cast<const float2*>(A.N + off);
+#pragma unroll
+  for (int e = 0; e < kNumParts; ++e)
+    if (e + 1 < A.ne) {
+      const float2 t = *reinterpret_cast<const float2*>(A.part[e] + off);
+      v.x += t.x;
+      v.y += t.y;
+    }
+  A.N[off] = v.x;
+  if (j + 1 < s.g.W) A.N[off + 1] = v.y;
+}
+
+template <int V>
+cudaError_t launch_numerator_t(const Shape& s, NumeratorArgs A, int chunk, const float* hka,
+                               cudaStream_t st) {
+  constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NT = TH / 4 * (TW / 16);
+  cudaError_t e = allow_max_dynamic_smem((const void*)taps_numerator_kernel<V>);
+  if (e != cudaSuccess) return e;
+  const size_t smem = taps_smem_bytes(s, TH, TW), kfl = (size_t)s.R2 * s.Kc * s.KP;
+  A.gx = cdiv(s.W, TW);
+  const int T = A.gx * cdiv(s.H, TH);
+  TapBank bank;
+  for (A.c0 = 0; A.c0 < s.n; A.c0 += chunk) {
+    A.ne = std::min(chunk, s.n - A.c0);
+    std::copy(hka + (size_t)A.c0 * kfl, hka + (size_t)(A.c0 + A.ne) * kfl, bank.k);
+    taps_numerator_kernel<V><<<dim3(T, s.R2, A.parts ? A.ne : 1), NT, smem, st>>>(s, A, bank);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (A.parts && A.ne > 1) {
+      numerator_sum_kernel<<<dim3(cdiv(s.W, 256), s.H, s.R2), 128, 0, st>>>(s, A);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+  }
+  return cudaSuccess;
+}
 
 // The log-likelihood's data term over the chunk (Eq. (1); the Student-t term
 // with STUDENT): part[group * T + tile] (+)= sum of u (y - z)^2 in FP64 over
@@ -649,17 +738,9 @@ cudaError_t launch_chi2_t(const Shape& s, const FusedArgs& a, const float* hkf,
   return cudaSuccess;
 }
 
-// w = u y of the exposures [c0, c0 + ne) for the numerator
-__global__ void __launch_bounds__(128) uy_kernel(const Shape s, const TapsArgs A) {
-  const int k = blockIdx.x, e = blockIdx.y;
-  const long long tp = (long long)(A.c0 + e) * s.g.plane;
-  store_uy(s.g, k / s.gx * 64, k % s.gx * kTile, 64, kTile, 128, A.a.u + tp, A.a.y + tp,
-           A.w + (long long)e * s.g.plane);
-}
-
 template <int V, bool STUDENT>
 cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
-                          const float* hkf, const float* hka, bool numerator, cudaStream_t st) {
+                          const float* hkf, const float* hka, cudaStream_t st) {
   constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NT = TH / 4 * (TW / 16);
   const size_t smem = taps_smem_bytes(s, TH, TW);
   cudaError_t e = allow_max_dynamic_smem((const void*)taps_forward_kernel<V, STUDENT>);
@@ -670,7 +751,6 @@ cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunc
   A.a = h.a;
   A.w = h.work;
   A.parts = p.parts;
-  A.numerator = numerator;
   A.gx = cdiv(s.W, TW);
   A.T = A.gx * cdiv(s.H, TH);
   TapBank bank;
@@ -681,12 +761,8 @@ cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunc
     // exposures per forward item (r = 1: its window is staged once): as many
     // as still leave 16 items an SM
     A.epi = s.R2 > 1 ? 1 : std::max(1, std::min(A.ne, A.T * A.ne / (16 * kSMs)));
-    if (numerator) {
-      uy_kernel<<<dim3(s.gx * cdiv(s.H, 64), A.ne), 128, 0, st>>>(s, A);
-    } else {
-      std::copy(hkf + (size_t)c0 * kfl, hkf + (size_t)(c0 + A.ne) * kfl, bank.k);
-      taps_forward_kernel<V, STUDENT><<<A.T * cdiv(A.ne, A.epi), NT, smem, st>>>(s, A, bank);
-    }
+    std::copy(hkf + (size_t)c0 * kfl, hkf + (size_t)(c0 + A.ne) * kfl, bank.k);
+    taps_forward_kernel<V, STUDENT><<<A.T * cdiv(A.ne, A.epi), NT, smem, st>>>(s, A, bank);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     std::copy(hka + (size_t)c0 * kfl, hka + (size_t)(c0 + A.ne) * kfl, bank.k);
     taps_adjoint_kernel<V, STUDENT>
@@ -702,7 +778,7 @@ cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunc
 
 template <int V, bool STUDENT>
 cudaError_t launch_split_t(const Shape& s, const DirectPlan& p, const DirectLaunch& h, float* xa,
-                           float* xb, int iters, bool numerator, cudaStream_t st) {
+                           float* xb, int iters, cudaStream_t st) {
   constexpr int NT = SplitTile<V>::TH / 2 * (SplitTile<V>::TW / SplitTile<V>::RX);
   const size_t smem = split_smem_bytes(s, SplitTile<V>::TH, SplitTile<V>::TW);
   const void* kern = (const void*)split_kernel<V, STUDENT>;
@@ -720,7 +796,6 @@ cudaError_t launch_split_t(const Shape& s, const DirectPlan& p, const DirectLaun
   A.a.xn = xb;
   A.chunk = p.chunk;
   A.iters = iters;
-  A.numerator = numerator;
   A.w = h.work;
   A.part = h.work + (long long)(STUDENT ? 2 : 1) * p.chunk * s.g.plane;
   A.ctrl = h.counters;
@@ -742,13 +817,32 @@ int direct_counter_ints(const Shape& s) {
 }
 
 cudaError_t launch_taps_iter(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
-                             const float* hkf, const float* hka, bool numerator,
-                             cudaStream_t st) {
-  if (h.a.nu > 0.f && !numerator)
-    return p.tile == 0 ? launch_taps_t<0, true>(s, p, h, hkf, hka, false, st)
-                       : launch_taps_t<1, true>(s, p, h, hkf, hka, false, st);
-  return p.tile == 0 ? launch_taps_t<0, false>(s, p, h, hkf, hka, numerator, st)
-                     : launch_taps_t<1, false>(s, p, h, hkf, hka, numerator, st);
+                             const float* hkf, const float* hka, cudaStream_t st) {
+  if (h.a.nu > 0.f)
+    return p.tile == 0 ? launch_taps_t<0, true>(s, p, h, hkf, hka, st)
+                       : launch_taps_t<1, true>(s, p, h, hkf, hka, st);
+  return p.tile == 0 ? launch_taps_t<0, false>(s, p, h, hkf, hka, st)
+                     : launch_taps_t<1, false>(s, p, h, hkf, hka, st);
+}
+
+int numerator_exposures(const Shape& s) {
+  return s.Kc >= 5 ? std::min(s.n, tap_bank_kernels(s) / s.R2) : 0;
+}
+
+cudaError_t launch_numerator(const Shape& s, const float* u, const float* y, const float* hka,
+                             float* N, float* const (&part)[kNumParts], cudaStream_t st) {
+  NumeratorArgs A{};
+  A.u = u;
+  A.y = y;
+  A.N = N;
+  std::copy(part, part + kNumParts, A.part);
+  // the rules of direct_plan: parts where tiles and phases alone do not fill the SMs,
+  // 64 x 64 tiles for few items
+  const long long T = (long long)s.gx * cdiv(s.H, 64);
+  A.parts = T * s.R2 < 4 * kSMs;
+  const int most = numerator_exposures(s), chunk = A.parts ? std::min(most, kNumParts + 1) : most;
+  return T * chunk >= 1500 ? launch_numerator_t<0>(s, A, chunk, hka, st)
+                           : launch_numerator_t<1>(s, A, chunk, hka, st);
 }
 
 cudaError_t launch_taps_chi2(const Shape& s, const DirectPlan& p, const FusedArgs& a,
@@ -762,12 +856,12 @@ cudaError_t launch_taps_chi2(const Shape& s, const DirectPlan& p, const FusedArg
 }
 
 cudaError_t launch_split_iters(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
-                               float* xa, float* xb, int iters, bool numerator, cudaStream_t st) {
-  if (h.a.nu > 0.f && !numerator)
-    return p.tile == 0 ? launch_split_t<0, true>(s, p, h, xa, xb, iters, false, st)
-                       : launch_split_t<1, true>(s, p, h, xa, xb, iters, false, st);
-  return p.tile == 0 ? launch_split_t<0, false>(s, p, h, xa, xb, iters, numerator, st)
-                     : launch_split_t<1, false>(s, p, h, xa, xb, iters, numerator, st);
+                               float* xa, float* xb, int iters, cudaStream_t st) {
+  if (h.a.nu > 0.f)
+    return p.tile == 0 ? launch_split_t<0, true>(s, p, h, xa, xb, iters, st)
+                       : launch_split_t<1, true>(s, p, h, xa, xb, iters, st);
+  return p.tile == 0 ? launch_split_t<0, false>(s, p, h, xa, xb, iters, st)
+                     : launch_split_t<1, false>(s, p, h, xa, xb, iters, st);
 }
 
 int split_iters_per_launch(const Shape& s) {

@@ -39,13 +39,18 @@ struct DirectLaunch {
 int direct_counter_ints(const Shape& s);
 
 // One iteration with the taps form; hkf, hka: host copies of all kernels.
-// numerator: N = sum_t F_t^T (u_t y_t) into a.Nw instead.
 cudaError_t launch_taps_iter(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
-                             const float* hkf, const float* hka, bool numerator, cudaStream_t st);
-// iters iterations with the split form, x buffers xa (current) and xb (or
-// the numerator, iters = 1)
+                             const float* hkf, const float* hka, cudaStream_t st);
+// iters iterations with the split form, x buffers xa (current) and xb
 cudaError_t launch_split_iters(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
-                               float* xa, float* xb, int iters, bool numerator, cudaStream_t st);
+                               float* xa, float* xb, int iters, cudaStream_t st);
+// N = sum_t F_t^T (u_t y_t), where numerator_exposures(s) > 0 (the exposures whose
+// kernels a launch can hold); hka: a host copy of the adjoint kernels; part: scratch,
+// R2 planes each.
+constexpr int kNumParts = 3;
+int numerator_exposures(const Shape& s);
+cudaError_t launch_numerator(const Shape& s, const float* u, const float* y, const float* hka,
+                             float* N, float* const (&part)[kNumParts], cudaStream_t st);
 // The log-likelihood's data term with the taps form: *nparts partial sums
 // into part (at most max_parts, at least one per 64 x 64 tile), to be added in
 // index order.
