@@ -28,6 +28,7 @@
 // summed in the same order (emd_corr.cuh), each exposure's adjoint sum starts
 // at zero, and the sums are added in exposure order.
 #include <algorithm>
+#include <type_traits>
 
 #include "emd_corr.cuh"
 #include "emd_taps.cuh"
@@ -127,6 +128,31 @@ __device__ __forceinline__ void corr_bank(float (&sum)[4][16], const SPlane& src
     corr_taps<16>(acc[3], q[0], xv);
     if (BLOCKS) corr_add<4, 16>(sum, acc);
   }
+}
+
+// Where a launch's taps are: in its parameters (TapBank), or, for a launch that is
+// captured into a graph, in the context's arena (TapMemory), because a graph keeps
+// the parameters of its capture and would replay the PSFs of that time after a new
+// frame set. The kernel's taps then pass through shared memory (ks), as in
+// halo_kernel, and the loop runs at its rate (corr_tile; the same bits).
+struct TapMemory {
+  const float* k;
+};
+
+template <int NT>
+__device__ __forceinline__ void corr_launch(float (&acc)[4][16], const SPlane& src, int oy, int ox,
+                                            const TapBank& bank, int koff, int KP, int Kc, float*) {
+  corr_bank(acc, src, oy, ox, bank, koff, KP, Kc);
+}
+template <int NT>
+__device__ __forceinline__ void corr_launch(float (&acc)[4][16], const SPlane& src, int oy, int ox,
+                                            const TapMemory& mem, int koff, int KP, int Kc,
+                                            float* ks) {
+  __syncthreads();  // readers of the previous kernel are done
+  for (int q = threadIdx.x; q < (Kc * KP) >> 2; q += NT)
+    reinterpret_cast<float4*>(ks)[q] = __ldg(reinterpret_cast<const float4*>(mem.k + koff) + q);
+  __syncthreads();
+  corr_tile<4, 16>(acc, src, oy, ox, ks, KP, Kc);
 }
 
 // ---------------------------------------------------------------------------
@@ -313,6 +339,18 @@ template <int V> struct TapsTile;
 template <> struct TapsTile<0> { static constexpr int TH = 64, TW = 128, MINB = 3, NUMB = 2; };
 template <> struct TapsTile<1> { static constexpr int TH = 64, TW = 64, MINB = 5, NUMB = 4; };
 
+template <int V, class Taps>
+constexpr int taps_min_blocks() {
+  // taps in shared memory: halo_kernel's registers
+  return std::is_same<Taps, TapBank>::value ? TapsTile<V>::MINB : V == 0 ? 2 : 4;
+}
+
+// floats of a staged window
+__host__ __device__ inline int taps_window_floats(const Shape& s, int TH, int TW) {
+  const int rows = TH + 2 * s.hc;
+  return rows * (TW + s.KP) + 4 * ((rows + 3) / 4);
+}
+
 struct TapsArgs {
   FusedArgs a;      // t0, t1: all exposures of the iteration
   float* w;         // chunk planes (heavy-tailed: then chunk planes of w2)
@@ -323,13 +361,15 @@ struct TapsArgs {
   int gx, T;        // tiles per row, tiles
 };
 
-template <int V, bool STUDENT>
-__global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), TapsTile<V>::MINB)
-    taps_forward_kernel(const Shape s, const TapsArgs A, const __grid_constant__ TapBank bank) {
+template <int V, bool STUDENT, class Taps>
+__global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16),
+                                  taps_min_blocks<V, Taps>())
+    taps_forward_kernel(const Shape s, const TapsArgs A, const __grid_constant__ Taps bank) {
   constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NY = TH / 4, NT = NY * (TW / 16);
   extern __shared__ __align__(128) float smem[];
   const Geom& g = s.g;
   const SPlane sp{smem, TW + s.KP};
+  float* ks = smem + taps_window_floats(s, TH, TW);  // TapMemory
   const int my = threadIdx.x % NY, mx = threadIdx.x / NY;
   const int grp = blockIdx.x / A.T, k = blockIdx.x - grp * A.T;
   const int i0 = (k / A.gx) * TH, j0 = (k % A.gx) * TW;
@@ -345,7 +385,8 @@ __global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), 
             TH + 2 * s.hc, TW + s.KP);
         __syncthreads();
       }
-      corr_bank(acc, sp, 4 * my, 16 * mx, bank, (e * s.R2 + phi) * s.Kc * s.KP, s.KP, s.Kc);
+      corr_launch<NT>(acc, sp, 4 * my, 16 * mx, bank, (e * s.R2 + phi) * s.Kc * s.KP, s.KP, s.Kc,
+                      ks);
     }
     const long long tp = (long long)(A.c0 + e) * g.plane;
     store_w<4, 16, STUDENT>(g, acc, i0 + 4 * my, j0 + 16 * mx, A.a.u + tp, A.a.y + tp, A.a.nu,
@@ -355,13 +396,15 @@ __global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), 
 
 // blockIdx.x: tile, y: phase; z: exposure of the chunk (parts) or one CTA
 // running all of them in order, adding each to Den (and N') in global memory
-template <int V, bool STUDENT>
-__global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), TapsTile<V>::MINB)
-    taps_adjoint_kernel(const Shape s, const TapsArgs A, const __grid_constant__ TapBank bank) {
+template <int V, bool STUDENT, class Taps>
+__global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16),
+                                  taps_min_blocks<V, Taps>())
+    taps_adjoint_kernel(const Shape s, const TapsArgs A, const __grid_constant__ Taps bank) {
   constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NY = TH / 4, NT = NY * (TW / 16);
   extern __shared__ __align__(128) float smem[];
   const Geom& g = s.g;
   const SPlane sp{smem, TW + s.KP};
+  float* ks = smem + taps_window_floats(s, TH, TW);  // TapMemory
   const int my = threadIdx.x % NY, mx = threadIdx.x / NY;
   const int k = blockIdx.x, phi = blockIdx.y;
   const int i0 = (k / A.gx) * TH, j0 = (k % A.gx) * TW;
@@ -379,7 +422,8 @@ __global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), 
           sp, A.w + (long long)(pass * A.ne + e) * g.plane + (long long)(i0 + s.hc) * g.P, g.P,
           j0 + s.hc, TH + 2 * s.hc, TW + s.KP);
       __syncthreads();
-      corr_bank(acc, sp, 4 * my, 16 * mx, bank, (e * s.R2 + phi) * s.Kc * s.KP, s.KP, s.Kc);
+      corr_launch<NT>(acc, sp, 4 * my, 16 * mx, bank, (e * s.R2 + phi) * s.Kc * s.KP, s.KP, s.Kc,
+                      ks);
       if (A.parts) {
         store_block(g, acc, i, j, A.part + (long long)(pass * A.ne + e) * s.R2 * g.plane + pb);
         continue;
@@ -541,8 +585,7 @@ __global__ void __launch_bounds__(SplitTile<V>::TH / 2 * (SplitTile<V>::TW / Spl
 }
 
 size_t taps_smem_bytes(const Shape& s, int TH, int TW) {
-  const int rows = TH + 2 * s.hc;
-  return ((size_t)rows * (TW + s.KP) + 4 * ((rows + 3) / 4)) * sizeof(float);
+  return (size_t)taps_window_floats(s, TH, TW) * sizeof(float);
 }
 
 size_t split_smem_bytes(const Shape& s, int TH, int TW) {
@@ -738,13 +781,23 @@ cudaError_t launch_chi2_t(const Shape& s, const FusedArgs& a, const float* hkf,
   return cudaSuccess;
 }
 
-template <int V, bool STUDENT>
+void set_taps(TapBank& bank, const float* host, const float*, size_t first, size_t count) {
+  std::copy(host + first, host + first + count, bank.k);
+}
+void set_taps(TapMemory& mem, const float*, const float* dev, size_t first, size_t) {
+  mem.k = dev + first;
+}
+
+template <int V, bool STUDENT, class Taps>
 cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
                           const float* hkf, const float* hka, cudaStream_t st) {
   constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NT = TH / 4 * (TW / 16);
-  const size_t smem = taps_smem_bytes(s, TH, TW);
-  cudaError_t e = allow_max_dynamic_smem((const void*)taps_forward_kernel<V, STUDENT>);
-  if (e == cudaSuccess) e = allow_max_dynamic_smem((const void*)taps_adjoint_kernel<V, STUDENT>);
+  const size_t smem = taps_smem_bytes(s, TH, TW) +
+                      (std::is_same<Taps, TapBank>::value ? 0 : s.Kc * s.KP * sizeof(float));
+  const auto forward = taps_forward_kernel<V, STUDENT, Taps>;
+  const auto adjoint = taps_adjoint_kernel<V, STUDENT, Taps>;
+  cudaError_t e = allow_max_dynamic_smem((const void*)forward);
+  if (e == cudaSuccess) e = allow_max_dynamic_smem((const void*)adjoint);
   if (e != cudaSuccess) return e;
   const size_t kfl = (size_t)s.R2 * s.Kc * s.KP;  // taps of one exposure
   TapsArgs A;
@@ -753,7 +806,7 @@ cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunc
   A.parts = p.parts;
   A.gx = cdiv(s.W, TW);
   A.T = A.gx * cdiv(s.H, TH);
-  TapBank bank;
+  Taps bank;
   for (int c0 = h.a.t0; c0 < h.a.t1; c0 += p.chunk) {
     A.c0 = c0;
     A.ne = std::min(p.chunk, h.a.t1 - c0);
@@ -761,12 +814,11 @@ cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunc
     // exposures per forward item (r = 1: its window is staged once): as many
     // as still leave 16 items an SM
     A.epi = s.R2 > 1 ? 1 : std::max(1, std::min(A.ne, A.T * A.ne / (16 * kSMs)));
-    std::copy(hkf + (size_t)c0 * kfl, hkf + (size_t)(c0 + A.ne) * kfl, bank.k);
-    taps_forward_kernel<V, STUDENT><<<A.T * cdiv(A.ne, A.epi), NT, smem, st>>>(s, A, bank);
+    set_taps(bank, hkf, h.a.kf, c0 * kfl, A.ne * kfl);
+    forward<<<A.T * cdiv(A.ne, A.epi), NT, smem, st>>>(s, A, bank);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    std::copy(hka + (size_t)c0 * kfl, hka + (size_t)(c0 + A.ne) * kfl, bank.k);
-    taps_adjoint_kernel<V, STUDENT>
-        <<<dim3(A.T, s.R2, p.parts ? A.ne : 1), NT, smem, st>>>(s, A, bank);
+    set_taps(bank, hka, h.a.ka, c0 * kfl, A.ne * kfl);
+    adjoint<<<dim3(A.T, s.R2, p.parts ? A.ne : 1), NT, smem, st>>>(s, A, bank);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (p.parts) {
       taps_sum_kernel<STUDENT><<<dim3(cdiv(s.W, 512), s.H, s.R2), 128, 0, st>>>(s, A);
@@ -774,6 +826,16 @@ cudaError_t launch_taps_t(const Shape& s, const DirectPlan& p, const DirectLaunc
     }
   }
   return cudaSuccess;
+}
+
+template <class Taps>
+cudaError_t launch_taps_of(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
+                           const float* hkf, const float* hka, cudaStream_t st) {
+  if (h.a.nu > 0.f)
+    return p.tile == 0 ? launch_taps_t<0, true, Taps>(s, p, h, hkf, hka, st)
+                       : launch_taps_t<1, true, Taps>(s, p, h, hkf, hka, st);
+  return p.tile == 0 ? launch_taps_t<0, false, Taps>(s, p, h, hkf, hka, st)
+                     : launch_taps_t<1, false, Taps>(s, p, h, hkf, hka, st);
 }
 
 template <int V, bool STUDENT>
@@ -818,11 +880,11 @@ int direct_counter_ints(const Shape& s) {
 
 cudaError_t launch_taps_iter(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
                              const float* hkf, const float* hka, cudaStream_t st) {
-  if (h.a.nu > 0.f)
-    return p.tile == 0 ? launch_taps_t<0, true>(s, p, h, hkf, hka, st)
-                       : launch_taps_t<1, true>(s, p, h, hkf, hka, st);
-  return p.tile == 0 ? launch_taps_t<0, false>(s, p, h, hkf, hka, st)
-                     : launch_taps_t<1, false>(s, p, h, hkf, hka, st);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(st, &cap);
+  if (e != cudaSuccess) return e;
+  return cap == cudaStreamCaptureStatusNone ? launch_taps_of<TapBank>(s, p, h, hkf, hka, st)
+                                            : launch_taps_of<TapMemory>(s, p, h, hkf, hka, st);
 }
 
 int numerator_exposures(const Shape& s) {

@@ -38,7 +38,9 @@ struct DirectLaunch {
 };
 int direct_counter_ints(const Shape& s);
 
-// One iteration with the taps form; hkf, hka: host copies of all kernels.
+// One iteration with the taps form; hkf, hka: host copies of all kernels. Under stream
+// capture the launches read h.a.kf and h.a.ka instead, so that a replay after a new
+// frame set uses its PSFs.
 cudaError_t launch_taps_iter(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
                              const float* hkf, const float* hka, cudaStream_t st);
 // iters iterations with the split form, x buffers xa (current) and xb
