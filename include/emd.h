@@ -74,20 +74,25 @@ enum emd_precision {
 /*
  * emd_create -- new context for n exposures of H x W pixels, K x K PSFs
  * (K odd, on the fine grid when r > 1) and super-resolution factor r >= 1
- * (Eq. (3); r = 1 is Eq. (1)). Allocates all device memory the context
- * will use (emd_ctx_bytes reports how much) on the current device.
+ * (Eq. (3); r = 1 is Eq. (1)). Allocates the device memory that every mode
+ * uses (emd_ctx_bytes reports how much) on the current device; a mode's own
+ * buffers come with its first use (emd_ctx_bytes_precision).
  * Returns NULL on error (emd_last_error explains): H, W, n < 1, K even or
  * < 1, r < 1, hc > EMD_MAX_HC, or out of device memory.
  */
 emd_ctx *emd_create(int H, int W, int n, int psf_k, int r);
 
-/* Device bytes a context of this shape holds (0 for invalid shapes). */
+/* Device bytes a context of this shape holds from emd_create on (0 for invalid
+ * shapes). */
 size_t emd_ctx_bytes(int H, int W, int n, int psf_k, int r);
 
 /* The same plus the buffers the mode adds (EMD_PREC_FP32: the w ring of
- * the halo-exchange kernel; the tensor-core operands; the FFT form's
- * spectra, w planes and scratch; nothing for EMD_PREC_FP32_PAIR); 0 for an
- * invalid shape or a mode this shape does not support. Host only. */
+ * the halo-exchange kernel, which batches and streaming passes run; the
+ * tensor-core operands; the FFT form's spectra, w planes and scratch; nothing
+ * for EMD_PREC_FP32_PAIR); 0 for an invalid shape or a mode this shape does not
+ * support. Host only. emd_iterate's launch forms (EMD_PREC_FP32) take work
+ * planes instead of the ring, at most half of emd_ctx_bytes or 64 MB, and run
+ * on the ring where there is no memory for them. */
 size_t emd_ctx_bytes_precision(int H, int W, int n, int psf_k, int r, int mode);
 
 /* Destroy a context and free its device memory. NULL is ignored. */
@@ -167,16 +172,23 @@ int emd_loglik_chi2(emd_ctx *ctx, double *out, double *chi2);
  * r > 1, a per-tile scratch of r^2 spectra (66.5 KB each), allocated on first
  * selection.
  * EMD_PREC_FP32 runs, per chunk of exposures, a forward launch (weighted model
- * images u_t z_t into work planes of the context, which emd_ctx_bytes counts:
- * at most four for large images) and an adjoint launch, whose kernels' taps
- * travel in the launch parameters; images of a few tiles run (tile, exposure)
- * items with grid barriers, many iterations per cooperative launch (about 2 ms
- * of them). PSFs too large for the launch parameters (r^2 kernels above 30 KB)
- * and contexts with a fixed tile shape (emd_set_tile_shape) run one persistent
- * kernel per iteration that passes u_t z_t between tiles through a ring of tile
- * buffers in device memory (about 1030 tiles of 32 KB at 4096^2, fewer for
- * smaller images; emd_ctx_bytes_precision counts them), allocated at the
- * first such iteration; batches and emd_iterate_streaming run it too.
+ * images u_t z_t into work planes, at most four for large images) and an adjoint
+ * launch, whose kernels' taps travel in the launch parameters. Images of a few
+ * tiles, and larger ones (below 500 tiles of 64 x 128, fewer than 4000 over the
+ * exposures) whose PSFs do not fit the launch parameters (r^2 kernels above 30 KB)
+ * or are below 5 x 5, run (tile, exposure) items with grid barriers, many
+ * iterations per cooperative launch (about 2 ms of them). The work planes come
+ * with the first iteration and take at most half of what the context holds, or
+ * 64 MB. Other shapes, contexts with a fixed tile shape
+ * (emd_set_tile_shape) and contexts whose work planes find no memory run one
+ * persistent kernel per iteration that passes u_t z_t between tiles through a
+ * ring of tile buffers in device memory (about 1030 tiles of 32 KB at 4096^2,
+ * fewer for smaller images), allocated at the first such iteration; batches and
+ * emd_iterate_streaming run it too. A captured iteration reads the PSFs from the
+ * context, so that a replay uses those of the frame set then loaded (the FFT and
+ * tensor-core forms' spectra and operands are those of the last uncaptured
+ * iteration), and takes no memory: captured before any other, it runs
+ * EMD_PREC_FP32_PAIR's kernel.
  * EMD_PREC_FP32_PAIR gives the same iterates bit for bit from the kernel that
  * keeps u_t z_t in the shared memory of a CTA pair per tile and recomputes the
  * forward model on a 2 hc halo around it (no extra memory, 1.48x the

@@ -37,7 +37,7 @@ void set_err(const char* fmt, ...) {
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 struct Layout {
-  size_t x0, x1, N, Den, u, y, kf, ka, fraw, part, sums, err, counters, work, total;
+  size_t x0, x1, N, Den, u, y, kf, ka, fraw, part, sums, err, total;
 };
 
 Layout make_layout(const Shape& s) {
@@ -61,12 +61,18 @@ Layout make_layout(const Shape& s) {
   L.part = take(parts * sizeof(double));
   L.sums = take(8 * sizeof(double));
   L.err = take(sizeof(int));
-  // the launch forms of the FP32 direct iteration (emd_taps.cuh)
-  const emd::DirectPlan dp = emd::direct_plan(s, false);
-  L.counters = take(dp.planes ? (size_t)emd::direct_counter_ints(s) * sizeof(int) : 0);
-  L.work = take((size_t)dp.planes * s.g.plane * sizeof(float));
   L.total = off;
   return L;
+}
+
+// bytes of the work planes and counters of the FP32 direct launch forms
+// (emd_taps.cuh), allocated at the first such iteration (0: halo-exchange kernel)
+size_t work_plane_bytes(const Shape& s) {
+  return align256((size_t)emd::direct_plan(s, false).planes * s.g.plane * sizeof(float));
+}
+size_t work_bytes(const Shape& s) {
+  const size_t planes = work_plane_bytes(s);
+  return planes ? planes + (size_t)emd::direct_counter_ints(s) * sizeof(int) : 0;
 }
 
 bool is_device_ptr(const void* p) {
@@ -110,7 +116,8 @@ struct emd_ctx {
   double *part = nullptr, *sums = nullptr;
   int* err = nullptr;
   // launch forms of the FP32 direct iteration: plans per noise model, work
-  // planes and counters in the arena, host copies of the kernels (taps form)
+  // planes and counters (allocated at the first such iteration), host copies of
+  // the kernels (taps form)
   emd::DirectPlan plan[2];
   int* counters = nullptr;
   float* work = nullptr;
@@ -389,8 +396,6 @@ emd_ctx* emd_create(int H, int W, int n, int psf_k, int r) {
   c->part = reinterpret_cast<double*>(c->arena + c->L.part);
   c->sums = reinterpret_cast<double*>(c->arena + c->L.sums);
   c->err = reinterpret_cast<int*>(c->arena + c->L.err);
-  c->counters = reinterpret_cast<int*>(c->arena + c->L.counters);
-  c->work = reinterpret_cast<float*>(c->arena + c->L.work);
   for (int m = 0; m < 2; ++m) c->plan[m] = emd::direct_plan(s, m == 1);
   g_err.clear();
   return c;
@@ -408,6 +413,7 @@ void emd_destroy(emd_ctx* c) {
   if (c->Ns) cudaFree(c->Ns);
   if (c->fft_arena) cudaFree(c->fft_arena);
   if (c->halo_arena) cudaFree(c->halo_arena);
+  if (c->work) cudaFree(c->work);
   delete c;
 }
 
@@ -482,6 +488,32 @@ int ensure_fft_spectra(emd_ctx* c) {
   CK(emd::launch_fft_spectra(c->s, c->ka, const_cast<float2*>(c->fft.spec),
                              const_cast<float2*>(c->fft.spec1), c->st));
   c->fft_ready = true;
+  return EMD_OK;
+}
+
+bool capturing(const emd_ctx* c) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->st, &cap) != cudaSuccess) cudaGetLastError();
+  return cap != cudaStreamCaptureStatusNone;
+}
+
+// The launch forms' work planes (zero outside the image) and counters (zero). *ok =
+// false, no error: they cannot be had now (the stream is capturing) or at all (no
+// memory: the halo-exchange kernel, whose ring is smaller, runs from then on).
+int ensure_work_planes(emd_ctx* c, bool* ok) {
+  *ok = c->work != nullptr;
+  if (*ok || capturing(c)) return EMD_OK;
+  void* p = nullptr;
+  const size_t bytes = work_bytes(c->s);
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    for (emd::DirectPlan& plan : c->plan) plan.form = emd::kFormHalo;
+    return EMD_OK;
+  }
+  CK(cudaMemsetAsync(p, 0, bytes, c->st));
+  c->work = static_cast<float*>(p);
+  c->counters = reinterpret_cast<int*>(static_cast<char*>(p) + work_plane_bytes(c->s));
+  *ok = true;
   return EMD_OK;
 }
 
@@ -894,8 +926,14 @@ int emd_iterate(emd_ctx* c, int k) {
     return EMD_OK;
   }
   // FP32 direct, no tile shape fixed: the launch form of this shape, if any
-  if (c->prec == EMD_PREC_FP32 && c->tile_forced < 0 && c->plan[0].form != emd::kFormHalo)
-    return iterate_direct(c, k);
+  bool pair = c->prec == EMD_PREC_FP32_PAIR;
+  if (!pair && k > 0 && c->tile_forced < 0 && c->plan[0].form != emd::kFormHalo) {
+    bool ok = false;
+    if (int rc = ensure_work_planes(c, &ok)) return rc;
+    if (ok) return iterate_direct(c, k);
+    // captured before any iteration: the kernel that needs no memory (same bits)
+    if (capturing(c)) pair = true;
+  }
   if (c->noise == EMD_NOISE_STUDENT_T) {
     // heavy-tailed EM: the numerator depends on x through the weights u' of
     // the current x. The halo-exchange kernel computes the forward model
@@ -903,7 +941,7 @@ int emd_iterate(emd_ctx* c, int k) {
     // kernel (EMD_PREC_FP32_PAIR) runs N' (mode 3), then Den' and the update
     // (mode 0), each with its own forward pass. Same iterates either way.
     bool halo = false;
-    if (c->prec == EMD_PREC_FP32 && k > 0)
+    if (!pair && k > 0)
       if (int rc = ensure_halo_arena(c, &halo)) return rc;
     for (int it = 0; halo && it < k; ++it) {
       emd::HaloLaunch h = c->halo;
@@ -923,7 +961,7 @@ int emd_iterate(emd_ctx* c, int k) {
     return EMD_OK;
   }
   bool halo = false;
-  if (c->prec == EMD_PREC_FP32 && k > 0)
+  if (!pair && k > 0)
     if (int rc = ensure_halo_arena(c, &halo)) return rc;
   for (int it = 0; it < k; ++it) {
     emd::FusedArgs a = fused_args(c);

@@ -933,37 +933,64 @@ int split_iters_per_launch(const Shape& s) {
   return std::max(1, (int)(2000.0 / us));
 }
 
+namespace {
+
+// Work planes a context may take: half as many as it holds anyway, or 64 MB where
+// that is more (small images, whose planes are small and whose items few).
+long long plane_budget(const Shape& s) {
+  const long long planes = 2LL * s.n + 4LL * s.R2;
+  return std::max(planes / 2, (64LL << 20) / (s.g.plane * (long long)sizeof(float)));
+}
+
+// exposures per chunk of `per` planes each: `want`, or what the budget allows, in
+// chunks of about equal size
+int fit_chunk(const Shape& s, int want, int per) {
+  const long long budget = plane_budget(s);
+  if ((long long)want * per <= budget) return want;
+  const int most = (int)std::max(1LL, budget / per);
+  return cdiv(s.n, cdiv(s.n, most));
+}
+
+}  // namespace
+
 DirectPlan direct_plan(const Shape& s, bool student) {
   DirectPlan p{};
   const long long T = (long long)s.gx * cdiv(s.H, 64);  // 64 x 128 tiles
   const int cap = s.Kc >= 5 ? tap_bank_kernels(s) / s.R2 : 0;  // exposures of one launch
+  // one CTA per tile and phase adds the exposures itself where those fill
+  // the SMs; else their partials take planes (2048^2 15, 8: 967 and 909 us;
+  // 1600 x 1500: 3352 and 3358; 4096^2: 62670 and 66560)
+  const int parts = T * s.R2 < 4 * kSMs;
   // Exposures of a taps launch: 8192 items (18 waves of three CTAs an SM)
   // leave little of a last wave idle; more would only take memory for w.
-  const int taps = (int)std::min<long long>({(long long)cap, (long long)s.n,
-                                             std::max(4LL, 8192 / T)});
+  int taps = (int)std::min<long long>({(long long)cap, (long long)s.n,
+                                       std::max(4LL, 8192 / T)});
+  taps = std::min(taps, fit_chunk(s, taps, 1 + parts * s.R2));
+  // The split form's 32 x 64 tiles, or 32 x 32 tiles with half the outputs per thread
+  // where even those give few warps (300^2 21, 12, 1.1 M outputs an operator: 106 and
+  // 90 us; 512^2 31, 12, 3.2 M: 342 and 389)
+  const int split_tile = (double)s.n * s.R2 * s.H * s.W >= 2e6 ? 0 : 1;
+  const int split = fit_chunk(s, s.n, 1 + s.R2);
+  const long long split_items = (long long)split * cdiv(s.W, split_tile == 0 ? 64 : 32) * cdiv(s.H, 32);
   // Measured (us an iteration, halo / taps / split; K, n): 128^2 15, 4: 166 /
-  // 78 / 22; 300^2 21, 12: 735 / 156 / 90; 512^2 31, 12 (T taps = 280): 1201 /
+  // 78 / 29; 300^2 21, 12: 735 / 156 / 90; 512^2 31, 12 (T taps = 280): 1201 /
   // 450 / 342; 700 x 800 31, 20 (539): 2035 / 1075 / 1101; 1021 x 1009 43, 33
   // (512): 6196 / 5675 / 5660; 1600 x 1500 31, 20: 4171 / 3352 / 4228; 4096^2
   // 43, 33: 80173 / 62670 / 93051. Below 500 items a taps launch leaves SMs
-  // idle and the split form, with every exposure's items in one phase, wins.
+  // idle and the split form, with every exposure's items in one phase, wins; where
+  // its planes are over the budget, while a chunk still has two items an SM.
   if (taps > 0 && T * taps >= 500) {
     p.form = kFormTaps;
     p.chunk = taps;
-    // one CTA per tile and phase adds the exposures itself where those fill
-    // the SMs; else their partials take planes (2048^2 15, 8: 967 and 909 us;
-    // 1600 x 1500: 3352 and 3358; 4096^2: 62670 and 66560)
-    p.parts = T * s.R2 < 4 * kSMs;
+    p.parts = parts;
     // 64 x 64 tiles divide few items more evenly (700 x 800: 1123 and 1075 us;
     // 1600 x 1500, 2100 items: 3352 and 3434)
     p.tile = T * taps >= 1500 ? 0 : 1;
-  } else if (T * s.n < 4000 && T < 500) {
+  } else if (T * s.n < 4000 && T < 500 && (split == s.n || split_items >= 2 * kSMs)) {
     p.form = kFormSplit;
     p.parts = 1;
-    p.chunk = s.n;
-    // 2 x 4 outputs per thread where even those give few warps (300^2 21, 12,
-    // 1.1 M outputs an operator: 106 and 90 us; 512^2 31, 12, 3.2 M: 342 and 389)
-    p.tile = (double)s.n * s.R2 * s.H * s.W >= 2e6 ? 0 : 1;
+    p.chunk = split;
+    p.tile = split_tile;
   } else {
     return p;  // halo_kernel: no work planes
   }

@@ -14,13 +14,13 @@ enum DirectForm {
 };
 
 // How a full FP32 direct iteration of this problem shape runs. Host only and
-// independent of the device, so that emd_ctx_bytes can count the work planes.
+// independent of the device.
 struct DirectPlan {
   int form;
   int tile;      // tile variant of the form
   int chunk;     // exposures per forward launch / phase
   int parts;     // 1: adjoint partials per exposure in work planes, summed in order
-  int planes;    // work planes of the context's arena (the same for both noise models)
+  int planes;    // work planes (the same for both noise models)
 };
 DirectPlan direct_plan(const Shape& s, bool student);
 
