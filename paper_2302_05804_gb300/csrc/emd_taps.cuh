@@ -25,9 +25,11 @@ struct DirectPlan {
 DirectPlan direct_plan(const Shape& s, bool student);
 
 constexpr int kTapFloats = 7600;  // taps of one launch (30,400 bytes of kernel parameters)
-struct TapBank {
+// 16-byte aligned among the parameters, whatever comes before it: it is read as float4
+struct alignas(16) TapBank {
   float k[kTapFloats];
 };
+static_assert(kTapFloats % 4 == 0, "the bank is read by quads");
 // kernels (Kc x KP floats each) that one launch's constant bank holds
 int tap_bank_kernels(const Shape& s);
 
