@@ -336,8 +336,8 @@ __device__ __forceinline__ bool last_to_arrive(int* counter, int ne, int* flag_s
 // chunk fills the SMs several times over, 64 x 64 (64 threads) otherwise, whose
 // items divide the SMs more evenly.
 template <int V> struct TapsTile;
-template <> struct TapsTile<0> { static constexpr int TH = 64, TW = 128, MINB = 3, NUMB = 2; };
-template <> struct TapsTile<1> { static constexpr int TH = 64, TW = 64, MINB = 5, NUMB = 4; };
+template <> struct TapsTile<0> { static constexpr int TH = 64, TW = 128, MINB = 3; };
+template <> struct TapsTile<1> { static constexpr int TH = 64, TW = 64, MINB = 5; };
 
 template <int V, class Taps>
 constexpr int taps_min_blocks() {
@@ -615,9 +615,14 @@ struct NumeratorArgs {
   int gx;                 // tiles per row
 };
 
-template <int V>
-__global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), TapsTile<V>::NUMB)
-    taps_numerator_kernel(const Shape s, const NumeratorArgs A,
+// CTAS per SM: the block sums need 240 registers, or 168 and a few spills, which
+// more CTAs on an SM outweigh (21 x 814 x 895, K = 15: 826 -> 720 us a frame set;
+// 24 x 900^2, K = 29: 1592 -> 1316; 4096^2 x 9, K = 43: 12.60 -> 12.31 ms) except on
+// 64 x 64 tiles whose windows leave shared memory for four only (33 x 1024^2, K = 43:
+// 5 % slower with 168).
+template <int V, int CTAS>
+__global__ void __launch_bounds__(TapsTile<V>::TH / 4 * (TapsTile<V>::TW / 16), CTAS)
+    taps_numerator_kernel(const Shape s, const __grid_constant__ NumeratorArgs A,
                           const __grid_constant__ TapBank bank) {
   constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NY = TH / 4, NT = NY * (TW / 16);
   extern __shared__ __align__(128) float smem[];
@@ -677,11 +682,11 @@ __global__ void __launch_bounds__(128)
   if (j + 1 < s.g.W) A.N[off + 1] = v.y;
 }
 
-template <int V>
+template <int V, int CTAS>
 cudaError_t launch_numerator_t(const Shape& s, NumeratorArgs A, int chunk, const float* hka,
                                cudaStream_t st) {
   constexpr int TH = TapsTile<V>::TH, TW = TapsTile<V>::TW, NT = TH / 4 * (TW / 16);
-  cudaError_t e = allow_max_dynamic_smem((const void*)taps_numerator_kernel<V>);
+  cudaError_t e = allow_max_dynamic_smem((const void*)taps_numerator_kernel<V, CTAS>);
   if (e != cudaSuccess) return e;
   const size_t smem = taps_smem_bytes(s, TH, TW), kfl = (size_t)s.R2 * s.Kc * s.KP;
   A.gx = cdiv(s.W, TW);
@@ -690,7 +695,7 @@ cudaError_t launch_numerator_t(const Shape& s, NumeratorArgs A, int chunk, const
   for (A.c0 = 0; A.c0 < s.n; A.c0 += chunk) {
     A.ne = std::min(chunk, s.n - A.c0);
     std::copy(hka + (size_t)A.c0 * kfl, hka + (size_t)(A.c0 + A.ne) * kfl, bank.k);
-    taps_numerator_kernel<V><<<dim3(T, s.R2, A.parts ? A.ne : 1), NT, smem, st>>>(s, A, bank);
+    taps_numerator_kernel<V, CTAS><<<dim3(T, s.R2, A.parts ? A.ne : 1), NT, smem, st>>>(s, A, bank);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (A.parts && A.ne > 1) {
       numerator_sum_kernel<<<dim3(cdiv(s.W, 256), s.H, s.R2), 128, 0, st>>>(s, A);
@@ -903,8 +908,10 @@ cudaError_t launch_numerator(const Shape& s, const float* u, const float* y, con
   const long long T = (long long)s.gx * cdiv(s.H, 64);
   A.parts = T * s.R2 < 4 * kSMs;
   const int most = numerator_exposures(s), chunk = A.parts ? std::min(most, kNumParts + 1) : most;
-  return T * chunk >= 1500 ? launch_numerator_t<0>(s, A, chunk, hka, st)
-                           : launch_numerator_t<1>(s, A, chunk, hka, st);
+  if (T * chunk >= 1500) return launch_numerator_t<0, 3>(s, A, chunk, hka, st);
+  return 6 * (taps_smem_bytes(s, 64, 64) + 1024) <= 228 * 1024
+             ? launch_numerator_t<1, 6>(s, A, chunk, hka, st)
+             : launch_numerator_t<1, 4>(s, A, chunk, hka, st);
 }
 
 cudaError_t launch_taps_chi2(const Shape& s, const DirectPlan& p, const FusedArgs& a,
