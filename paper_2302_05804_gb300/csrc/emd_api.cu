@@ -468,6 +468,7 @@ int ensure_fft_arena(emd_ctx* c) {
   c->fft.err = c->err;
   c->fft.spec = at(F.spec);
   c->fft.spec1 = student ? at(F.spec1) : nullptr;
+  c->fft.inv_scale = reinterpret_cast<float*>(c->fft_arena + F.scale);
   c->fft.w = at(F.w);
   c->fft.scratch = at(F.scratch);
   c->fft.partials = at(F.partials);
@@ -485,7 +486,8 @@ int ensure_fft_arena(emd_ctx* c) {
 // the PSF spectra, once per frame set
 int ensure_fft_spectra(emd_ctx* c) {
   if (c->fft_ready) return EMD_OK;
-  CK(emd::launch_fft_spectra(c->s, c->ka, const_cast<float2*>(c->fft.spec),
+  CK(emd::launch_fft_spectra(c->s, c->ka, const_cast<float*>(c->fft.inv_scale),
+                             const_cast<float2*>(c->fft.spec),
                              const_cast<float2*>(c->fft.spec1), c->st));
   c->fft_ready = true;
   return EMD_OK;

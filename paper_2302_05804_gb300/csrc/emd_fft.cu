@@ -18,6 +18,11 @@
 //   adjoint  the real part of IFFT(FFT(w_a + i w_b) conj(k^)) is
 //            corr(w_a, k_a) + corr(w_b, k_b), which is all Den needs (the
 //            imaginary part holds cross terms and is dropped).
+// The rounding of one exposure's half is of the size of the other's, so the two
+// kernels are brought to the same size first: k_t stands for s_t k_t, s_t the power
+// of two (exact) that takes the kernel's sum nearest to 1, and the forward pass
+// divides it out again (PSFs may carry the exposures' flux scales). The spectra
+// also carry the 1 / 128^2 of the inverse transforms.
 // Heavy-tailed noise packs the two images of one exposure instead: with the
 // real kernel k_t, IFFT(FFT(w + i w2) conj(k_t^)) = Den_t + i N'_t.
 // x is real, so x^(-m, -f) = conj(x^(m, f)): 64 column slots (m = 1 .. 63, and
@@ -511,12 +516,38 @@ __device__ __forceinline__ void tmem_store(uint32_t addr, const float2 (&v)[16])
 // spectra of the kernels
 // ---------------------------------------------------------------------------
 
+// 1 / s_t of exposure blockIdx.x: the power of two nearest, in logarithm, to the sum
+// of its |taps| (of one of R2 phases on average: 1 for a PSF of unit sum)
+__global__ void __launch_bounds__(256)
+    fft_scale_kernel(const float* __restrict__ ka, int taps, int R2,
+                     float* __restrict__ inv_scale) {
+  __shared__ double red[8];
+  const float* k = ka + (long long)blockIdx.x * R2 * taps;
+  double v = 0.0;
+  for (int e = threadIdx.x; e < R2 * taps; e += blockDim.x) v += fabs((double)k[e]);
+  const double sum = block_sum_f64(v, red);
+  if (threadIdx.x == 0) {
+    const bool ok = sum > 0.0 && isfinite(sum);  // no taps, or none that are numbers
+    const int e = ok ? max(-40, min(40, ilogb(sum / R2 * 1.4142135623730951))) : 0;
+    inv_scale[blockIdx.x] = exp2f((float)e);
+  }
+}
+
+// inv_scale[n]: whether any is not 1 (only then the forward pass loads and multiplies
+// by them, 1 to 2 % of its time)
+__global__ void __launch_bounds__(256) fft_scaled_kernel(int n, float* __restrict__ inv_scale) {
+  bool any = false;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) any |= inv_scale[t] != 1.f;
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) inv_scale[n] = any ? 1.f : 0.f;
+}
+
 // One CTA per (pair, phase): S1 and S2 of k_a + i k_b; single = true: per
 // (exposure, phase) the slots and column 64 of k_t alone. The Kc x Kc phase
 // kernels (row pitch KP; for r = 1 the PSFs) at the top-left of a zero tile.
 __global__ void __launch_bounds__(kFThreads, 1)
-    fft_spectra_kernel(const float* __restrict__ ka, int n, int R2, int Kc, int KP, bool single,
-                       float2* __restrict__ out) {
+    fft_spectra_kernel(const float* __restrict__ ka, const float* __restrict__ inv_scale, int n,
+                       int R2, int Kc, int KP, bool single, float2* __restrict__ out) {
   extern __shared__ __align__(16) float2 fsm[];
   __shared__ float4 tw[kFT / 2];
   init_twiddles(tw);
@@ -525,12 +556,15 @@ __global__ void __launch_bounds__(kFThreads, 1)
   const int ta = single ? q : 2 * q, tb = ta + 1;
   const float* fa = ka + ((long long)ta * R2 + phi) * Kc * KP;
   const float* fb = !single && tb < n ? ka + ((long long)tb * R2 + phi) * Kc * KP : nullptr;
+  // with the inverse transform's 1 / 128^2, exact as well
+  const float sa = single ? kFScale : kFScale / inv_scale[ta];
+  const float sb = fb ? kFScale / inv_scale[tb] : 1.f;
   rows_forward(fsm, tw, L, [&](int r, float2 (&v)[16]) {
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const int c = L.t + 8 * i;
       const bool in = r < Kc && c < Kc;
-      v[i] = make_float2(in ? fa[r * KP + c] : 0.f, in && fb ? fb[r * KP + c] : 0.f);
+      v[i] = make_float2(in ? sa * fa[r * KP + c] : 0.f, in && fb ? sb * fb[r * KP + c] : 0.f);
     }
   });
   const int m = L.slot();
@@ -601,6 +635,7 @@ __device__ void fft_forward_tile(const Shape& s, const FftLaunch& a, int ty, int
   const int m = L.slot(), m2 = second_col(m);
   const int pmax = min(B, g.H - i0), qmax = min(B, g.W - j0);
   float2* st = buf + kFBuf + L.warp * kStage;
+  const bool scaled = __ldg(a.inv_scale + s.n) != 0.f;  // some s_t is not 1
   auto prefetch_pair = [&](int q) {  // u (and y) of the tile
     for (int t = 2 * q; t < min(2 * q + 2, s.n); ++t) {
       const long long off = (long long)t * g.plane + (long long)(g.B + i0) * g.P + g.B + j0;
@@ -740,12 +775,18 @@ __device__ void fft_forward_tile(const Shape& s, const FftLaunch& a, int ty, int
       load_freqs(buf + r * kFP, v, L.t);
       ifft_row(v, buf + r * kFP, tw, L.t);
       if (!row_ok) continue;
+      if (scaled) {  // z = v / s_t; the adjoint's source for the kernel s_t k_t is w / s_t
+        const float ia = __ldg(a.inv_scale + ta), ib = __ldg(a.inv_scale + tb);
+        const float fa = STUDENT ? ia : ia * ia, fb = STUDENT ? ib : ib * ib;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = make_float2(v[i].x * fa, v[i].y * fb);
+      }
       if (!STUDENT) {
         float2* w = a.w + (long long)q * g.plane + rowoff;
 #pragma unroll
         for (int i = 0; i < 16; ++i)
           if (8 * i >= c_lo && 8 * i < c_hi)
-            w[8 * i] = make_float2(u[i].x * (v[i].x * kFScale), u[i].y * (v[i].y * kFScale));
+            w[8 * i] = make_float2(u[i].x * v[i].x, u[i].y * v[i].y);
       } else {
         // heavy-tailed weights u' = u (nu+1) / (nu + u (y - z)^2): (u' z, u' y) per
         // exposure
@@ -759,7 +800,7 @@ __device__ void fft_forward_tile(const Shape& s, const FftLaunch& a, int ty, int
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             if (8 * i >= c_lo && 8 * i < c_hi) {
-              const float z = (e ? v[i].y : v[i].x) * kFScale, uv = e ? u[i].y : u[i].x;
+              const float z = e ? v[i].y : v[i].x, uv = e ? u[i].y : u[i].x;
               const float y = e ? yb[STUDENT ? i : 0] : yv[STUDENT ? i : 0];
               const float d = y - z;
               const float us = uv > 0.f ? uv * nu1 / fmaf(uv * d, d, a.nu) : 0.f;
@@ -834,7 +875,7 @@ __device__ __forceinline__ void rows_update(const Shape& s, const FftLaunch& a, 
 __device__ __forceinline__ void columns_gauss(const float2 (&acc)[16], const float2* a64, float2* buf,
                                               const float4* tw, const Lane& L) {
   const int m = L.slot(), m2 = second_col(m);
-  const float sc = m ? 0.5f * kFScale : kFScale;
+  const float sc = m ? 0.5f : 1.f;
   // column 64 first (slot 0's group, and with it its warp, for the warp
   // barriers), then the slots: one copy of the transform's code
 #pragma unroll 1
@@ -869,8 +910,6 @@ __device__ __forceinline__ void columns_student(float2 (&f)[16], const float2 (&
       for (int i = 0; i < 16; ++i) f[i] = gv[i];
     }
     ifft_col(f, col, tw, L.t);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) f[i] = make_float2(kFScale * f[i].x, kFScale * f[i].y);
     store_col(col, f, L.t, h && m != 0);
   }
   __syncthreads();
@@ -1647,7 +1686,7 @@ int fft_groups(const Shape& s) {
   return best;
 }
 
-// pair spectra, single spectra (Student-t), w planes, scratch, partials, counters
+// pair spectra, single spectra (Student-t), scales, w planes, scratch, partials, counters
 FftLayout fft_layout(const Shape& s, bool student, int split_ctas) {
   FftLayout L{};
   const size_t NP = (s.n + 1) / 2, tiles = fft_tiles_total(s), G = fft_groups(s);
@@ -1656,6 +1695,7 @@ FftLayout fft_layout(const Shape& s, bool student, int split_ctas) {
   auto take = [&](size_t bytes) { const size_t o = off; off += up256(bytes); return o; };
   L.spec = take(NP * s.R2 * kPairSpec * sizeof(float2));
   L.spec1 = take(student ? (size_t)s.n * s.R2 * kCol * sizeof(float2) : 0);
+  L.scale = take((size_t)(s.n + 1) * sizeof(float));
   L.w = take(wplanes * s.g.plane * sizeof(float2));
   const bool r1 = s.R2 == 1;
   L.scratch = take(r1 ? 0 : tiles * G * scratch_floats2(s.R2, student) * sizeof(float2));
@@ -1674,15 +1714,20 @@ size_t fft_smem_bytes() {
   return (size_t)(kFBuf + std::max(kFThreads / 32 * kStage, 64 * kFP)) * sizeof(float2);
 }
 
-cudaError_t launch_fft_spectra(const Shape& s, const float* ka, float2* spec, float2* spec1,
-                               cudaStream_t st) {
+cudaError_t launch_fft_spectra(const Shape& s, const float* ka, float* inv_scale, float2* spec,
+                               float2* spec1, cudaStream_t st) {
   const size_t smem = fft_smem_bytes();
   cudaError_t e = allow_max_dynamic_smem((const void*)fft_spectra_kernel);
   if (e != cudaSuccess) return e;
-  fft_spectra_kernel<<<(s.n + 1) / 2 * s.R2, kFThreads, smem, st>>>(ka, s.n, s.R2, s.Kc, s.KP,
-                                                                    false, spec);
+  fft_scale_kernel<<<s.n, 256, 0, st>>>(ka, s.Kc * s.KP, s.R2, inv_scale);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  fft_scaled_kernel<<<1, 256, 0, st>>>(s.n, inv_scale);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  fft_spectra_kernel<<<(s.n + 1) / 2 * s.R2, kFThreads, smem, st>>>(ka, inv_scale, s.n, s.R2, s.Kc,
+                                                                    s.KP, false, spec);
   if ((e = cudaGetLastError()) != cudaSuccess || !spec1) return e;
-  fft_spectra_kernel<<<s.n * s.R2, kFThreads, smem, st>>>(ka, s.n, s.R2, s.Kc, s.KP, true, spec1);
+  fft_spectra_kernel<<<s.n * s.R2, kFThreads, smem, st>>>(ka, inv_scale, s.n, s.R2, s.Kc, s.KP,
+                                                          true, spec1);
   return cudaGetLastError();
 }
 
