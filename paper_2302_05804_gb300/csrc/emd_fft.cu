@@ -24,7 +24,10 @@
 // divides it out again (PSFs may carry the exposures' flux scales). The spectra
 // also carry the 1 / 128^2 of the inverse transforms.
 // Heavy-tailed noise packs the two images of one exposure instead: with the
-// real kernel k_t, IFFT(FFT(w + i w2) conj(k_t^)) = Den_t + i N'_t.
+// real kernel k_t, IFFT(FFT(w + i w2) conj(k_t^)) = Den_t + i N'_t. There, too, one
+// half's rounding is of the other's size, and far from convergence the data
+// exceed the model by any factor: w2 is brought to w's size by a power of two per
+// tile (student_scale), taken out of N' again.
 // x is real, so x^(-m, -f) = conj(x^(m, f)): 64 column slots (m = 1 .. 63, and
 // columns 0 and 64 in slot 0) stand for the 128 columns. Slot m serves the
 // columns m and 128 - m, the second by conjugation:
@@ -838,10 +841,11 @@ __device__ __forceinline__ float update_pixel(float xo, float d, float nraw, flo
 
 // From the columns in the buffer (every column of every row): inverse row
 // transforms of the rows [0, B) and the update of one phase. STUDENT: real part
-// Den, imaginary part N'. Starts and ends at a CTA barrier.
+// Den, imaginary part N' over inv_scale. Starts and ends at a CTA barrier.
 template <bool STUDENT>
 __device__ __forceinline__ void rows_update(const Shape& s, const FftLaunch& a, int phi, int i0,
-                                            int j0, float2* buf, const float4* tw, const Lane& L) {
+                                            int j0, float2* buf, const float4* tw, const Lane& L,
+                                            float inv_scale = 1.f) {
   const Geom& g = s.g;
   const int B = kFT - 2 * s.hc;
   const int pmax = min(B, g.H - i0), qmax = min(B, g.W - j0);
@@ -864,7 +868,8 @@ __device__ __forceinline__ void rows_update(const Shape& s, const FftLaunch& a, 
 #pragma unroll
     for (int i = 0; i < 16; ++i)
       if (L.t + 8 * i < qmax)
-        a.xn[off + 8 * i] = update_pixel(xo[i], v[i].x, nraw[i], STUDENT ? v[i].y : nraw[i]);
+        a.xn[off + 8 * i] =
+            update_pixel(xo[i], v[i].x, nraw[i], STUDENT ? v[i].y * inv_scale : nraw[i]);
   }
   __syncthreads();
 }
@@ -945,13 +950,55 @@ __device__ __forceinline__ void copies_ready() {
   __syncwarp();
 }
 
+// Heavy-tailed adjoint: the power of two that brings w2 = u' y to the size of
+// w = u' z on the tile's region with origin (r0, c0), from the largest |w| and |w2| of
+// every fourth row of the first exposure that has any (all exposures see one sky).
+// Every group of a tile takes the same one. Called by the whole CTA.
+__device__ float student_scale(const FftLaunch& a, const Geom& g, int n, int r0, int c0) {
+  __shared__ unsigned peak[2];
+  float scale = 1.f;
+  for (int t = 0; t < n; ++t) {
+    __syncthreads();  // the last readers of the peaks are done
+    if (threadIdx.x < 2) peak[threadIdx.x] = 0u;
+    __syncthreads();
+    const float2* w = a.w + (long long)t * g.plane + (long long)g.B * g.P + g.B;
+    float m1 = 0.f, m2 = 0.f;
+#pragma unroll
+    for (int k = 0; k < kFT * kFT / 4 / kFThreads; ++k) {
+      const int e = threadIdx.x + k * kFThreads, i = r0 + 4 * (e / kFT), j = c0 + e % kFT;
+      if (i >= 0 && i < g.H && j >= 0 && j < g.W) {
+        const float2 v = __ldcg(w + (long long)i * g.P + j);
+        m1 = fmaxf(m1, fabsf(v.x));
+        m2 = fmaxf(m2, fabsf(v.y));
+      }
+    }
+    // (values >= 0: ordered as their bits)
+    m1 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m1)));
+    m2 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m2)));
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(&peak[0], __float_as_uint(m1));
+      atomicMax(&peak[1], __float_as_uint(m2));
+    }
+    __syncthreads();
+    const float p1 = __uint_as_float(peak[0]), p2 = __uint_as_float(peak[1]);
+    if (p1 > 0.f && p2 > 0.f) {
+      if (isfinite(p1) && isfinite(p2))
+        scale = exp2f((float)max(-60, min(60, ilogbf(p1) - ilogbf(p2))));
+      break;
+    }
+  }
+  return scale;
+}
+
 // Row transforms of a w region. The warp's rows of the blocks 0 and 1 are
 // in flight to or in its part of the staging buffer (copy_w a column phase
 // ago), or, stage null, in flight to their place in buf; those of the blocks
-// 2 and 3 come straight to their place during the first transforms. Ends at a
-// CTA barrier.
+// 2 and 3 come straight to their place during the first transforms. STUDENT: the
+// second image times scale. Ends at a CTA barrier.
+template <bool STUDENT>
 __device__ __forceinline__ void w_rows(float2* stage, const float2* w, const Geom& g, int r0,
-                                       int c0, float2* buf, const float4* tw, const Lane& L) {
+                                       int c0, float2* buf, const float4* tw, const Lane& L,
+                                       float scale = 1.f) {
   const int blk = L.warp >> 3;
   copies_ready();
   copy_w(buf + (blk + 2) * 32 * kFP, w, g, r0, c0, blk + 2, L);
@@ -962,7 +1009,10 @@ __device__ __forceinline__ void w_rows(float2* stage, const float2* w, const Geo
     if (round) copies_ready();
     float2 v[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = src[L.t + 8 * i];
+    for (int i = 0; i < 16; ++i) {
+      v[i] = src[L.t + 8 * i];
+      if (STUDENT) v[i].y *= scale;
+    }
     fft_row(v, buf + r * kFP, tw, L.t);
     store_freqs(buf + r * kFP, v, L.t);
   }
@@ -1064,6 +1114,7 @@ __device__ void fft_adjoint_tile(const Shape& s, const FftLaunch& a, int ty, int
     }
   }
   const int k0 = STUDENT ? 2 * q0 : q0, k1 = STUDENT ? min(2 * q1, s.n) : q1;
+  const float scale = STUDENT ? student_scale(a, g, s.n, i0 - hc, j0 - hc) : 1.f;
   float2* stage = buf + kFBuf;
   float2* st = stage + L.warp * kStage;  // Student-t: this warp's slice of the spectrum
   if (!STUDENT)
@@ -1089,9 +1140,9 @@ __device__ void fft_adjoint_tile(const Shape& s, const FftLaunch& a, int ty, int
       stage_slot(st, S1);
       if (L.warp == 0)
         for (int e = threadIdx.x; e < kFT; e += 32) a64[e] = __ldg(S1 + kSlots + e);
-      w_rows(nullptr, w, g, i0 - hc, j0 - hc, buf, tw, L);
+      w_rows<true>(nullptr, w, g, i0 - hc, j0 - hc, buf, tw, L, scale);
     } else {
-      w_rows(stage, w, g, i0 - hc, j0 - hc, buf, tw, L);
+      w_rows<false>(stage, w, g, i0 - hc, j0 - hc, buf, tw, L);
       if (k + 1 < k1)
         copy_w(stage + blk * 32 * kFP, w + g.plane, g, i0 - hc, j0 - hc, blk, L);
     }
@@ -1172,7 +1223,7 @@ __device__ void fft_adjoint_tile(const Shape& s, const FftLaunch& a, int ty, int
     }
     columns_gauss(acc, a64, buf, tw, L);
   }
-  rows_update<STUDENT>(s, a, 0, i0, j0, buf, tw, L);
+  rows_update<STUDENT>(s, a, 0, i0, j0, buf, tw, L, 1.f / scale);
 }
 
 // The same for r > 1, with the accumulators in this item's scratch (`mine`).
@@ -1189,13 +1240,14 @@ __device__ void fft_adjoint_tile_scratch(const Shape& s, const FftLaunch& a, int
   const int m = L.slot(), m2 = second_col(m);
   const int per = STUDENT ? 2 * kSlots : kCol;
   const int k0 = STUDENT ? 2 * q0 : q0, k1 = STUDENT ? min(2 * q1, s.n) : q1;
+  const float scale = STUDENT ? student_scale(a, g, s.n, i0 - hc, j0 - hc) : 1.f;
   float2* stage = buf + kFBuf;
   copy_w(stage + (L.warp >> 3) * 32 * kFP, a.w + (long long)k0 * g.plane, g, i0 - hc, j0 - hc,
          L.warp >> 3, L);
   for (int k = k0; k < k1; ++k) {
     const float2* w = a.w + (long long)k * g.plane;
     if (k + 1 < k1) prefetch_region(w + g.plane, 8, g, i0 - hc, j0 - hc);
-    w_rows(stage, w, g, i0 - hc, j0 - hc, buf, tw, L);
+    w_rows<STUDENT>(stage, w, g, i0 - hc, j0 - hc, buf, tw, L, scale);
     if (k + 1 < k1)
       copy_w(stage + (L.warp >> 3) * 32 * kFP, w + g.plane, g, i0 - hc, j0 - hc, L.warp >> 3, L);
     float2 f[16], c[16];  // the transforms of column m and of its partner
@@ -1271,7 +1323,7 @@ __device__ void fft_adjoint_tile_scratch(const Shape& s, const FftLaunch& a, int
       columns_student(f, c, buf, tw, L);
     else
       columns_gauss(f, a64, buf, tw, L);
-    rows_update<STUDENT>(s, a, ph, i0, j0, buf, tw, L);
+    rows_update<STUDENT>(s, a, ph, i0, j0, buf, tw, L, 1.f / scale);
   }
 }
 
@@ -1291,7 +1343,7 @@ __device__ void fft_adjoint_tile_tmem(const Shape& s, const FftLaunch& a, int ty
   for (int q = q0; q < q1; ++q) {
     const float2* w = a.w + (long long)q * g.plane;
     if (q + 1 < q1) prefetch_region(w + g.plane, 8, g, i0 - hc, j0 - hc);
-    w_rows(buf + kFBuf, w, g, i0 - hc, j0 - hc, buf, tw, L);
+    w_rows<false>(buf + kFBuf, w, g, i0 - hc, j0 - hc, buf, tw, L);
     if (q + 1 < q1) copy_w(stage, w + g.plane, g, i0 - hc, j0 - hc, L.warp >> 3, L);
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
