@@ -136,16 +136,28 @@ def direct_form(H, W, n, K, r, nu, tile_shape):
     hc = ((K - 1) // 2 + r - 1) // r
     Kc = 2 * hc + 1
     KP = (Kc + 3) // 4 * 4
-    T = -(-W // 128) * -(-H // 64)
+    # the padded plane (make_shape) and the work planes a context may take
+    gx, gy, Rw = -(-W // 128), -(-H // 128), (128 + 2 * hc + 7) // 8 * 8
+    P = (max((gx - 1) * 128 + (128 + 2 * hc + 15) // 16 * 16 + KP, 2 * hc + W + 1) + 7) // 8 * 8
+    PH = max((gy - 1) * 128 + Rw + 4 * hc + 8, 2 * hc + H + 1, H + 64 + 3 * hc)
+    budget = max((2 * n + 4 * r * r) // 2, (64 << 20) // (4 * P * PH))
+
+    def fit(want, per):
+        return want if want * per <= budget else -(-n // -(-n // max(1, budget // per)))
+
+    T = gx * -(-H // 64)
+    parts = T * r * r < 4 * 152
     cap = 7600 // (Kc * KP) // (r * r) if Kc >= 5 else 0
     taps = min(cap, n, max(4, 8192 // T))
+    taps = min(taps, fit(taps, 1 + (r * r if parts else 0)))
     if not tile_shape and taps > 0 and T * taps >= 500:
-        parts = T * r * r < 4 * 152
         per = 1 + (r * r if parts else 0)
         chunk = min(taps, max(taps, 2) * per // (2 * per)) if nu > 0 else taps
         names = "taps_forward_kernel + taps_adjoint_kernel" + (" + taps_sum_kernel" if parts else "")
         return names, -(-n // chunk) * (3 if parts else 2)
-    if not tile_shape and T * n < 4000 and T < 500:
+    split = fit(n, 1 + r * r)
+    items = split * -(-W // (64 if n * r * r * H * W >= 2e6 else 32)) * -(-H // 32)
+    if not tile_shape and T * n < 4000 and T < (100 if Kc >= 5 else 500) and (split == n or items >= 2 * 152):
         return "split_kernel", 1
     return "halo_kernel", 1
 

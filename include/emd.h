@@ -173,11 +173,11 @@ int emd_loglik_chi2(emd_ctx *ctx, double *out, double *chi2);
  * selection.
  * EMD_PREC_FP32 runs, per chunk of exposures, a forward launch (weighted model
  * images u_t z_t into work planes, at most four for large images) and an adjoint
- * launch, whose kernels' taps travel in the launch parameters. Images of a few
- * tiles, and larger ones (below 500 tiles of 64 x 128, fewer than 4000 over the
- * exposures) whose PSFs do not fit the launch parameters (r^2 kernels above 30 KB)
- * or are below 5 x 5, run (tile, exposure) items with grid barriers, many
- * iterations per cooperative launch (about 2 ms of them). The work planes come
+ * launch, whose kernels' taps travel in the launch parameters (up to 30 KB of
+ * them). Images too small to fill the GPU that way (below 100 tiles of 64 x 128,
+ * or 500 with PSFs below 5 x 5; fewer than 4000 tiles over the exposures) run
+ * (tile, exposure) items with grid barriers, many iterations per cooperative
+ * launch (about 2 ms of them). The work planes come
  * with the first iteration and take at most half of what the context holds, or
  * 64 MB. Other shapes, contexts with a fixed tile shape
  * (emd_set_tile_shape) and contexts whose work planes find no memory run one

@@ -985,7 +985,12 @@ DirectPlan direct_plan(const Shape& s, bool student) {
   // (512): 6196 / 5675 / 5660; 1600 x 1500 31, 20: 4171 / 3352 / 4228; 4096^2
   // 43, 33: 80173 / 62670 / 93051. Below 500 items a taps launch leaves SMs
   // idle and the split form, with every exposure's items in one phase, wins; where
-  // its planes are over the budget, while a chunk still has two items an SM.
+  // its planes are over the budget, while a chunk still has two items an SM. From 100
+  // tiles on it loses to halo_kernel's 32-row tiles (us, split / halo; K, n, r: 900 x
+  // 1000 43, 10: 2332 / 1581; 1100 x 1150 47, 20: 5962 / 4620; 1000^2 47, 31, 8: 40426
+  // / 23371; 900^2 93, 12, 2: 10899 / 8411; 800^2, T = 91, 43, 24: 3378 / 3038; 700^2,
+  // T = 66, 43, 24: 2336 / 2722), except with kernels below 5 x 5, whose windows cost
+  // little (1200^2 3, 12: 263 / 278; 1900^2, T = 450, 3, 4: 246 / 223).
   if (taps > 0 && T * taps >= 500) {
     p.form = kFormTaps;
     p.chunk = taps;
@@ -993,7 +998,7 @@ DirectPlan direct_plan(const Shape& s, bool student) {
     // 64 x 64 tiles divide few items more evenly (700 x 800: 1123 and 1075 us;
     // 1600 x 1500, 2100 items: 3352 and 3434)
     p.tile = T * taps >= 1500 ? 0 : 1;
-  } else if (T * s.n < 4000 && T < 500 && (split == s.n || split_items >= 2 * kSMs)) {
+  } else if (T * s.n < 4000 && T < (s.Kc >= 5 ? 100 : 500) && (split == s.n || split_items >= 2 * kSMs)) {
     p.form = kFormSplit;
     p.parts = 1;
     p.chunk = split;
