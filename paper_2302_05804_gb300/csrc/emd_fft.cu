@@ -1751,10 +1751,11 @@ FftLayout fft_layout(const Shape& s, bool student, int split_ctas) {
   L.w = take(wplanes * s.g.plane * sizeof(float2));
   const bool r1 = s.R2 == 1;
   L.scratch = take(r1 ? 0 : tiles * G * scratch_floats2(s.R2, student) * sizeof(float2));
-  // slots of the split launch (one per CTA) or of the groups
+  // slots of the split launch (one per CTA) and of the groups, which a shape of the
+  // split launch has in a batch where the device has few SMs
   const bool split = r1 && !student && split_ctas > 0 && tiles >= (size_t)split_ctas;
-  L.partials = take((split ? (size_t)split_ctas : r1 && G > 1 ? tiles * G : 0) *
-                    (student ? 2 * kSlots : kCol) * sizeof(float2));
+  const size_t slots = std::max(split ? (size_t)split_ctas : 0, r1 && G > 1 ? tiles * G : 0);
+  L.partials = take(slots * (student ? 2 * kSlots : kCol) * sizeof(float2));
   L.counters = take(split || G > 1 ? tiles * sizeof(int) : 0);
   L.total = off;
   return L;
