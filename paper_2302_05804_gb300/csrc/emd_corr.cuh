@@ -77,19 +77,6 @@ __device__ __forceinline__ float (&corr_target(float (&sum)[RY][RX], float (&)[1
   return sum;
 }
 
-// The loop that bounds every direct-form kernel, on blocks of RY x RX outputs
-// (oy a multiple of RY; Kc odd). Tap quads outside, source rows inside: a
-// quad that a source row brings for output row 0 stays in a register for
-// output row 1 at the next source row. Every output sums its taps in the
-// same order (quads ascending, in a quad rows ascending, in a row columns
-// ascending) whatever block it falls in.
-//
-// RY = 2, 16 warps an SM: 62 TFLOP/s at K = 43 on a 64 x 128 tile (loop
-// alone, 80.5 derived peak). The same loop on 4 x 16 blocks, 8 warps an SM,
-// reaches 52-58 however it is unrolled or prefetched, rows outside and quads
-// inside 55: all execute over 90 % FMAs, and what differs is the dispatch
-// stall (0.3-0.5 per issue), which more warps cover and a larger block, with
-// fewer loads, does not.
 // U source rows (U = 2 or 4) of a block of four output rows, the first at row
 // s: xb[0] holds its window, q[j] the quad of kernel row s - 1 - j; skew: 4 if
 // s mod 4 = 3 (the rows' skew steps at the next row), else 0. The next row's
@@ -113,6 +100,19 @@ __device__ __forceinline__ void corr4_rows(float (&acc)[4][RX], float4 (&q)[3],
   for (int j = 0; j < (U == 2 ? 2 : 3); ++j) q[j] = nw[U - 1 - j];
 }
 
+// The loop that bounds every direct-form kernel, on blocks of RY x RX outputs
+// (oy a multiple of RY; Kc odd). Tap quads outside, source rows inside: a
+// quad that a source row brings for output row 0 stays in a register for
+// output row 1 at the next source row. Every output sums its taps in the
+// same order (quads ascending, in a quad rows ascending, in a row columns
+// ascending) whatever block it falls in.
+//
+// RY = 2, 16 warps an SM: 62 TFLOP/s at K = 43 on a 64 x 128 tile (loop
+// alone, 80.5 derived peak). The same loop on 4 x 16 blocks, 8 warps an SM,
+// reaches 52-58 however it is unrolled or prefetched, rows outside and quads
+// inside 55: all execute over 90 % FMAs, and what differs is the dispatch
+// stall (0.3-0.5 per issue), which more warps cover and a larger block, with
+// fewer loads, does not.
 //
 // BLOCKS (the numerator): the taps of each quad of columns are summed from zero
 // and the blocks then added. One FP32 chain of Kc^2 terms would leave an error

@@ -21,7 +21,8 @@
 // (tile, exposure) items are independent: every exposure's adjoint sum goes
 // to a work plane of its own and the last CTA to finish a tile adds the planes
 // in exposure order. One cooperative launch runs many iterations, two
-// grid barriers each; tiles shrink with the image. Bound by barriers and latency
+// grid barriers each; tiles of 32 x 64, or 32 x 32 for small images. Bound by barriers
+// and latency
 // (128 x 128 x 4, K = 15: 104 -> 29 us an iteration).
 //
 // Both give halo_kernel's iterates bit for bit: every output's taps are
@@ -483,10 +484,6 @@ __global__ void __launch_bounds__(128) taps_sum_kernel(const Shape s, const Taps
 template <int V> struct SplitTile;
 template <> struct SplitTile<0> { static constexpr int TH = 32, TW = 64, RX = 16; };
 template <> struct SplitTile<1> { static constexpr int TH = 32, TW = 32, RX = 8; };
-template <> struct SplitTile<2> { static constexpr int TH = 16, TW = 32, RX = 4; };
-
-constexpr int split_rows(int v) { return v == 2 ? 16 : 32; }
-constexpr int split_cols(int v) { return v == 0 ? 64 : 32; }
 
 struct SplitArgs {
   FusedArgs a;      // x, xn: current and next buffers of the first iteration
@@ -514,11 +511,10 @@ __global__ void __launch_bounds__(SplitTile<V>::TH / 2 * (SplitTile<V>::TW / Spl
   FusedArgs a = A.a;
   int round = 0;
   bool ok = true;
-  auto stage = [&](const float* plane, const float* taps, int i0, int j0, bool window) {
+  auto stage = [&](const float* plane, const float* taps, int i0, int j0) {
     __syncthreads();  // readers of the previous window and taps are done
-    if (window)
-      stage_window<2, NT, 4, true>(sp, plane + (long long)(i0 + s.hc) * g.P, g.P, j0 + s.hc, rows,
-                                   cols);
+    stage_window<2, NT, 4, true>(sp, plane + (long long)(i0 + s.hc) * g.P, g.P, j0 + s.hc, rows,
+                                 cols);
     const float4* kg = reinterpret_cast<const float4*>(taps);
     for (int q = threadIdx.x; q < kf4; q += NT) reinterpret_cast<float4*>(ks)[q] = __ldg(kg + q);
     __syncthreads();
@@ -534,7 +530,7 @@ __global__ void __launch_bounds__(SplitTile<V>::TH / 2 * (SplitTile<V>::TW / Spl
         zero_block(acc);
         for (int phi = 0; phi < s.R2; ++phi) {
           stage(a.x + (long long)phi * g.plane,
-                a.kf + ((long long)t * s.R2 + phi) * s.Kc * s.KP, i0, j0, true);
+                a.kf + ((long long)t * s.R2 + phi) * s.Kc * s.KP, i0, j0);
           corr_tile<2, RX>(acc, sp, 2 * my, RX * mx, ks, s.KP, s.Kc);
         }
         const long long tp = (long long)t * g.plane;
@@ -553,7 +549,7 @@ __global__ void __launch_bounds__(SplitTile<V>::TH / 2 * (SplitTile<V>::TW / Spl
           float acc[2][RX];
           zero_block(acc);
           stage(A.w + (long long)(pass * ne + e) * g.plane,
-                a.ka + ((long long)t * s.R2 + phi) * s.Kc * s.KP, i0, j0, true);
+                a.ka + ((long long)t * s.R2 + phi) * s.Kc * s.KP, i0, j0);
           corr_tile<2, RX>(acc, sp, 2 * my, RX * mx, ks, s.KP, s.Kc);
           store_block(g, acc, i0 + 2 * my, j0 + RX * mx,
                       A.part + (long long)((pass * ne + e) * s.R2 + phi) * g.plane);
@@ -880,7 +876,7 @@ cudaError_t launch_split_t(const Shape& s, const DirectPlan& p, const DirectLaun
 int tap_bank_kernels(const Shape& s) { return kTapFloats / (s.Kc * s.KP); }
 
 int direct_counter_ints(const Shape& s) {
-  return 64 + s.R2 * cdiv(s.W, 32) * cdiv(s.H, 16);
+  return 64 + s.R2 * cdiv(s.W, 32) * cdiv(s.H, 32);  // of the smaller tiles
 }
 
 cudaError_t launch_taps_iter(const Shape& s, const DirectPlan& p, const DirectLaunch& h,
