@@ -268,7 +268,8 @@ int emd_get_tile_shape(emd_ctx *ctx, int *shape, int *decided);
 int emd_selftest_wait_timeout(emd_ctx *ctx, int spins);
 
 /* Inspection: the numerator N ((rH) x (rW)) and the weights u (n x H x W)
- * prepared by emd_set_frames. */
+ * prepared by emd_set_frames. An N of exactly 0 reads +0 where no valid pixel
+ * lies in the footprint and -0 elsewhere. */
 int emd_get_numerator(emd_ctx *ctx, float *out);
 int emd_get_weights(emd_ctx *ctx, float *out);
 
