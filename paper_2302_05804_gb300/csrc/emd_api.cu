@@ -10,6 +10,7 @@
 #include <cmath>
 #include <map>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -752,6 +753,15 @@ int emd_set_frames(emd_ctx* c, const float* y, const float* v, const float* f,
   c->fft_ready = false;
   c->nt_ready = false;
   const size_t npix = (size_t)s.n * s.H * s.W;
+  const size_t nk = (size_t)s.n * s.R2 * s.Kc * s.KP;
+  const bool taps_numerator = emd::numerator_exposures(s) > 0;
+  try {  // host copies of the kernels; no exception leaves a C entry
+    if (c->plan[0].form == emd::kFormTaps) c->hkf.resize(nk);
+    if (taps_numerator) c->hka.resize(nk);
+  } catch (const std::bad_alloc&) {
+    set_err("emd_set_frames: no host memory for a copy of the kernels");
+    return EMD_ENOMEM;
+  }
   // this device's arrays are read by the set-up kernel as they are (33
   // exposures of 1024^2: two copies per exposure and a pass less); others go
   // to the planes first and are converted in place
@@ -779,14 +789,10 @@ int emd_set_frames(emd_ctx* c, const float* y, const float* v, const float* f,
   if (tmp) CK(cudaFreeAsync(tmp, c->st));
   CK(emd::launch_reduce_final(c->part, emd::kRedBlocks, 4, c->sums, c->st));
   CK(emd::launch_build_kernels(s, c->fraw, c->kf, c->ka, c->st));
-  const size_t nk = (size_t)s.n * s.R2 * s.Kc * s.KP;
   if (c->plan[0].form == emd::kFormTaps) {
-    c->hkf.resize(nk);
     CK(cudaMemcpyAsync(c->hkf.data(), c->kf, nk * sizeof(float), cudaMemcpyDeviceToHost, c->st));
   }
-  const bool taps_numerator = emd::numerator_exposures(s) > 0;
   if (taps_numerator) {
-    c->hka.resize(nk);
     CK(cudaMemcpyAsync(c->hka.data(), c->ka, nk * sizeof(float), cudaMemcpyDeviceToHost, c->st));
   }
   double h[4];
