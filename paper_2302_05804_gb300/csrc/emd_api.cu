@@ -665,6 +665,19 @@ int tile_for_launch(emd_ctx* c, bool student, int* trial) {
   return c->trial_cfg[0];  // all trials issued, not yet read
 }
 
+// Tile shape of streaming launches that nothing else decides: 64-row or 48-row tiles
+// (where three CTAs fit an SM), by the rows an SM runs one after the other. Measured
+// (us a pass, 64 / 48 rows; K, n): 600^2 31, 12: 1792 / 1378; 1024^2 31, 8: 1813 / 1920;
+// 2048^2 43, 6: 4599 / 4246; 4096^2 43, 3: 7729 / 7556.
+int streaming_tile(const Shape& s) {
+  const int sms = std::max(1, current_device_sms());
+  auto cost = [&](int rows) {
+    const double waves = (double)s.gx * ((s.H + rows - 1) / rows) / sms;
+    return rows * (waves > 8.0 ? waves : std::ceil(waves));
+  };
+  return cost(48) <= 1.02 * cost(64) && emd::halo_tile_ctas_per_sm(s, 1) >= 3 ? 1 : 0;
+}
+
 // One halo-exchange launch of a full iteration, with the autotuner's shape.
 int halo_launch_full(emd_ctx* c, const emd::HaloLaunch& h, bool student) {
   int trial = -1;
@@ -1075,6 +1088,17 @@ int emd_iterate_streaming(emd_ctx* c, int k, const int* order) {
   bool halo = false;
   if (c->prec != EMD_PREC_FP32_PAIR && k > 0)
     if (int rc = ensure_halo_arena(c, &halo)) return rc;
+  // one-exposure launches: the shape fixed by the caller or decided for the full
+  // iteration, without trials of their own
+  int cfg = c->tile_forced;
+  if (halo && cfg < 0) {
+    {
+      std::lock_guard<std::mutex> lk(g_tile_mu);
+      auto f = g_tile_decided.find(tile_key(c, false));
+      if (f != g_tile_decided.end()) cfg = f->second;
+    }
+    if (cfg < 0) cfg = streaming_tile(s);
+  }
   for (int it = 0; it < k; ++it) {
     for (int q = 0; q < s.n; ++q) {
       const int t = ord[q];
@@ -1083,14 +1107,6 @@ int emd_iterate_streaming(emd_ctx* c, int k, const int* order) {
       a.t0 = t;
       a.t1 = t + 1;
       if (halo) {
-        // one-exposure launches: the shape decided for the full iteration
-        // (or fixed by the caller), without trials of their own
-        int cfg = c->tile_forced;
-        if (cfg < 0) {
-          std::lock_guard<std::mutex> lk(g_tile_mu);
-          auto f = g_tile_decided.find(tile_key(c, false));
-          cfg = f != g_tile_decided.end() ? f->second : 0;
-        }
         emd::HaloLaunch h = c->halo;
         h.a = a;
         CK(emd::launch_halo_iter(s, h, cfg, c->st));
@@ -1675,13 +1691,15 @@ int emd_batch_step(emd_batch* b, int* finished) {
       b->cur = it->second;
     } else {
       // candidates: the FP32 jobs' form (halo-exchange: round-robin or most
-      // expensive job first, 64-row tiles; most expensive first on 48-row
-      // tiles (three CTAs per SM); CTA pairs: all or 3/4 of the resident
-      // pairs)
+      // expensive job first, on 64-row tiles and on 48-row tiles (three CTAs
+      // per SM); CTA pairs: all or 3/4 of the resident pairs)
       const int full = b->max_clusters, part = b->max_clusters - b->max_clusters / 4;
       b->trying.push_back({full, 0, 0, 0});
       b->trying.push_back({full, 1, 0, 0});
-      if (b->halo_ctas[1] > 0) b->trying.push_back({full, 1, 0, 1});
+      if (b->halo_ctas[1] > 0) {
+        b->trying.push_back({full, 0, 0, 1});
+        b->trying.push_back({full, 1, 0, 1});
+      }
       b->trying.push_back({full, 1, 1, 0});
       b->trying.push_back({part, 1, 1, 0});
       b->dirty = true;

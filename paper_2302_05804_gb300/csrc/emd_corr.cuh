@@ -100,6 +100,26 @@ __device__ __forceinline__ void corr4_rows(float (&acc)[4][RX], float4 (&q)[3],
   for (int j = 0; j < (U == 2 ? 2 : 3); ++j) q[j] = nw[U - 1 - j];
 }
 
+// U source rows of a block of three output rows, the first at row s = 2 mod 3 (or a
+// later one of its three, skew 0): q[j] the quad of kernel row s - 1 - j.
+template <int U, int RX>
+__device__ __forceinline__ void corr3_rows(float (&acc)[3][RX], float4 (&q)[2], const float*& row,
+                                           const float*& kq, int pitch, int KP, int skew) {
+  float4 nw[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    float xv[RX + 4];
+    corr_window<RX>(xv, row);
+    nw[u] = *reinterpret_cast<const float4*>(kq);
+    kq += KP;
+    row += u == 0 ? pitch + skew : pitch;
+#pragma unroll
+    for (int p = 0; p < 3; ++p) corr_taps<RX>(acc[p], p <= u ? nw[u - p] : q[p - u - 1], xv);
+  }
+  q[1] = U == 1 ? q[0] : nw[U == 1 ? 0 : U - 2];
+  q[0] = nw[U - 1];
+}
+
 // The loop that bounds every direct-form kernel, on blocks of RY x RX outputs
 // (oy a multiple of RY; Kc odd). Tap quads outside, source rows inside: a
 // quad that a source row brings for output row 0 stays in a register for
@@ -118,7 +138,12 @@ __device__ __forceinline__ void corr4_rows(float (&acc)[4][RX], float4 (&q)[3],
 // and the blocks then added. One FP32 chain of Kc^2 terms would leave an error
 // that no later iteration takes out again, since N is computed once per frame set;
 // blocks of 4 Kc leave about half of it (43 x 43, 2e-7 -> 9e-8).
-template <int RY, int RX, bool BLOCKS = false>
+//
+// CHECKED (halo_kernel's 64-row tiles): the loop with its edges checked inside instead
+// of the unrolled triangles. No quad moves between
+// registers: 5 x 4096^2, K = 43: 12.73 -> 12.41 ms, K = 25, 12 x 2048^2: 3.47 -> 3.27 (one image of
+// few tiles, where a chain of items sets the time, 16 x 900^2, K = 43: 2.98 -> 3.18).
+template <int RY, int RX, bool BLOCKS = false, bool CHECKED = false>
 __device__ __forceinline__ void corr_tile(float (&sum)[RY][RX], const SPlane& src, int oy,
                                           int ox, const float* __restrict__ ks, int KP,
                                           int Kc) {
@@ -160,7 +185,43 @@ __device__ __forceinline__ void corr_tile(float (&sum)[RY][RX], const SPlane& sr
     }
     return;
   }
-  if constexpr (RY == 4) {
+  if constexpr (RY == 3) {
+    // rows 0, 1 and Kc, Kc + 1 as unrolled triangles, three rows at a time between
+    // (edges checked inside the loop: 16 x 900^2, K = 43: 3.22 ms, 2.81 here)
+    if (Kc >= 3) {
+#pragma unroll 1
+      for (int b = 0; b < KP; b += 4) {
+        const float* row = col + b;  // row s at row + s * pitch + 4 * (s / 3)
+        const float* kq = ks + b;
+        float xv[RX + 4];
+        float4 q[2];
+        corr_window<RX>(xv, row);
+        q[1] = *reinterpret_cast<const float4*>(kq);
+        corr_taps<RX>(acc[0], q[1], xv);
+        row += pitch;
+        corr_window<RX>(xv, row);
+        q[0] = *reinterpret_cast<const float4*>(kq + KP);
+        corr_taps<RX>(acc[0], q[0], xv);
+        corr_taps<RX>(acc[1], q[1], xv);
+        row += pitch;
+        kq += 2 * KP;
+        int s = 2;
+#pragma unroll 1
+        for (; s + 3 <= Kc; s += 3) corr3_rows<3, RX>(acc, q, row, kq, pitch, KP, 4);
+#pragma unroll 1
+        for (int skew = 4; s < Kc; ++s, skew = 0)
+          corr3_rows<1, RX>(acc, q, row, kq, pitch, KP, skew);
+        corr_window<RX>(xv, row);
+        corr_taps<RX>(acc[1], q[0], xv);
+        corr_taps<RX>(acc[2], q[1], xv);
+        row += Kc % 3 == 2 ? pitch + 4 : pitch;
+        corr_window<RX>(xv, row);
+        corr_taps<RX>(acc[2], q[0], xv);
+      }
+      return;
+    }
+  }
+  if constexpr (RY == 4 && !CHECKED) {
     // rows 0 .. 2 and Kc .. Kc + 2 as unrolled triangles, no checks between
     if (Kc >= 3) {
 #pragma unroll 1

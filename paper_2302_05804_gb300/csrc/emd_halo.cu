@@ -349,7 +349,7 @@ __device__ __forceinline__ void halo_item(const Shape& s, const HaloLaunch& h, c
       }
     }
     __syncthreads();  // also orders the slot check above before the stores below
-    corr_tile<RY, 16>(acc, sp, RY * my, 16 * mx, ks, s.KP, s.Kc);
+    corr_tile<RY, 16, false, RY == 4>(acc, sp, RY * my, 16 * mx, ks, s.KP, s.Kc);
     if (fwd) continue;
     // ---------------- adjoint epilogue: running sum, or the update ----------------
     float* run = pass == 0 ? a.Den : a.Nw;  // running sum over the exposures
