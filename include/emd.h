@@ -288,9 +288,9 @@ int emd_get_weights(emd_ctx *ctx, float *out);
  * An online autotuner picks, per job mix (a signature of the active jobs'
  * size class, Kc, r, exposure count and mode), the FP32 jobs' kernel form,
  * tile shape and work order and the resident CTA count: the first steps of
- * a new mix each run one candidate (halo-exchange kernel on 64-row and 48-row
- * tiles with jobs interleaved round-robin or most expensive first; CTA pairs,
- * all or 3/4 resident), timed with CUDA events, and the
+ * a new mix each run one candidate (halo-exchange kernel on 64-row tiles with
+ * jobs interleaved round-robin or most expensive first, or on 48-row tiles
+ * interleaved; CTA pairs, all or 3/4 resident), timed with CUDA events, and the
  * fastest is kept. Heavy-tailed noise is not batched.
  * -------------------------------------------------------------------------*/
 typedef struct emd_batch emd_batch;

@@ -1691,15 +1691,13 @@ int emd_batch_step(emd_batch* b, int* finished) {
       b->cur = it->second;
     } else {
       // candidates: the FP32 jobs' form (halo-exchange: round-robin or most
-      // expensive job first, on 64-row tiles and on 48-row tiles (three CTAs
-      // per SM); CTA pairs: all or 3/4 of the resident pairs)
+      // expensive job first, 64-row tiles; round-robin on 48-row tiles (three
+      // CTAs per SM), the fastest on full batches; CTA pairs: all or 3/4 of the
+      // resident pairs). Five: jobs of five iterations still decide.
       const int full = b->max_clusters, part = b->max_clusters - b->max_clusters / 4;
       b->trying.push_back({full, 0, 0, 0});
       b->trying.push_back({full, 1, 0, 0});
-      if (b->halo_ctas[1] > 0) {
-        b->trying.push_back({full, 0, 0, 1});
-        b->trying.push_back({full, 1, 0, 1});
-      }
+      if (b->halo_ctas[1] > 0) b->trying.push_back({full, 0, 0, 1});
       b->trying.push_back({full, 1, 1, 0});
       b->trying.push_back({part, 1, 1, 0});
       b->dirty = true;
