@@ -636,6 +636,7 @@ int tile_for_launch(emd_ctx* c, bool student, int* trial) {
     auto it = g_tile_decided.find(tile_key(c, student));
     if (it != g_tile_decided.end()) return it->second;
   }
+  if (capturing(c)) return 0;  // events of a capture have no times
   if (c->trial_cfg.empty() || c->trial_student != student) {
     const std::vector<int> cand = tile_candidates(c);
     if (cand.size() < 2) {
@@ -952,9 +953,11 @@ int emd_iterate(emd_ctx* c, int k) {
     bool ok = false;
     if (int rc = ensure_work_planes(c, &ok)) return rc;
     if (ok) return iterate_direct(c, k);
-    // captured before any iteration: the kernel that needs no memory (same bits)
-    if (capturing(c)) pair = true;
   }
+  // captured before the memory for it was taken: the kernel that needs none (same bits)
+  const bool student = c->noise == EMD_NOISE_STUDENT_T;
+  if (!pair && k > 0 && c->halo_bytes < emd::halo_buffer_bytes(c->s, student) && capturing(c))
+    pair = true;
   if (c->noise == EMD_NOISE_STUDENT_T) {
     // heavy-tailed EM: the numerator depends on x through the weights u' of
     // the current x. The halo-exchange kernel computes the forward model

@@ -80,10 +80,12 @@ def test_chunks_within_the_bound_give_the_same_bits(H, W, n, K, r, nu):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("H,W,n,K,nu", [(701, 803, 9, 21, 0.0), (128, 131, 4, 15, 3.0)])
+@pytest.mark.parametrize("H,W,n,K,nu", [(701, 803, 9, 21, 0.0), (128, 131, 4, 15, 3.0),
+                                        (900, 1000, 4, 43, 0.0), (900, 1000, 3, 43, 2.0)])
 def test_first_iteration_under_capture(H, W, n, K, nu):
     """No memory is taken then: the CTA-pair kernel runs, with the same bits; the next
-    uncaptured iteration runs the launch form."""
+    uncaptured iteration runs the launch form, or the halo-exchange kernel (the last
+    two shapes)."""
     import torch
     import synth
     p = synth.make_problem("hsc", H=H, W=W, n=n, K=K, r=1, mask_frac=0.03, fwhm=(1.2, 2.5),
